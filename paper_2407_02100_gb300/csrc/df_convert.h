@@ -6,17 +6,18 @@
 // compile the same code (it is checked on the host against exact
 // arithmetic).
 //
-// to_df: hi is x truncated to 24 significant bits, lo the remaining 29 bits
-//   rounded to 24 (|lo| < ulp(hi)), so hi + lo = x to 2^-47 relative.  Exact
+// to_df: hi is x rounded to 24 significant bits (halves away from zero), lo
+//   the remaining signed 29 bits rounded to 24 (|lo| <= ulp(hi) / 2), so
+//   hi + lo = x to 2^-49 relative.  Exact
 //   integer path for 2^-74 <= |x| < 2^115; other magnitudes (zero aside) take
 //   the rounded FP64 path; zero and FP64 subnormals give (0, 0).  The range
 //   of double-float is that of float: below |x| = 2^-100 lo is a float
 //   subnormal and the error becomes absolute (at most 2^-149); from 2^128 on
 //   hi is infinite.
-// from_df: hi + lo rounded to double (to 2^-52 relative; the bits of lo below
-//   the double's last place are truncated) for normal hi and lo with
-//   |lo| <= ulp(hi) and lo far below hi or zero; other cases use the FP64 sum.
+// from_df: hi + lo rounded to double (to 2^-52 relative) for hi normal and at
+//   least 2^-75 and |lo| <= ulp(hi); other cases use the FP64 sum.
 #pragma once
+#include <cmath>
 #include <cstdint>
 #include <cstring>
 
@@ -28,11 +29,16 @@ namespace dfconv {
 // the FP64 fallbacks live in functions of their own, so that the compiler
 // does not predicate their FP64 instructions into the common path
 __device__ __noinline__ void to_df_rounded(double x, float& hi, float& lo) {
+  if (((uint64_t)__double_as_longlong(x) >> 52 & 0x7FF) == 0) {
+    hi = lo = 0.f;
+    return;
+  }
   hi = __double2float_rn(x);
   lo = __double2float_rn(x - (double)hi);
 }
 __device__ __noinline__ double from_df_fp64(float hi, float lo) { return (double)hi + (double)lo; }
-__device__ __forceinline__ float u2f_rn(uint32_t v) { return __uint2float_rn(v); }
+__device__ __forceinline__ float i2f_rn(int32_t v) { return __int2float_rn(v); }
+__device__ __forceinline__ int32_t f2i_rn(float v) { return __float2int_rn(v); }
 __device__ __forceinline__ float fmul_rn(float a, float b) { return __fmul_rn(a, b); }
 __device__ __forceinline__ uint64_t dbits(double x) { return (uint64_t)__double_as_longlong(x); }
 __device__ __forceinline__ double bitsd(uint64_t b) { return __longlong_as_double((long long)b); }
@@ -40,13 +46,18 @@ __device__ __forceinline__ uint32_t fbits(float x) { return __float_as_uint(x); 
 __device__ __forceinline__ float bitsf(uint32_t b) { return __uint_as_float(b); }
 #else
 #define GMG_DFC inline
-inline float u2f_rn(uint32_t v) { return (float)v; }
+inline float i2f_rn(int32_t v) { return (float)v; }
+inline int32_t f2i_rn(float v) { return (int32_t)std::lrint(v); }
 inline float fmul_rn(float a, float b) { return a * b; }
 inline uint64_t dbits(double x) { uint64_t b; std::memcpy(&b, &x, 8); return b; }
 inline double bitsd(uint64_t b) { double x; std::memcpy(&x, &b, 8); return x; }
 inline uint32_t fbits(float x) { uint32_t b; std::memcpy(&b, &x, 4); return b; }
 inline float bitsf(uint32_t b) { float x; std::memcpy(&x, &b, 4); return x; }
 inline void to_df_rounded(double x, float& hi, float& lo) {
+  if ((dbits(x) >> 52 & 0x7FF) == 0) {  // zero or FP64 subnormal (below the float range)
+    hi = lo = 0.f;
+    return;
+  }
   hi = (float)x;
   lo = (float)(x - (double)hi);
 }
@@ -55,47 +66,36 @@ inline double from_df_fp64(float hi, float lo) { return (double)hi + (double)lo;
 
 GMG_DFC void to_df(double x, float& hi, float& lo) {
   const uint64_t b = dbits(x);
-  const int e = (int)((b >> 52) & 0x7FF);  // biased exponent
-  if (e == 0) {                            // zero or FP64 subnormal (below the float range)
-    hi = 0.f;
-    lo = 0.f;
-    return;
-  }
-  if (e < 949 || e > 1137) {  // outside the exact integer path: rounded conversions
+  const uint32_t top = (uint32_t)(b >> 32);
+  const uint32_t e = (top >> 20) & 0x7FFu;  // biased exponent
+  if (e - 949u > 188u) {  // outside the exact integer path: zero, or rounded conversions
     to_df_rounded(x, hi, lo);
     return;
   }
-  const uint32_t sign = (uint32_t)(b >> 32) & 0x80000000u;
-  const uint64_t m = b & 0xFFFFFFFFFFFFFull;  // 52 explicit significand bits
-  hi = bitsf(sign | ((uint32_t)(e - 896) << 23) | (uint32_t)(m >> 29));
-  // x - hi = (low 29 bits) * 2^(e - 1075), with the sign of x; e >= 949 keeps
-  // the scale 2^(e - 1075) a normal float
-  const float r = fmul_rn(u2f_rn((uint32_t)(m & 0x1FFFFFFFu)), bitsf((uint32_t)(e - 948) << 23));
-  lo = sign ? -r : r;
+  const uint32_t sign = top & 0x80000000u;
+  // exponent and significand of |x|, rounded at bit 29 (a carry moves into the
+  // exponent), with the exponent rebased to float's
+  const uint64_t m = (b & 0x7FFFFFFFFFFFFFFFull) + (1ull << 28);
+  hi = bitsf(sign | ((uint32_t)(m >> 29) - (896u << 23)));
+  // x - hi = (low 29 bits, signed) * 2^(e - 1075) with the sign of x; e >= 949
+  // keeps the scale 2^(e - 1075) a normal float
+  lo = fmul_rn(i2f_rn((int32_t)((uint32_t)b << 3) >> 3), bitsf(sign | ((e - 948u) << 23)));
 }
 
 GMG_DFC double from_df(float hi, float lo) {
-  const uint32_t hb = fbits(hi), lb = fbits(lo);
-  const int eh = (int)((hb >> 23) & 0xFF), el = (int)((lb >> 23) & 0xFF);
-  if (eh == 0 || eh == 255 || el == 255 || (el == 0 && (lb & 0x7FFFFFFFu) != 0) || el > eh - 24)
-    return from_df_fp64(hi, lo);  // zero or subnormal hi, inf/nan, subnormal or large lo
-  const uint64_t sgn = (uint64_t)(hb & 0x80000000u) << 32;
-  int64_t S = (int64_t)((hb & 0x7FFFFFu) | 0x800000u) << 29;  // 53 bits, units 2^(eh - 127 - 52)
-  int ex = eh - 127 + 1023;
-  if (el != 0) {
-    const int64_t L = (int64_t)((lb & 0x7FFFFFu) | 0x800000u);  // units 2^(el - 127 - 23)
-    const int d = eh - el - 29;                                  // L in units of S: L * 2^-d, d >= -5
-    const int64_t Ls = d >= 63 ? 0 : d >= 0 ? (L >> d) : (L << -d);
-    S = ((hb ^ lb) & 0x80000000u) ? S - Ls : S + Ls;
-    if (S >= ((int64_t)1 << 53)) {
-      S >>= 1;
-      ++ex;
-    } else if (S < ((int64_t)1 << 52)) {
-      S <<= 1;
-      --ex;
-    }
-  }
-  return bitsd(sgn | ((uint64_t)ex << 52) | ((uint64_t)S & 0xFFFFFFFFFFFFFull));
+  const uint32_t hb = fbits(hi);
+  // lo in units of the double's last place at hi's exponent, 2^(eh - 127 - 52),
+  // negated where hi is negative: an integer of at most 2^29.  306 - eh as an
+  // exponent, with hi's sign: the subtraction borrows the sign bit through.
+  const float t = fmul_rn(lo, bitsf(0x99000000u - (hb & 0xFF800000u)));
+  if ((hb & 0x7FFFFFFFu) - (52u << 23) >= 203u << 23 || !(fabsf(t) <= 536870912.f))
+    return from_df_fp64(hi, lo);  // zero, tiny, inf or nan, or a large lo
+  int32_t L = f2i_rn(t);
+  // below a power of two the last place is half as large
+  if ((hb & 0x7FFFFFu) == 0 && L < 0) L *= 2;
+  // |hi| as a double's bits (sign apart), plus lo: a carry moves into the exponent
+  const uint64_t S = (uint64_t)(hb & 0x7FFFFFFFu) * 0x20000000u + (uint64_t)(int64_t)L;
+  return bitsd(S + ((uint64_t)(896u << 20 | (hb & 0x80000000u)) << 32));
 }
 
 #undef GMG_DFC

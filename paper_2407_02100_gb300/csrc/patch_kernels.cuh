@@ -248,7 +248,8 @@ __device__ __forceinline__ void patch_entry_df(int i, int j, float& hi, float& l
 
 // acc += (or -= with NEG) sum_j E[i][j] x[j] over the band of closure row
 // i+1 of E = M_p (KIND 0) or K_p (KIND 1), double-float (Dot2)
-template <int K, int KIND, bool NEG = false>
+// (FIRST: the accumulator starts with this sum)
+template <int K, int KIND, bool NEG = false, bool FIRST = false>
 __device__ __forceinline__ void patch_row_df(int i, const dfv (&x)[2 * K + 1], df_acc& acc) {
   constexpr int C = 2 * K + 1;
 #pragma unroll
@@ -256,13 +257,14 @@ __device__ __forceinline__ void patch_row_df(int i, const dfv (&x)[2 * K + 1], d
     if (j >= band_lo(i + 1, K) && j <= band_hi(i + 1, K)) {
       float h, l;
       patch_entry_df<K, KIND, NEG>(i, j, h, l);
-      df_acc_add(acc, h, l, x[j]);
+      if (FIRST && j == band_lo(i + 1, K)) acc = df_acc_first(h, l, x[j]);
+      else df_acc_add(acc, h, l, x[j]);
     }
   }
 }
 
 // the same over the interior columns 1..2K-1 (x[a] at closure column a + 1)
-template <int K, int KIND>
+template <int K, int KIND, bool FIRST = false>
 __device__ __forceinline__ void patch_row_int_df(int i, const dfv (&x)[2 * K - 1], df_acc& acc) {
   constexpr int M = 2 * K - 1;
 #pragma unroll
@@ -270,7 +272,8 @@ __device__ __forceinline__ void patch_row_int_df(int i, const dfv (&x)[2 * K - 1
     if (a + 1 >= band_lo(i + 1, K) && a + 1 <= band_hi(i + 1, K)) {
       float h, l;
       patch_entry_df<K, KIND>(i, a + 1, h, l);
-      df_acc_add(acc, h, l, x[a]);
+      if (FIRST && a + 1 == cmax(1, band_lo(i + 1, K))) acc = df_acc_first(h, l, x[a]);
+      else df_acc_add(acc, h, l, x[a]);
     }
   }
 }
@@ -577,19 +580,22 @@ __global__ void __launch_bounds__(NT) patch_colour_kernel(const __grid_constant_
               const dfv u0 = df_from_double(U[0]), uc = df_from_double(U[(C - 1) * C * XU]);
 #pragma unroll
               for (int i = 0; i < M; ++i) {
-                df_acc a = {0.f, 0.f}, b = {0.f, 0.f};
+                df_acc a, b;
                 float h, lo;
                 if (band_lo(i + 1, K) == 0) {
                   patch_entry_df<K, 0>(i, 0, h, lo);
-                  df_acc_add(a, h, lo, u0);
+                  a = df_acc_first(h, lo, u0);
                   patch_entry_df<K, 1>(i, 0, h, lo);
-                  df_acc_add(b, h, lo, u0);
+                  b = df_acc_first(h, lo, u0);
                 }
                 if (band_hi(i + 1, K) == 2 * K) {
+                  const bool both = band_lo(i + 1, K) == 0;  // the centre row
                   patch_entry_df<K, 0>(i, C - 1, h, lo);
-                  df_acc_add(a, h, lo, uc);
+                  if (both) df_acc_add(a, h, lo, uc);
+                  else a = df_acc_first(h, lo, uc);
                   patch_entry_df<K, 1>(i, C - 1, h, lo);
-                  df_acc_add(b, h, lo, uc);
+                  if (both) df_acc_add(b, h, lo, uc);
+                  else b = df_acc_first(h, lo, uc);
                 }
                 B2[l + i * C * C] = stf(df_acc_value(a));
                 B2[C * C * M + l + i * C * C] = stf(df_acc_value(b));
@@ -600,9 +606,9 @@ __global__ void __launch_bounds__(NT) patch_colour_kernel(const __grid_constant_
               for (int j = 0; j < C; ++j) xv[j] = df_from_double(U[j * C * XU]);
 #pragma unroll
               for (int i = 0; i < M; ++i) {
-                df_acc a = {0.f, 0.f}, b = {0.f, 0.f};
-                patch_row_df<K, 0>(i, xv, a);
-                patch_row_df<K, 1>(i, xv, b);
+                df_acc a, b;
+                patch_row_df<K, 0, false, true>(i, xv, a);
+                patch_row_df<K, 1, false, true>(i, xv, b);
                 B2[l + i * C * C] = stf(df_acc_value(a));
                 B2[C * C * M + l + i * C * C] = stf(df_acc_value(b));
               }
@@ -660,9 +666,9 @@ __global__ void __launch_bounds__(NT) patch_colour_kernel(const __grid_constant_
           }
 #pragma unroll
           for (int i = 0; i < M; ++i) {
-            df_acc a = {0.f, 0.f}, b = {0.f, 0.f};
-            patch_row_df<K, 0>(i, p, a);
-            patch_row_df<K, 1>(i, p, b);
+            df_acc a, b;
+            patch_row_df<K, 0, false, true>(i, p, a);
+            patch_row_df<K, 1, false, true>(i, p, b);
             patch_row_df<K, 0>(i, r, b);
             A2[x0 + i * C + z * C * M] = stf(df_acc_value(a));
             A2[C * M * M + x0 + i * C + z * C * M] = stf(df_acc_value(b));
@@ -695,9 +701,9 @@ __global__ void __launch_bounds__(NT) patch_colour_kernel(const __grid_constant_
           for (int j = 0; j < C; ++j) xv[j] = df_from_double(U[j * XU]);
 #pragma unroll
           for (int i = 0; i < M; ++i) {
-            df_acc a = {0.f, 0.f}, b = {0.f, 0.f};
-            patch_row_df<K, 0>(i, xv, a);
-            patch_row_df<K, 1>(i, xv, b);
+            df_acc a, b;
+            patch_row_df<K, 0, false, true>(i, xv, a);
+            patch_row_df<K, 1, false, true>(i, xv, b);
             A2[l + i * C] = stf(df_acc_value(a));
             A2[C * M + l + i * C] = stf(df_acc_value(b));
           }
@@ -738,8 +744,7 @@ __global__ void __launch_bounds__(NT) patch_colour_kernel(const __grid_constant_
           }
 #pragma unroll
           for (int i = 0; i < M; ++i) {
-            const dfv bb = df_mul(df_from_double(Bq[i]), {sbf, 0.f});
-            df_acc acc = {bb.hi, bb.lo};
+            df_acc acc = df_acc_scaled(sbf, df_from_double(Bq[i]));
             patch_row_df<K, 1, true>(i, a1, acc);
             patch_row_df<K, 0, true>(i, a2, acc);
             rd[i] = df_acc_value(acc);

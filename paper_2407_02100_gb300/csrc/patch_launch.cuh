@@ -5,6 +5,7 @@
 #include <vector>
 
 #include "../../include/gmg.h"
+#include "coef_split.h"
 #include "tma_host.h"
 #include "staged_apply.cuh"
 
@@ -298,9 +299,8 @@ static int upload(int k, const double* Mp, const double* Kp, const double* That,
   for (int i = 0; i < M * C; ++i) {
     mhi[i] = (float)Mp[i];
     mlo[i] = (float)(Mp[i] - (double)mhi[i]);
-    khi[i] = (float)Kp[i];
-    klo[i] = (float)(Kp[i] - (double)khi[i]);
   }
+  split_zero_sum_rows(Kp, M, C, khi, klo);
   const size_t po = off_patch(k) * sizeof(float), pb = mhi.size() * sizeof(float);
   e = e == cudaSuccess ? cudaMemcpyToSymbol(c_Mphi, mhi.data(), pb, po) : e;
   e = e == cudaSuccess ? cudaMemcpyToSymbol(c_Mplo, mlo.data(), pb, po) : e;
@@ -311,9 +311,8 @@ static int upload(int k, const double* Mp, const double* Kp, const double* That,
   for (int i = 0; i < nc; ++i) {
     mch[i] = (float)Mc[i];
     mcl[i] = (float)(Mc[i] - (double)mch[i]);
-    kch[i] = (float)Kc[i];
-    kcl[i] = (float)(Kc[i] - (double)kch[i]);
   }
+  split_zero_sum_rows(Kc, k + 1, k + 1, kch, kcl);
   const size_t co = off_cell(k) * sizeof(float), cb = nc * sizeof(float);
   e = e == cudaSuccess ? cudaMemcpyToSymbol(c_Mchi, mch.data(), cb, co) : e;
   e = e == cudaSuccess ? cudaMemcpyToSymbol(c_Mclo, mcl.data(), cb, co) : e;

@@ -50,8 +50,8 @@ constexpr int wide_threads() {
 // acc += sum over the band of closure row i + 1 of E (M_p or K_p, pairs in
 // shared memory, rows of C) of E[i][j] x[j * s]: rows left of the patch
 // centre couple to closure columns 0..k, rows right of it to k..2k, the
-// centre row to all 2k + 1
-template <int K>
+// centre row to all 2k + 1 (FIRST: the accumulator starts with this sum)
+template <int K, bool FIRST>
 __device__ __forceinline__ void wide_row(df_acc& acc, int i, const float2* E, const float2* x, int s) {
   constexpr int C = 2 * K + 1;
   const int j0 = i + 1 > K ? K : 0;
@@ -60,7 +60,8 @@ __device__ __forceinline__ void wide_row(df_acc& acc, int i, const float2* E, co
   for (int q = 0; q <= K; ++q) {
     const int j = j0 + q;
     const float2 v = x[j * s], c = e[j];
-    df_acc_add(acc, c.x, c.y, {v.x, v.y});
+    if (FIRST && q == 0) acc = df_acc_first(c.x, c.y, {v.x, v.y});
+    else df_acc_add(acc, c.x, c.y, {v.x, v.y});
   }
   if (i + 1 == K) {  // the centre row also reaches the right cell
 #pragma unroll
@@ -77,11 +78,12 @@ __device__ __forceinline__ void wide_row(df_acc& acc, int i, const float2* E, co
 template <int K, bool FORWARD>
 __device__ __forceinline__ dfv wide_fd(int i, const float2* T, const float2* x, int s) {
   constexpr int M = 2 * K - 1;
-  df_acc acc = {0.f, 0.f};
+  df_acc acc;
 #pragma unroll
   for (int j = 0; j < M; ++j) {
     const float2 v = x[j * s], c = T[FORWARD ? j * M + i : i * M + j];
-    df_acc_add(acc, c.x, c.y, {v.x, v.y});
+    if (j == 0) acc = df_acc_first(c.x, c.y, {v.x, v.y});
+    else df_acc_add(acc, c.x, c.y, {v.x, v.y});
   }
   return df_acc_value(acc);
 }
@@ -121,9 +123,9 @@ __global__ void __launch_bounds__(NT) patch_wide_df_kernel(const PatchLaunch pl,
     // ---- stage z: P = Mp_z u, Q = Kp_z u;  Y = P, Q [z][y][x], z interior ----
     for (int t = threadIdx.x; t < C * C * M; t += NT) {
       const int l = t % (C * C), i = t / (C * C);
-      df_acc p = {0.f, 0.f}, q = {0.f, 0.f};
-      wide_row<K>(p, i, Mp, X + l, C * C);
-      wide_row<K>(q, i, Kp, X + l, C * C);
+      df_acc p, q;
+      wide_row<K, true>(p, i, Mp, X + l, C * C);
+      wide_row<K, true>(q, i, Kp, X + l, C * C);
       Y[l + i * C * C] = st(df_acc_value(p));
       Y[C * C * M + l + i * C * C] = st(df_acc_value(q));
     }
@@ -132,10 +134,10 @@ __global__ void __launch_bounds__(NT) patch_wide_df_kernel(const PatchLaunch pl,
     for (int t = threadIdx.x; t < C * M * M; t += NT) {
       const int x = t % C, z = (t / C) % M, i = t / (C * M);
       const int src = x + z * C * C;
-      df_acc a1 = {0.f, 0.f}, a2 = {0.f, 0.f};
-      wide_row<K>(a1, i, Mp, Y + src, C);
-      wide_row<K>(a2, i, Kp, Y + src, C);
-      wide_row<K>(a2, i, Mp, Y + C * C * M + src, C);
+      df_acc a1, a2;
+      wide_row<K, true>(a1, i, Mp, Y + src, C);
+      wide_row<K, true>(a2, i, Kp, Y + src, C);
+      wide_row<K, false>(a2, i, Mp, Y + C * C * M + src, C);
       X[x + i * C + z * C * M] = st(df_acc_value(a1));
       X[C * M * M + x + i * C + z * C * M] = st(df_acc_value(a2));
     }
@@ -144,9 +146,9 @@ __global__ void __launch_bounds__(NT) patch_wide_df_kernel(const PatchLaunch pl,
     // ---- stage y: P = Mp_y u, Q = Kp_y u;  Y = P, Q [y][x], y interior ----
     for (int t = threadIdx.x; t < C * M; t += NT) {
       const int l = t % C, i = t / C;
-      df_acc p = {0.f, 0.f}, q = {0.f, 0.f};
-      wide_row<K>(p, i, Mp, X + l, C);
-      wide_row<K>(q, i, Kp, X + l, C);
+      df_acc p, q;
+      wide_row<K, true>(p, i, Mp, X + l, C);
+      wide_row<K, true>(q, i, Kp, X + l, C);
       Y[l + i * C] = st(df_acc_value(p));
       Y[C * M + l + i * C] = st(df_acc_value(q));
     }
@@ -163,9 +165,9 @@ __global__ void __launch_bounds__(NT) patch_wide_df_kernel(const PatchLaunch pl,
       const int i = t % M, l = t / M;  // x, and the line (y, z)
       const long long row = origin + 1 + py * ((DIM == 3 ? l % M : l) + 1) + (DIM == 3 ? pz * (l / M + 1) : 0);
       const dfv bb = df_mul(df_from_double(b[row + i]), {sbf, 0.f});
-      df_acc acc = {0.f, 0.f};
-      wide_row<K>(acc, i, Kp, S1 + C * l, 1);
-      wide_row<K>(acc, i, Mp, S1 + PLANE + C * l, 1);
+      df_acc acc;
+      wide_row<K, true>(acc, i, Kp, S1 + C * l, 1);
+      wide_row<K, false>(acc, i, Mp, S1 + PLANE + C * l, 1);
       R[t] = st(df_add(bb, df_neg(df_acc_value(acc))));
     }
   }

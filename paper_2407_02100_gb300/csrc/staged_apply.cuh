@@ -162,39 +162,45 @@ __global__ void __launch_bounds__(128) axis_pass_df_kernel(const void* __restric
       b[w] = {vb.x, vb.y};
     }
   }
-  // acc += global row p of the cell matrix `kind` applied to the window v
-  auto row = [&](int p, int kind, const dfv (&v)[W], df_acc& acc) {
+  // acc += (first: =) global row p of the cell matrix `kind` applied to the window v
+  auto row = [&](int p, int kind, const dfv (&v)[W], df_acc& acc, bool first) {
     auto eh = [&](int r, int q) { return kind == 0 ? c_Mchi[off_cell(K) + r * (K + 1) + q] : c_Kchi[off_cell(K) + r * (K + 1) + q]; };
     auto el = [&](int r, int q) { return kind == 0 ? c_Mclo[off_cell(K) + r * (K + 1) + q] : c_Kclo[off_cell(K) + r * (K + 1) + q]; };
     if (p == 0) {
 #pragma unroll
-      for (int q = 0; q <= K; ++q) df_acc_add(acc, eh(K, q), el(K, q), v[q]);
+      for (int q = 0; q <= K; ++q) {
+        if (first && q == 0) acc = df_acc_first(eh(K, q), el(K, q), v[q]);
+        else df_acc_add(acc, eh(K, q), el(K, q), v[q]);
+      }
     }
 #pragma unroll
-    for (int q = 0; q <= K; ++q) df_acc_add(acc, eh(p, q), el(p, q), v[K + q]);
+    for (int q = 0; q <= K; ++q) {
+      if (first && p > 0 && q == 0) acc = df_acc_first(eh(p, q), el(p, q), v[K + q]);
+      else df_acc_add(acc, eh(p, q), el(p, q), v[K + q]);
+    }
   };
 #pragma unroll
   for (int p = 0; p < K; ++p) {
     const int node = c * K + p;
     if (node < 1 || node > N - 2) continue;
     const long long o = base + stride * (K + p);
-    df_acc r0 = {0.f, 0.f}, r1 = {0.f, 0.f};
+    df_acc r0, r1;
     if constexpr (AX == 2) {
-      row(p, 0, a, r0);
-      row(p, 1, a, r1);
+      row(p, 0, a, r0, true);
+      row(p, 1, a, r1, true);
       const dfv v0 = df_acc_value(r0), v1 = df_acc_value(r1);
       out0[o] = make_float2(v0.hi, v0.lo);
       out1[o] = make_float2(v1.hi, v1.lo);
     } else if constexpr (AX == 1) {
-      row(p, 0, a, r0);
-      row(p, 1, a, r1);
-      row(p, 0, b, r1);
+      row(p, 0, a, r0, true);
+      row(p, 1, a, r1, true);
+      row(p, 0, b, r1, false);
       const dfv v0 = df_acc_value(r0), v1 = df_acc_value(r1);
       out0[o] = make_float2(v0.hi, v0.lo);
       out1[o] = make_float2(v1.hi, v1.lo);
     } else {
-      row(p, 1, a, r0);
-      row(p, 0, b, r0);
+      row(p, 1, a, r0, true);
+      row(p, 0, b, r0, false);
       double v = alpha * df_to_double(df_acc_value(r0));
       if (bvec) v = fma(beta, bvec[o], v);
       yout[o] = v;

@@ -103,16 +103,16 @@ __global__ void __launch_bounds__(256) transfer_df_kernel(const TI* __restrict__
     }
     // coarse node c = K j + r sits at output index c - 1 + out_off = c along AX
     if (j > 0) {
-      df_acc acc = {0.f, 0.f};
+      df_acc acc = df_acc_first(a.c[0].x, a.c[0].y, x[0]);
 #pragma unroll
-      for (int w = 0; w < W; ++w) df_acc_add(acc, a.c[w].x, a.c[w].y, x[w]);
+      for (int w = 1; w < W; ++w) df_acc_add(acc, a.c[w].x, a.c[w].y, x[w]);
       store_df<TO, ACC>(out + obase + (long long)(K * j) * so, df_acc_value(acc));
     }
 #pragma unroll
     for (int r = 1; r < K; ++r) {
-      df_acc acc = {0.f, 0.f};
+      df_acc acc = df_acc_first(a.c[r * W + 2 * K].x, a.c[r * W + 2 * K].y, x[2 * K]);
 #pragma unroll
-      for (int w = 2 * K; w < W; ++w) df_acc_add(acc, a.c[r * W + w].x, a.c[r * W + w].y, x[w]);
+      for (int w = 2 * K + 1; w < W; ++w) df_acc_add(acc, a.c[r * W + w].x, a.c[r * W + w].y, x[w]);
       store_df<TO, ACC>(out + obase + (long long)(K * j + r) * so, df_acc_value(acc));
     }
   } else {
@@ -126,9 +126,9 @@ __global__ void __launch_bounds__(256) transfer_df_kernel(const TI* __restrict__
 #pragma unroll
     for (int r = 0; r < 2 * K; ++r) {
       if (r < nr) {
-        df_acc acc = {0.f, 0.f};
+        df_acc acc = df_acc_first(a.c[r * W].x, a.c[r * W].y, x[0]);
 #pragma unroll
-        for (int q = 0; q < W; ++q) df_acc_add(acc, a.c[r * W + q].x, a.c[r * W + q].y, x[q]);
+        for (int q = 1; q < W; ++q) df_acc_add(acc, a.c[r * W + q].x, a.c[r * W + q].y, x[q]);
         store_df<TO, ACC>(out + obase + (long long)(2 * K * j + r) * so, df_acc_value(acc));
       }
     }

@@ -112,12 +112,14 @@ __device__ __forceinline__ void cell_operator(T* X, T* P, T* Q, T* A1, T* A2, T*
 
 // The same cell operator in double-float arithmetic (FP64 problems): X, P,
 // Q, A1, A2, OUT hold float pairs; the unit-cell matrices as float pairs.
-template <int K, int KIND>
+template <int K, int KIND, bool FIRST = false>
 __device__ __forceinline__ void cell1d_df(int i, const dfv (&x)[K + 1], df_acc& acc) {
 #pragma unroll
   for (int j = 0; j <= K; ++j) {
     const int o = off_cell(K) + i * (K + 1) + j;
-    df_acc_add(acc, KIND == 0 ? c_Mchi[o] : c_Kchi[o], KIND == 0 ? c_Mclo[o] : c_Kclo[o], x[j]);
+    const float h = KIND == 0 ? c_Mchi[o] : c_Kchi[o], l = KIND == 0 ? c_Mclo[o] : c_Kclo[o];
+    if (FIRST && j == 0) acc = df_acc_first(h, l, x[j]);
+    else df_acc_add(acc, h, l, x[j]);
   }
 }
 
@@ -138,9 +140,9 @@ __device__ __forceinline__ void cell_operator_df(float2* X, float2* P, float2* Q
       for (int j = 0; j < E; ++j) v[j] = ld(X[c * S + l + j * E * E]);
 #pragma unroll
       for (int i = 0; i < E; ++i) {
-        df_acc a = {0.f, 0.f}, b = {0.f, 0.f};
-        cell1d_df<K, 0>(i, v, a);
-        cell1d_df<K, 1>(i, v, b);
+        df_acc a, b;
+        cell1d_df<K, 0, true>(i, v, a);
+        cell1d_df<K, 1, true>(i, v, b);
         P[c * S + l + i * E * E] = st(a);
         Q[c * S + l + i * E * E] = st(b);
       }
@@ -157,9 +159,9 @@ __device__ __forceinline__ void cell_operator_df(float2* X, float2* P, float2* Q
       }
 #pragma unroll
       for (int i = 0; i < E; ++i) {
-        df_acc a = {0.f, 0.f}, b = {0.f, 0.f};
-        cell1d_df<K, 0>(i, p, a);
-        cell1d_df<K, 1>(i, p, b);
+        df_acc a, b;
+        cell1d_df<K, 0, true>(i, p, a);
+        cell1d_df<K, 1, true>(i, p, b);
         cell1d_df<K, 0>(i, q, b);
         A1[c * S + x0 + i * E + z * E * E] = st(a);
         A2[c * S + x0 + i * E + z * E * E] = st(b);
@@ -176,8 +178,8 @@ __device__ __forceinline__ void cell_operator_df(float2* X, float2* P, float2* Q
       }
 #pragma unroll
       for (int i = 0; i < E; ++i) {
-        df_acc a = {0.f, 0.f};
-        cell1d_df<K, 1>(i, a1, a);
+        df_acc a;
+        cell1d_df<K, 1, true>(i, a1, a);
         cell1d_df<K, 0>(i, a2, a);
         OUT[c * S + l * E + i] = st(a);
       }
@@ -191,9 +193,9 @@ __device__ __forceinline__ void cell_operator_df(float2* X, float2* P, float2* Q
       for (int j = 0; j < E; ++j) v[j] = ld(X[c * S + l + j * E]);
 #pragma unroll
       for (int i = 0; i < E; ++i) {
-        df_acc a = {0.f, 0.f}, b = {0.f, 0.f};
-        cell1d_df<K, 0>(i, v, a);
-        cell1d_df<K, 1>(i, v, b);
+        df_acc a, b;
+        cell1d_df<K, 0, true>(i, v, a);
+        cell1d_df<K, 1, true>(i, v, b);
         P[c * S + l + i * E] = st(a);
         Q[c * S + l + i * E] = st(b);
       }
@@ -209,8 +211,8 @@ __device__ __forceinline__ void cell_operator_df(float2* X, float2* P, float2* Q
       }
 #pragma unroll
       for (int i = 0; i < E; ++i) {
-        df_acc a = {0.f, 0.f};
-        cell1d_df<K, 1>(i, p, a);
+        df_acc a;
+        cell1d_df<K, 1, true>(i, p, a);
         cell1d_df<K, 0>(i, q, a);
         OUT[c * S + l * E + i] = st(a);
       }

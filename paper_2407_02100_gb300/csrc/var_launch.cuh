@@ -5,6 +5,7 @@
 #include <vector>
 
 #include "../../include/gmg.h"
+#include "coef_split.h"
 #include "tma_host.h"
 
 namespace gmg {
@@ -116,7 +117,7 @@ int upload_var_tables<GMG_T>(int k, const double* Mc, const double* Kc, const do
     split(Mc, nc, h, l);
     if (e == cudaSuccess) e = cudaMemcpyToSymbol(c_Mchi, h.data(), cb, co);
     if (e == cudaSuccess) e = cudaMemcpyToSymbol(c_Mclo, l.data(), cb, co);
-    split(Kc, nc, h, l);
+    split_zero_sum_rows(Kc, k + 1, k + 1, h, l);
     if (e == cudaSuccess) e = cudaMemcpyToSymbol(c_Kchi, h.data(), cb, co);
     if (e == cudaSuccess) e = cudaMemcpyToSymbol(c_Kclo, l.data(), cb, co);
     split(That, M * M, h, l);
