@@ -710,6 +710,7 @@ int gmg::detail::create_problem(const gmg_desc* d, gmg_problem* p, const CreateO
   if (!generalized_eigen_mirror(m, Mi, Ki, Tp, lp)) return GMG_ERR_INVALID_ARG;
   CHECK(upload_patch_tables<double>(k, Mp.data(), Kp.data(), Tp.data(), Mc.data(), Kc.data(), p->stream));
   CHECK(upload_patch_tables<float>(k, Mp.data(), Kp.data(), Tp.data(), Mc.data(), Kc.data(), p->stream));
+  if (p->esize == 8 && dim == 3) CHECK(upload_pair_sweep_tables(k, Mp.data(), Kp.data(), Tp.data()));
   if (d->precision == GMG_FP32_TC || d->precision == GMG_FP32_TF32)
     CHECK(upload_tc_tables(k, Mp.data(), Kp.data(), Tp.data()));
   const int nint = dim == 3 ? m * m * m : m * m;

@@ -60,6 +60,14 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* mbar, uint32_t parity, uint3
   return false;
 }
 
+// asynchronous copy of 8 bytes from global into shared memory, and the wait
+// for all of this thread's copies
+__device__ __forceinline__ void copy8(void* dst, const void* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(smem_u32(dst)), "l"(__cvta_generic_to_global(src))
+               : "memory");
+}
+__device__ __forceinline__ void copy_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
+
 // order this thread's generic-proxy shared-memory accesses with later
 // async-proxy ones (TMA writes, tensor-core reads)
 __device__ __forceinline__ void fence_proxy_async() {

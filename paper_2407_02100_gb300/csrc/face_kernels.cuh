@@ -1,7 +1,7 @@
 // Shared-face form of the 3D patch sweep (combined colourised smoother,
-// Algorithm 4, constant coefficient, degrees 3..8).  Included by patch_f64.cu
-// and patch_f32.cu after patch_kernels.cuh and patch_launch.cuh (T = double
-// or float).
+// Algorithm 4, constant coefficient, degrees 3..8) for FP32 problems; FP64
+// ones run it in pair_sweep_f64.cu.  Included by patch_f32.cu after
+// patch_kernels.cuh and patch_launch.cuh.
 //
 // The local solver is exact, so the updated interior of patch j is
 // A_j^{-1} (b_j - bar A_j bar u_j^0), bar u_j^0 its closure with the interior
@@ -27,28 +27,12 @@
 // valid while its patches are updated.
 #pragma once
 #include "async.cuh"
+#include "face_geom.cuh"
 
 namespace gmg {
 namespace GMG_NS {
 
-// Faces of one colour.  Patch (i_x, i_y, i_z) of the colour owns
-//   x faces fx = i_x, i_x + 1 of X[(i_z c_y + i_y)(c_x + 1) + fx],
-//   y faces fy = i_y, i_y + 1 of Y[(i_z (c_y + 1) + fy) c_x + i_x],
-//   z faces fz = i_z, i_z + 1 of Z[(fz c_y + i_y) c_x + i_x].
-// Each face holds two M x M fields: x faces F1, F2 as [l][j] (l the z row,
-// j the y row), y faces G1, G2 as [l][i], z faces H1, H2 as [j][i]
-// (i the x row), padded to a multiple of 16 bytes (face_fields elements);
-// the families start at foff[0..2] elements.
-struct FaceGeom {
-  long long py, pz;
-  int first[3], count[3];
-  long long nf[3];
-  long long foff[3];
-};
-
-__host__ __device__ constexpr int face_fields(int k) {
-  return (2 * (2 * k - 1) * (2 * k - 1) + 16 / (int)sizeof(T) - 1) / (16 / (int)sizeof(T)) * (16 / (int)sizeof(T));
-}
+__host__ __device__ constexpr int face_elems(int k) { return face_fields(k, (int)sizeof(T)); }
 
 // acc + sum over the interior columns of row i of M_p (KIND 0) or K_p
 // (KIND 1), x[a] the value at interior column a (closure column a + 1)
@@ -63,37 +47,6 @@ __device__ __forceinline__ T patch_row_int(int i, const T (&x)[2 * K - 1], T acc
     }
   }
   return acc;
-}
-
-// element offset of the first node of face f of family fam (0 x, 1 y, 2 z):
-// the face planes of patch (i_x, i_y, i_z) sit at its closure origin (index
-// i) and at the next patch's (index i + 1); in-plane the data start at the
-// closure origin (axes the face spans completely) or one node inside it
-// (interior rows)
-template <int K>
-__device__ __forceinline__ long long face_origin(const FaceGeom& fg, int fam, long long f) {
-  const int cx = fg.count[0], cy = fg.count[1];
-  long long ix, iy, iz;
-  if (fam == 0) {
-    ix = f % (cx + 1);
-    const long long r = f / (cx + 1);
-    iy = r % cy;
-    iz = r / cy;
-  } else if (fam == 1) {
-    ix = f % cx;
-    const long long r = f / cx;
-    iy = r % (cy + 1);
-    iz = r / (cy + 1);
-  } else {
-    ix = f % cx;
-    const long long r = f / cx;
-    iy = r % cy;
-    iz = r / cy;
-  }
-  const long long X = (fg.first[0] + 2 * ix - 1) * K + (fam == 0 ? 0 : 1);
-  const long long Y = (fg.first[1] + 2 * iy - 1) * K + (fam == 2 ? 1 : 0);
-  const long long Z = (fg.first[2] + 2 * iz - 1) * K;
-  return X + fg.py * Y + fg.pz * Z;
 }
 
 // faces per CTA of the face kernel: enough first-stage lines for NT threads
@@ -114,7 +67,7 @@ template <int K, int NT>
 __global__ void __launch_bounds__(NT) face_kernel(const T* __restrict__ u, T* __restrict__ faces,
                                                   const __grid_constant__ FaceGeom fg, int bx, int by) {
   using F = FaceCfg<K, NT>;
-  constexpr int C = F::C, M = F::M, FS = face_fields(K);
+  constexpr int C = F::C, M = F::M, FS = face_elems(K);
   extern __shared__ __align__(128) unsigned char smem_raw[];
   T* const S = reinterpret_cast<T*>(smem_raw);
   int fam, blk;
@@ -226,139 +179,6 @@ __global__ void __launch_bounds__(NT) face_kernel(const T* __restrict__ u, T* __
   }
 }
 
-// The face kernel of FP64 problems in double-float arithmetic: the node
-// values are read as doubles and split into float pairs, both stages
-// accumulate in Dot2 form with the float-pair patch matrices, and the face
-// fields are stored as float pairs (the same 8 bytes per entry as a double).
-template <int K, int NT>
-__global__ void __launch_bounds__(NT) face_kernel_df(const double* __restrict__ u, float2* __restrict__ faces,
-                                                     const __grid_constant__ FaceGeom fg, int bx, int by) {
-  using F = FaceCfg<K, NT>;
-  constexpr int C = F::C, M = F::M, FS = face_fields(K);
-  extern __shared__ __align__(128) unsigned char smem_raw[];
-  float2* const S = reinterpret_cast<float2*>(smem_raw);
-  int fam, blk;
-  if ((int)blockIdx.x < bx) { fam = 0; blk = blockIdx.x; }
-  else if ((int)blockIdx.x < bx + by) { fam = 1; blk = blockIdx.x - bx; }
-  else { fam = 2; blk = blockIdx.x - bx - by; }
-  const int per = fam == 0 ? F::FX : F::FYZ;
-  const long long f0 = (long long)blk * per;
-  const int nq = (int)min((long long)per, fg.nf[fam] - f0);
-  float2* const out = faces + fg.foff[fam] + f0 * FS;
-  auto ld = [](const float2 v) -> dfv { return {v.x, v.y}; };
-  auto st = [](const dfv v) -> float2 { return make_float2(v.hi, v.lo); };
-  if (fam == 0) {
-    float2* V = S;
-    float2* P = S + F::FX * C * C;
-    float2* Q = P + F::FX * C * M;
-    for (int t = threadIdx.x; t < nq * C * C; t += NT) {
-      const int q = t % nq, e = t / nq, y = e % C, z = e / C;
-      V[q * C * C + y * C + z] = st(df_from_double(u[face_origin<K>(fg, 0, f0 + q) + fg.py * y + fg.pz * z]));
-    }
-    __syncthreads();
-    for (int t = threadIdx.x; t < nq * C; t += NT) {
-      const int q = t / C, y = t % C;
-      dfv v[C];
-#pragma unroll
-      for (int z = 0; z < C; ++z) v[z] = ld(V[q * C * C + y * C + z]);
-#pragma unroll
-      for (int l = 0; l < M; ++l) {
-        df_acc a = {0.f, 0.f}, b = {0.f, 0.f};
-        patch_row_df<K, 0>(l, v, a);
-        patch_row_df<K, 1>(l, v, b);
-        P[(q * C + y) * M + l] = st(df_acc_value(a));
-        Q[(q * C + y) * M + l] = st(df_acc_value(b));
-      }
-    }
-    __syncthreads();
-    for (int t = threadIdx.x; t < nq * M; t += NT) {
-      const int q = t / M, l = t % M;
-      dfv p[C], r[C];
-#pragma unroll
-      for (int y = 0; y < C; ++y) {
-        p[y] = ld(P[(q * C + y) * M + l]);
-        r[y] = ld(Q[(q * C + y) * M + l]);
-      }
-      float2* o = out + (long long)q * FS + l * M;
-#pragma unroll
-      for (int j = 0; j < M; ++j) {
-        df_acc a = {0.f, 0.f}, b = {0.f, 0.f};
-        patch_row_df<K, 0>(j, p, a);
-        patch_row_df<K, 1>(j, p, b);
-        patch_row_df<K, 0>(j, r, b);
-        o[j] = st(df_acc_value(a));
-        o[M * M + j] = st(df_acc_value(b));
-      }
-    }
-    return;
-  }
-  float2* P = S + F::FYZ * (fam == 1 ? M * C : M * M);
-  float2* Q = P + F::FYZ * M * M;
-  if (fam == 1) {
-    float2* W = S;
-    for (int t = threadIdx.x; t < nq * M * C; t += NT) {
-      const int a = t % M, e = t / M, z = e % C, q = e / C;
-      W[(q * M + a) * C + z] = st(df_from_double(u[face_origin<K>(fg, 1, f0 + q) + a + fg.pz * z]));
-    }
-    __syncthreads();
-    for (int t = threadIdx.x; t < nq * M; t += NT) {
-      const int q = t / M, a = t % M;
-      dfv v[C];
-#pragma unroll
-      for (int z = 0; z < C; ++z) v[z] = ld(W[(q * M + a) * C + z]);
-#pragma unroll
-      for (int l = 0; l < M; ++l) {
-        df_acc x = {0.f, 0.f}, y = {0.f, 0.f};
-        patch_row_df<K, 0>(l, v, x);
-        patch_row_df<K, 1>(l, v, y);
-        P[(q * M + a) * M + l] = st(df_acc_value(x));
-        Q[(q * M + a) * M + l] = st(df_acc_value(y));
-      }
-    }
-  } else {
-    float2* Sz = S;
-    for (int t = threadIdx.x; t < nq * M * M; t += NT) {
-      const int a = t % M, e = t / M, b = e % M, q = e / M;
-      Sz[(q * M + a) * M + b] = st(df_from_double(u[face_origin<K>(fg, 2, f0 + q) + a + fg.py * b]));
-    }
-    __syncthreads();
-    for (int t = threadIdx.x; t < nq * M; t += NT) {
-      const int q = t / M, a = t % M;
-      dfv v[M];
-#pragma unroll
-      for (int b = 0; b < M; ++b) v[b] = ld(Sz[(q * M + a) * M + b]);
-#pragma unroll
-      for (int j = 0; j < M; ++j) {
-        df_acc x = {0.f, 0.f}, y = {0.f, 0.f};
-        patch_row_int_df<K, 0>(j, v, x);
-        patch_row_int_df<K, 1>(j, v, y);
-        P[(q * M + a) * M + j] = st(df_acc_value(x));
-        Q[(q * M + a) * M + j] = st(df_acc_value(y));
-      }
-    }
-  }
-  __syncthreads();
-  for (int t = threadIdx.x; t < nq * M; t += NT) {
-    const int q = t / M, l = t % M;
-    dfv p[M], r[M];
-#pragma unroll
-    for (int a = 0; a < M; ++a) {
-      p[a] = ld(P[(q * M + a) * M + l]);
-      r[a] = ld(Q[(q * M + a) * M + l]);
-    }
-    float2* o = out + (long long)q * FS + l * M;
-#pragma unroll
-    for (int i = 0; i < M; ++i) {
-      df_acc x = {0.f, 0.f}, y = {0.f, 0.f};
-      patch_row_int_df<K, 1>(i, p, x);
-      patch_row_int_df<K, 0>(i, r, x);
-      patch_row_int_df<K, 0>(i, p, y);
-      o[i] = st(df_acc_value(x));
-      o[M * M + i] = st(df_acc_value(y));
-    }
-  }
-}
-
 // Shared-memory plan of the shared-face sweep, per patch (elements of T):
 //   IN (NBUF copies): interior rows of b (TMA box rows of XB, as in the
 //       closure kernel), then the face blocks X0 X1 Y0 Y1 Z0 Z1 of the patch
@@ -374,7 +194,7 @@ struct FaceSweepSmem {
   static constexpr int XB = (C + A - 1 + A - 1) / A * A;
   static constexpr int R128 = 128 / (int)sizeof(T);
   static constexpr int NBIN = (M * M * XB + R128 - 1) / R128 * R128;
-  static constexpr int FS = face_fields(K);
+  static constexpr int FS = face_elems(K);
   static constexpr int IN = (NBIN + 6 * FS + R128 - 1) / R128 * R128;
   static constexpr int WB = M * M * M;
   static constexpr int SUMS = 2 * FS;
@@ -410,15 +230,10 @@ __global__ void __launch_bounds__(NT) patch_face_kernel(const __grid_constant__ 
                                                         const __grid_constant__ CUtensorMap bmap) {
   using Z = FaceSweepSmem<K>;
   constexpr int C = Z::C, M = Z::M, XB = Z::XB, FS = Z::FS, LINES = M * M;
-  // FP64: the FD transforms run in double-float arithmetic (pairs of floats
-  // in WB; the diagonal's float pairs follow the FP64 diagonal in dinv)
-  constexpr bool DF = sizeof(T) == 8;
   static_assert(PPC <= 32, "one lane of warp 0 issues the copies of one patch");
   extern __shared__ __align__(128) unsigned char smem_raw[];
   T* const IN0 = reinterpret_cast<T*>(smem_raw + ((128 - (async::smem_u32(smem_raw) & 127)) & 127));
   T* const WB = IN0 + NBUF * PPC * Z::IN;
-  float2* const WB2 = reinterpret_cast<float2*>(WB);  // used when DF: same element size
-  const float2* const dinv_df = reinterpret_cast<const float2*>(fa.dinv + M * M * M);
   T* const SUMS = WB + PPC * Z::WB;
   __shared__ long long s_origin[2][PPC];
   __shared__ int s_x[2][PPC][3];     // closure origin (lattice coordinates)
@@ -512,13 +327,7 @@ __global__ void __launch_bounds__(NT) patch_face_kernel(const __grid_constant__ 
     for (int idx = threadIdx.x; idx < nvalid * Z::SUMS; idx += NT) {
       const int q = idx / Z::SUMS, e = idx % Z::SUMS;
       const T* F = IN + q * Z::IN + Z::NBIN + (e < FS ? 2 * FS : 4 * FS) + e % FS;
-      if constexpr (DF) {
-        const float2* F2 = reinterpret_cast<const float2*>(F);
-        const dfv v = df_add({F2[0].x, F2[0].y}, {F2[FS].x, F2[FS].y});
-        reinterpret_cast<float2*>(SUMS)[idx] = make_float2(v.hi, v.lo);
-      } else {
-        SUMS[idx] = F[0] + F[FS];
-      }
+      SUMS[idx] = F[0] + F[FS];
     }
     __syncthreads();
 
@@ -533,51 +342,6 @@ __global__ void __launch_bounds__(NT) patch_face_kernel(const __grid_constant__ 
       // sum) and those of row l for the z faces (H1[j][.], H2[j][.])
       const T* FY = (j < K - 1 ? FX + 2 * FS : j > K - 1 ? FX + 3 * FS : SUMS + q * Z::SUMS) + l * M;
       const T* FZ = (l < K - 1 ? FX + 4 * FS : l > K - 1 ? FX + 5 * FS : SUMS + q * Z::SUMS + FS) + j * M;
-      if constexpr (DF) {
-        // the same residual in double-float: faces and sums are float pairs
-        auto ld = [](const T* p, int i) -> dfv {
-          const float2 v = reinterpret_cast<const float2*>(p)[i];
-          return {v.x, v.y};
-        };
-        const dfv f10 = ld(FX, l * M + j), f20 = ld(FX, M * M + l * M + j);
-        const dfv f11 = ld(FX, FS + l * M + j), f21 = ld(FX, FS + M * M + l * M + j);
-        const int cj = j < K ? 0 : C - 1, cl = l < K ? 0 : C - 1;
-        float myh, myl, kyh, kyl, mzh, mzl, kzh, kzl;
-        patch_entry_df<K, 0, true>(j, cj, myh, myl);
-        patch_entry_df<K, 1, true>(j, cj, kyh, kyl);
-        patch_entry_df<K, 0, true>(l, cl, mzh, mzl);
-        patch_entry_df<K, 1, true>(l, cl, kzh, kzl);
-        const float sbf = (float)fa.sb;  // h^{2-d} = n, exact in float
-        dfv rd[M], yd[M];
-#pragma unroll
-        for (int i = 0; i < M; ++i) {
-          const dfv bb = df_mul(df_from_double(Bq[i]), {sbf, 0.f});
-          df_acc acc = {bb.hi, bb.lo};
-          float h, lo;
-          if (band_lo(i + 1, K) == 0) {
-            patch_entry_df<K, 1, true>(i, 0, h, lo);
-            df_acc_add(acc, h, lo, f10);
-            patch_entry_df<K, 0, true>(i, 0, h, lo);
-            df_acc_add(acc, h, lo, f20);
-          }
-          if (band_hi(i + 1, K) == 2 * K) {
-            patch_entry_df<K, 1, true>(i, C - 1, h, lo);
-            df_acc_add(acc, h, lo, f11);
-            patch_entry_df<K, 0, true>(i, C - 1, h, lo);
-            df_acc_add(acc, h, lo, f21);
-          }
-          df_acc_add(acc, kyh, kyl, ld(FY, M * M + i));
-          df_acc_add(acc, myh, myl, ld(FY, i));
-          df_acc_add(acc, kzh, kzl, ld(FZ, M * M + i));
-          df_acc_add(acc, mzh, mzl, ld(FZ, i));
-          rd[i] = df_acc_value(acc);
-        }
-        fd_forward_df<K>(rd, yd);
-        float2* R = WB2 + q * Z::WB + M * ln;
-#pragma unroll
-        for (int i = 0; i < M; ++i) R[i] = make_float2(yd[i].hi, yd[i].lo);
-        continue;
-      }
       const T f10 = FX[l * M + j], f20 = FX[M * M + l * M + j];
       const T f11 = FX[FS + l * M + j], f21 = FX[FS + M * M + l * M + j];
       // column 0 (rows up to K-1) or 2K of rows j and l
@@ -604,41 +368,28 @@ __global__ void __launch_bounds__(NT) patch_face_kernel(const __grid_constant__ 
     // ---- local solve by fast diagonalisation (App. A.3), in place in WB ----
     for (int idx = threadIdx.x; idx < nvalid * LINES; idx += NT) {  // forward y
       const int q = idx / LINES, l = idx % LINES;
-      if constexpr (DF) fd_smem_line_df<K, true>(WB2 + q * Z::WB + (l % M) + (l / M) * M * M, M);
-      else fd_smem_line<K, true>(WB + q * Z::WB + (l % M) + (l / M) * M * M, M);
+      fd_smem_line<K, true>(WB + q * Z::WB + (l % M) + (l / M) * M * M, M);
     }
     __syncthreads();
     for (int idx = threadIdx.x; idx < nvalid * LINES; idx += NT) {  // forward z, diagonal, backward z
       const int q = idx / LINES, l = idx % LINES;
-      if constexpr (DF) fd_smem_line_solve_df<K>(WB2 + q * Z::WB + l, M * M, dinv_df + l, M * M);
-      else fd_smem_line_solve<K>(WB + q * Z::WB + l, M * M, fa.dinv + l, M * M);
+      fd_smem_line_solve<K>(WB + q * Z::WB + l, M * M, fa.dinv + l, M * M);
     }
     __syncthreads();
     for (int idx = threadIdx.x; idx < nvalid * LINES; idx += NT) {  // backward y
       const int q = idx / LINES, l = idx % LINES;
-      if constexpr (DF) fd_smem_line_df<K, false>(WB2 + q * Z::WB + (l % M) + (l / M) * M * M, M);
-      else fd_smem_line<K, false>(WB + q * Z::WB + (l % M) + (l / M) * M * M, M);
+      fd_smem_line<K, false>(WB + q * Z::WB + (l % M) + (l / M) * M * M, M);
     }
     __syncthreads();
     // ---- backward FD along x and scatter (eq. "scatter") ----
     for (int idx = threadIdx.x; idx < nvalid * LINES; idx += NT) {
       const int q = idx / LINES, l = idx % LINES;
       T d[M];
-      if constexpr (DF) {
-        const float2* R = WB2 + q * Z::WB + M * l;
-        dfv yv[M], dd[M];
+      const T* R = WB + q * Z::WB + M * l;
+      T yv[M];
 #pragma unroll
-        for (int i = 0; i < M; ++i) yv[i] = {R[i].x, R[i].y};
-        fd_backward_df<K>(yv, dd);
-#pragma unroll
-        for (int i = 0; i < M; ++i) d[i] = df_to_double(dd[i]);
-      } else {
-        const T* R = WB + q * Z::WB + M * l;
-        T yv[M];
-#pragma unroll
-        for (int i = 0; i < M; ++i) yv[i] = R[i];
-        fd_backward<K>(yv, d);
-      }
+      for (int i = 0; i < M; ++i) yv[i] = R[i];
+      fd_backward<K>(yv, d);
       T* __restrict__ row = fa.u + s_origin[cur][q] + 1 + fa.py * (l % M + 1) + fa.pz * (l / M + 1);
       if (om == T(1)) {
 #pragma unroll
@@ -659,15 +410,10 @@ __global__ void __launch_bounds__(NT) patch_face_kernel(const __grid_constant__ 
 // patches per CTA, threads and input buffers of the shared-face sweep
 template <int K>
 struct FaceSweepCfg {
-  // FP64 (double-float arithmetic, bound by FP32 issue) at k = 3, 4: one input
-  // buffer, which leaves room for more resident CTAs (measured on GB300 at
-  // 64^3: k = 3 1.30 -> 1.12 ms, k = 4 3.16 -> 3.03 ms per sweep); FP32 and
-  // the other degrees keep the double-buffered inputs
-  static constexpr bool F64 = sizeof(T) == 8;
-  static constexpr int PPC = K == 3 ? (F64 ? 5 : 10) : K == 4 ? 5 : K == 5 ? 3 : K == 6 ? 2 : 1;
-  // (FP32 k = 7: 160 threads, 2.75 -> 2.67 ms per 48^3 sweep)
-  static constexpr int NT = K == 7 ? (F64 ? 192 : 160) : K == 3 && F64 ? 128 : 256;
-  static constexpr int NBUF = (K <= 4 && !F64) || K == 7 ? 2 : 1;
+  static constexpr int PPC = K == 3 ? 10 : K == 4 ? 5 : K == 5 ? 3 : K == 6 ? 2 : 1;
+  // (k = 7: 160 threads, 2.75 -> 2.67 ms per 48^3 sweep)
+  static constexpr int NT = K == 7 ? 160 : 256;
+  static constexpr int NBUF = K <= 4 || K == 7 ? 2 : 1;
   static constexpr int SMEM = PPC * FaceSweepSmem<K>::per_patch(NBUF) * (int)sizeof(T) + 128;
   static_assert(SMEM <= 227 * 1024, "shared-face sweep exceeds the shared memory of a CTA");
   static_assert(PPC * (2 * K - 1) * (2 * K - 1) <= NT + 32 * 2,
@@ -675,35 +421,12 @@ struct FaceSweepCfg {
 };
 constexpr int kFaceThreads = 128;
 
-static FaceGeom face_geom(const PatchLaunch& pl) {
-  FaceGeom fg;
-  fg.py = pl.g.py;
-  fg.pz = pl.g.pz;
-  for (int a = 0; a < 3; ++a) {
-    fg.first[a] = pl.first[a];
-    fg.count[a] = pl.count[a];
-  }
-  const long long cx = pl.count[0], cy = pl.count[1], cz = pl.count[2];
-  fg.nf[0] = (cx + 1) * cy * cz;
-  fg.nf[1] = cx * (cy + 1) * cz;
-  fg.nf[2] = cx * cy * (cz + 1);
-  const long long fs = face_fields(pl.g.k);
-  fg.foff[0] = 0;
-  fg.foff[1] = fg.nf[0] * fs;
-  fg.foff[2] = fg.foff[1] + fg.nf[1] * fs;
-  return fg;
-}
-
 template <int K>
 static int face_sweep_impl(const PatchLaunch& pl, T* u, const T* b, const T* dinv, T* faces, cudaStream_t s) {
   using FC = FaceCfg<K, kFaceThreads>;
   using SC = FaceSweepCfg<K>;
   using Z = FaceSweepSmem<K>;
-  // FP64 problems evaluate the faces in double-float (float-pair fields)
-  auto fk = [] {
-    if constexpr (sizeof(T) == 8) return face_kernel_df<K, kFaceThreads>;
-    else return face_kernel<K, kFaceThreads>;
-  }();
+  auto fk = face_kernel<K, kFaceThreads>;
   auto pk = patch_face_kernel<K, SC::NT, SC::PPC, SC::NBUF>;
   static PerDevice<int> per_sm_dev;
   int* const per_sm_p = per_sm_dev.get();
@@ -715,15 +438,11 @@ static int face_sweep_impl(const PatchLaunch& pl, T* u, const T* b, const T* din
         per_sm <= 0)
       return GMG_ERR_CUDA;
   }
-  const FaceGeom fg = face_geom(pl);
+  const FaceGeom fg = face_geom(pl, (int)sizeof(T));
   const long long bx = (fg.nf[0] + FC::FX - 1) / FC::FX, by = (fg.nf[1] + FC::FYZ - 1) / FC::FYZ,
                   bz = (fg.nf[2] + FC::FYZ - 1) / FC::FYZ;
   if (bx + by + bz > (1LL << 31) - 1) return GMG_ERR_UNSUPPORTED;
-  if constexpr (sizeof(T) == 8)
-    fk<<<(unsigned)(bx + by + bz), kFaceThreads, FC::SMEM, s>>>(u, reinterpret_cast<float2*>(faces), fg, (int)bx,
-                                                                (int)by);
-  else
-    fk<<<(unsigned)(bx + by + bz), kFaceThreads, FC::SMEM, s>>>(u, faces, fg, (int)bx, (int)by);
+  fk<<<(unsigned)(bx + by + bz), kFaceThreads, FC::SMEM, s>>>(u, faces, fg, (int)bx, (int)by);
   count_launch();
   if (cudaGetLastError() != cudaSuccess) return GMG_ERR_CUDA;
 
@@ -752,12 +471,6 @@ static int face_sweep_impl(const PatchLaunch& pl, T* u, const T* b, const T* din
   return cudaGetLastError() == cudaSuccess ? GMG_OK : GMG_ERR_CUDA;
 }
 
-// elements of the face buffer for one colour launch of pl's geometry
-inline long long face_buffer_elems_t(const PatchLaunch& pl) {
-  const FaceGeom fg = face_geom(pl);
-  return (fg.nf[0] + fg.nf[1] + fg.nf[2]) * face_fields(pl.g.k);
-}
-
 }  // namespace GMG_NS
 }  // namespace gmg
 
@@ -782,7 +495,7 @@ int launch_patch_faces<GMG_T>(const PatchLaunch& pl, GMG_T* u, const GMG_T* b, c
 
 template <>
 long long face_buffer_elems<GMG_T>(const PatchLaunch& pl) {
-  return GMG_NS::face_buffer_elems_t(pl);
+  return face_buffer_total(pl, (int)sizeof(GMG_T));
 }
 
 }  // namespace gmg

@@ -141,6 +141,8 @@ template <typename T>
 int launch_patch_faces(const PatchLaunch& pl, T* u, const T* b, const T* dinv, T* faces, cudaStream_t s);
 template <typename T>
 long long face_buffer_elems(const PatchLaunch& pl);
+// coefficient tables of the FP64 form (pair_sweep_f64.cu)
+int upload_pair_sweep_tables(int k, const double* Mp, const double* Kp, const double* That);
 
 template <typename T>
 int launch_apply(const ApplyLaunch& al, const T* x, T* y, const T* bvec, cudaStream_t s);

@@ -3,7 +3,6 @@
 #define GMG_NS f64
 #include "patch_kernels.cuh"
 #include "patch_launch.cuh"
-#include "face_kernels.cuh"
 #include "small_kernels.cuh"
 
 namespace gmg {
