@@ -111,6 +111,9 @@ long long launch_count();
 template <typename T>
 int upload_patch_tables(int k, const double* Mp, const double* Kp, const double* That,
                         const double* Mc, const double* Kc, cudaStream_t s);
+// tables of the closure form of the sweep (called by upload_patch_tables)
+template <typename T>
+int upload_closure_tables(int k, const double* Mp, const double* Kp, const double* That);
 template <typename T>
 int launch_patch_colour(const PatchLaunch& pl, T* u, const T* b, const T* dinv, cudaStream_t s);
 // one colour of a coarse level with the one-output-per-thread kernel (FP64 problems,
@@ -123,6 +126,9 @@ int launch_patch_small(const PatchLaunch& pl, T* u, const T* b, const T* dinv, c
 template <typename T>
 int launch_patch_table(int dim, int k, const PatchLaunch* pls, T* const* us, const T* const* bs,
                        int n, const T* dinv, int ppc, cudaStream_t s);
+// the FP64 3D closure form at degrees 7 and 8, one patch per thread (patch_f64.cu)
+int launch_line_table(int k, const PatchLaunch* pls, double* const* us, const double* const* bs, int n,
+                      const double* dinv, cudaStream_t s);
 // Tensor-core sweep (patch_tc.cu): 3D, FP32 data, degrees 4..7, combined
 // mode only (GMG_ERR_UNSUPPORTED otherwise).
 bool tc_supported(int dim, int k);

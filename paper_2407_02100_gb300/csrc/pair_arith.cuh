@@ -105,5 +105,70 @@ __device__ __forceinline__ void df2_acc_add(df2_acc& a, df2_coef c, df2 x) {
 }
 __device__ __forceinline__ df2 df2_acc_value(df2_acc a) { return df2_norm(a.s, a.e); }
 
+// The two arithmetics of the pair kernels, under the same names: a value, an
+// accumulator, a coefficient and their forms in shared and constant memory.
+struct PairDF {  // double-float (FP64 problems)
+  using T = double;
+  using val = df2;
+  using acc = df2_acc;
+  using coef = df2_coef;
+  using mem = float4;  // (hi, hi, lo, lo)
+  using tab = float4;  // (h, h, l, l)
+  static __device__ __forceinline__ val load(const mem& a) {
+    const ulonglong2 v = reinterpret_cast<const ulonglong2&>(a);
+    return {{v.x}, {v.y}};
+  }
+  static __device__ __forceinline__ void store(mem& a, val v) {
+    reinterpret_cast<ulonglong2&>(a) = make_ulonglong2(v.hi.v, v.lo.v);
+  }
+  static __device__ __forceinline__ coef coefficient(const tab& c) {
+    const ulonglong2 v = reinterpret_cast<const ulonglong2&>(c);
+    return {{v.x}, {v.y}};
+  }
+  static __device__ __forceinline__ acc zero() { return {{0}, {0}}; }
+  static __device__ __forceinline__ acc first(coef c, val x) { return df2_acc_first(c, x); }
+  static __device__ __forceinline__ void add(acc& a, coef c, val x) { df2_acc_add(a, c, x); }
+  static __device__ __forceinline__ val value(acc a) { return df2_acc_value(a); }
+  static __device__ __forceinline__ val sum(val a, val b) { return df2_add(a, b); }
+  static __device__ __forceinline__ val diff(val a, val b) { return df2_sub(a, b); }
+  static __device__ __forceinline__ acc scaled(float c, val x) { return df2_acc_scaled(f2_dup(c), x); }
+  static __device__ __forceinline__ val pack(T a, T b) { return df2_make(df_from_double(a), df_from_double(b)); }
+  static __device__ __forceinline__ val pack_neg(T a, T b) {  // (a negated double would be an FP64 instruction)
+    return df2_make(df_neg(df_from_double(a)), df_neg(df_from_double(b)));
+  }
+  // times entry i of the FD diagonal (n entries, followed by their float pairs)
+  static __device__ __forceinline__ val diagonal(const T* dinv, int n, int i, val v) {
+    const float2 d = __ldg(reinterpret_cast<const float2*>(dinv + n) + i);
+    return value(first({f2_dup(d.x), f2_dup(d.y)}, v));
+  }
+  static __device__ __forceinline__ T x(val v) { return df_to_double(df2_x(v)); }
+  static __device__ __forceinline__ T y(val v) { return df_to_double(df2_y(v)); }
+};
+struct PairF32 {  // single precision
+  using T = float;
+  using val = f2;
+  using acc = f2;
+  using coef = f2;
+  using mem = float2;
+  using tab = float2;  // (c, c)
+  static __device__ __forceinline__ val load(const mem& a) { return {reinterpret_cast<const unsigned long long&>(a)}; }
+  static __device__ __forceinline__ void store(mem& a, val v) { reinterpret_cast<unsigned long long&>(a) = v.v; }
+  static __device__ __forceinline__ coef coefficient(const tab& c) { return load(c); }
+  static __device__ __forceinline__ acc zero() { return {0}; }
+  static __device__ __forceinline__ acc first(coef c, val x) { return f2_fma(c, x, f2{0}); }
+  static __device__ __forceinline__ void add(acc& a, coef c, val x) { a = f2_fma(c, x, a); }
+  static __device__ __forceinline__ val value(acc a) { return a; }
+  static __device__ __forceinline__ val sum(val a, val b) { return f2_add(a, b); }
+  static __device__ __forceinline__ val diff(val a, val b) { return f2_sub(a, b); }
+  static __device__ __forceinline__ acc scaled(float c, val x) { return f2_fma(f2_dup(c), x, f2{0}); }
+  static __device__ __forceinline__ val pack(T a, T b) { return f2_make(a, b); }
+  static __device__ __forceinline__ val pack_neg(T a, T b) { return f2_make(-a, -b); }
+  static __device__ __forceinline__ val diagonal(const T* dinv, int, int i, val v) {
+    return f2_fma(f2_dup(__ldg(dinv + i)), v, f2{0});
+  }
+  static __device__ __forceinline__ T x(val v) { return f2_x(v); }
+  static __device__ __forceinline__ T y(val v) { return f2_y(v); }
+};
+
 }  // namespace
 }  // namespace gmg

@@ -1,0 +1,49 @@
+// Closure form of the patch sweep in double precision.
+#define GMG_PAIR_ARITH PairDF
+#include "pair_closure.cuh"
+
+namespace gmg {
+namespace {
+
+template <int DIM, int K>
+int table_launches(const PatchLaunch* pls, T* const* us, const T* const* bs, int n, const T* dinv, int ppc,
+                   cudaStream_t s) {
+  // a pair of the largest patches does not fit in shared memory: one patch
+  // per thread for those
+  if constexpr (!closure_pairs<DIM, K>()) {
+    return launch_line_table(K, pls, us, bs, n, dinv, s);
+  } else {
+    for (int i0 = 0; i0 < n; i0 += kMaxTable) {
+      PatchTable tab;
+      tab.n = 0;
+      tab.mode = pls[i0].mode;
+      tab.omega = pls[i0].omega;
+      for (int i = i0; i < std::min(n, i0 + kMaxTable); ++i)
+        if (pls[i].n_patches > 0) fill_entry(tab.e[tab.n++], pls[i], us[i], bs[i]);
+      if (tab.n == 0) continue;
+      const int st = closure_table<DIM, K>(tab, dinv, ppc, s);
+      if (st != GMG_OK) return st;
+    }
+    return GMG_OK;
+  }
+}
+
+}  // namespace
+
+template <>
+int upload_closure_tables<double>(int k, const double* Mp, const double* Kp, const double* That) {
+  return pl_upload(k, Mp, Kp, That);
+}
+
+template <>
+int launch_patch_table<double>(int dim, int k, const PatchLaunch* pls, double* const* us, const double* const* bs, int n,
+                             const double* dinv, int ppc, cudaStream_t s) {
+  GMG_DISPATCH(table_launches, dim, k, pls, us, bs, n, dinv, ppc, s)
+}
+
+template <>
+int launch_patch_colour<double>(const PatchLaunch& pl, double* u, const double* b, const double* dinv, cudaStream_t s) {
+  return launch_patch_table<double>(pl.g.dim, pl.g.k, &pl, &u, &b, 1, dinv, 0, s);
+}
+
+}  // namespace gmg

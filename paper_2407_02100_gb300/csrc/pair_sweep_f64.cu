@@ -39,6 +39,7 @@
 #include "async.cuh"
 #include "face_geom.cuh"
 #include "kernels.h"
+#define GMG_PAIR_ARITH PairDF
 #include "pair_lines.cuh"
 #include "tma_host.h"
 
@@ -61,12 +62,6 @@ struct FacePairCfg {
   static constexpr int SX = C * C + C * M, SY = M * C + M * M, SZ = 2 * M * M;
   static constexpr int SMEM = imax(PX * SX, PYZ * imax(SY, SZ)) * 16;
 };
-
-__device__ __forceinline__ df2 ld_pair(const float4& a) {
-  const ulonglong2 v = reinterpret_cast<const ulonglong2&>(a);
-  return {{v.x}, {v.y}};
-}
-__device__ __forceinline__ void st_pair(float4& a, df2 v) { reinterpret_cast<ulonglong2&>(a) = make_ulonglong2(v.hi.v, v.lo.v); }
 
 // CTAs [0, bx) evaluate x faces, [bx, bx + by) y faces, the rest z faces, two
 // consecutive faces of a family per thread.  First stage: contract z (x and y
@@ -126,14 +121,14 @@ __device__ __forceinline__ void face_family(const double* __restrict__ u, float*
         pl_cell_row<K, 0, true, Q1>(i, v, a);
         pl_cell_row<K, 1, true, Q1>(i, v, b);
         const int l = r ? M - i : i - 1;
-        st_pair(p[l], df2_acc_value(a));
-        st_pair(q[l], df2_acc_value(b));
+        PA::store(p[l], df2_acc_value(a));
+        PA::store(q[l], df2_acc_value(b));
       }
       pl_centre<K, 0, Q1>(r == 0, v, ca);
       pl_centre<K, 1, Q1>(r == 0, v, cb);
     }
-    st_pair(p[K - 1], df2_acc_value(ca));
-    st_pair(q[K - 1], df2_acc_value(cb));
+    PA::store(p[K - 1], df2_acc_value(ca));
+    PA::store(q[K - 1], df2_acc_value(cb));
   }
   __syncthreads();
   // second stage, line l of a pair: M p and K p + M q; the two-term sum is
@@ -160,8 +155,8 @@ __device__ __forceinline__ void face_family(const double* __restrict__ u, float*
 #pragma unroll
       for (int c = Q2; c <= K; ++c) {
         const int y = r ? N1 - 1 - (c - Q2) : c - Q2;
-        v[c] = ld_pair(p[y * L1]);
-        w[c] = ld_pair(q[y * M]);
+        v[c] = PA::load(p[y * L1]);
+        w[c] = PA::load(q[y * M]);
       }
 #pragma unroll
       for (int i = 1; i < K; ++i) {

@@ -6,6 +6,7 @@
 
 #include "../../include/gmg.h"
 #include "coef_split.h"
+#include "patch_dispatch.h"
 #include "tma_host.h"
 #include "staged_apply.cuh"
 
@@ -13,28 +14,6 @@ namespace gmg {
 namespace GMG_NS {
 
 constexpr int kApplyThreads = 128;
-
-// Sweep kernel configuration: patches per CTA (enough interior lines per
-// stage to fill whole warps), threads, and double buffering of the inputs
-// whenever two input buffers fit in about half of the shared memory.
-template <int DIM, int K>
-struct SweepCfg {
-  // FP64 is bound by the FP64 pipe: many patches per CTA for full warps, one
-  // input buffer (occupancy hides the gather).  FP32 is bound by issue and
-  // latency: fewer patches per CTA, double-buffered inputs.
-  static constexpr bool F64 = sizeof(T) == 8;
-  // FP32 3D k = 4: one patch per CTA of 64 threads (many small CTAs hide the
-  // stage barriers better; measured 1.023 -> 0.934 ms per 64^3 sweep)
-  static constexpr int PPC = DIM == 2 ? 8
-                           : F64 ? (K <= 2 ? 8 : K <= 4 ? 4 : K <= 6 ? 2 : 1)
-                                 : (K <= 2 ? 8 : K == 3 ? 4 : 1);
-  static constexpr int NT = DIM == 3 && !F64 && K == 4 ? 64
-                          : DIM == 3 && (K >= 6 || (F64 && K >= 3)) ? 256 : 128;
-  static constexpr int NBUF =
-      !F64 && PPC * SweepSmem<DIM, K>::per_patch(2) * (int)sizeof(T) <= 110 * 1024 ? 2 : 1;
-  static constexpr int SMEM = PPC * SweepSmem<DIM, K>::per_patch(NBUF) * (int)sizeof(T);
-  static_assert(SMEM <= 227 * 1024, "sweep kernel shared memory exceeds the per-CTA limit");
-};
 
 // Tile of the operator kernel (cells per direction x, y, z) and its threads.
 // A tile recomputes a halo of K + 1 nodes below it in each direction, so
@@ -71,133 +50,6 @@ template <typename KernelT>
 static int prepare(KernelT kern, int smem) {
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
     return GMG_ERR_CUDA;
-  return GMG_OK;
-}
-
-// Fill the table entries' group ranges for PPC patches per CTA.
-static inline int table_groups(PatchTable& tab, int ppc) {
-  int g = 0;
-  for (int i = 0; i < tab.n; ++i) {
-    tab.e[i].group_begin = g;
-    g += (tab.e[i].n_patches + ppc - 1) / ppc;
-  }
-  tab.total_groups = g;
-  return g;
-}
-
-// ---- TMA gather: every vector of the table must allow the boxes ----
-static bool tma_usable(const PatchTable& tab, int dim) {
-  for (int i = 0; i < tab.n; ++i) {
-    const PatchEntry& e = tab.e[i];
-    if (e.N < 2 || !tma_vector_ok(e.u, (int)sizeof(T), dim, e.py, e.pz) ||
-        !tma_vector_ok(e.b, (int)sizeof(T), dim, e.py, e.pz))
-      return false;
-  }
-  return true;
-}
-
-template <int DIM, int K, int PPC, int NT, int NBUF, int ME>
-static int launch_table_cfg(PatchTable& tab, const T* dinv, cudaStream_t s) {
-  using Z = SweepSmem<DIM, K, (ME > 0)>;
-  constexpr int SMEM = PPC * Z::per_patch(NBUF) * (int)sizeof(T) + (ME > 0 ? 128 : 0);
-  static_assert(SMEM <= 227 * 1024, "sweep kernel shared memory exceeds the per-CTA limit");
-  auto kern = patch_colour_kernel<DIM, K, NT, PPC, NBUF, ME>;
-  static PerDevice<int> per_sm_dev;  // resident CTAs per SM (persistent grid)
-  int* const per_sm_p = per_sm_dev.get();
-  if (!per_sm_p) return GMG_ERR_CUDA;
-  int& per_sm = *per_sm_p;
-  if (per_sm == 0) {
-    if (prepare(kern, SMEM) != GMG_OK) return GMG_ERR_CUDA;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, NT, SMEM) != cudaSuccess ||
-        per_sm <= 0)
-      return GMG_ERR_CUDA;
-  }
-  const int ngroups = table_groups(tab, PPC);
-  if (ngroups <= 0) return GMG_OK;
-  TmaMaps<ME> maps;
-  if constexpr (ME > 0) {
-    for (int i = 0; i < tab.n; ++i) {
-      const PatchEntry& e = tab.e[i];
-      if (!tma_encode(&maps.u[i], e.u, (int)sizeof(T), DIM, e.N, e.py, e.pz, Z::XU, Z::C) ||
-          !tma_encode(&maps.b[i], e.b, (int)sizeof(T), DIM, e.N, e.py, e.pz, Z::XB, Z::M))
-        return GMG_ERR_CUDA;
-    }
-  }
-  int* const flag = device_wait_flag();
-  if (!flag) return GMG_ERR_CUDA;
-  const int grid = std::min(ngroups, per_sm * sm_count());
-  kern<<<grid, NT, SMEM, s>>>(tab, dinv, maps, flag);
-  count_launch();
-  return cudaGetLastError() == cudaSuccess ? GMG_OK : GMG_ERR_CUDA;
-}
-
-// the TMA-gather variant when every vector of the table allows it, else the
-// per-element cp.async gather
-template <int DIM, int K, int PPC, int NT, int NBUF>
-static int launch_table_gather(PatchTable& tab, const T* dinv, cudaStream_t s) {
-  if (tma_usable(tab, DIM)) {
-    if (tab.n == 1) return launch_table_cfg<DIM, K, PPC, NT, NBUF, 1>(tab, dinv, s);
-    return launch_table_cfg<DIM, K, PPC, NT, NBUF, kMaxTable>(tab, dinv, s);
-  }
-  return launch_table_cfg<DIM, K, PPC, NT, NBUF, 0>(tab, dinv, s);
-}
-
-// default configuration (SweepCfg), or a tuned patches-per-CTA variant
-template <int DIM, int K>
-static int launch_table(PatchTable& tab, const T* dinv, int ppc, cudaStream_t s) {
-  using Cfg = SweepCfg<DIM, K>;
-  if constexpr (DIM == 3 && sizeof(T) == 4 && K <= 4) {
-    constexpr int NB = SweepCfg<DIM, K>::NBUF;
-    if (ppc == 1) return launch_table_gather<DIM, K, 1, 128, NB>(tab, dinv, s);
-    if (ppc == 2) return launch_table_gather<DIM, K, 2, 128, NB>(tab, dinv, s);
-    if (ppc == 4) return launch_table_gather<DIM, K, 4, 128, NB>(tab, dinv, s);
-  }
-  return launch_table_gather<DIM, K, Cfg::PPC, Cfg::NT, Cfg::NBUF>(tab, dinv, s);
-}
-
-static void fill_entry(PatchEntry& e, const PatchLaunch& pl, void* u, const void* b) {
-  e.N = pl.g.N;
-  e.py = pl.g.py;
-  e.pz = pl.g.pz;
-  for (int a = 0; a < 3; ++a) {
-    e.first[a] = pl.first[a];
-    e.count[a] = pl.count[a];
-  }
-  e.n_patches = pl.n_patches;
-  e.group_begin = 0;
-  e.sb = pl.sb;
-  e.u = u;
-  e.b = b;
-  e.plist = pl.plist;
-}
-
-template <int DIM, int K>
-static int patch_impl(const PatchLaunch& pl, T* u, const T* b, const T* dinv, cudaStream_t s) {
-  if (pl.n_patches <= 0) return GMG_OK;
-  PatchTable tab;
-  tab.n = 1;
-  tab.mode = pl.mode;
-  tab.omega = pl.omega;
-  fill_entry(tab.e[0], pl, u, b);
-  return launch_table<DIM, K>(tab, dinv, 0, s);
-}
-
-template <int DIM, int K>
-static int table_impl(const PatchLaunch* pls, T* const* us, const T* const* bs, int n, const T* dinv,
-                      int ppc, cudaStream_t s) {
-  for (int i0 = 0; i0 < n; i0 += kMaxTable) {
-    PatchTable tab;
-    tab.n = 0;
-    tab.mode = pls[i0].mode;
-    tab.omega = pls[i0].omega;
-    for (int i = i0; i < std::min(n, i0 + kMaxTable); ++i) {
-      if (pls[i].n_patches <= 0) continue;
-      fill_entry(tab.e[tab.n++], pls[i], us[i], bs[i]);
-    }
-    if (tab.n == 0) continue;
-    const int st = launch_table<DIM, K>(tab, dinv, ppc, s);
-    if (st != GMG_OK) return st;
-  }
   return GMG_OK;
 }
 
@@ -253,27 +105,6 @@ static int apply_impl(const ApplyLaunch& al, const T* x, T* y, const T* bvec, cu
   return apply_cfg<DIM, K, Cfg::BX, Cfg::BY, Cfg::BZ, Cfg::NT>(al, x, y, bvec, s);
 }
 
-#define GMG_DISPATCH(FN, DIMV, KV, ...)                                  \
-  switch ((DIMV) * 16 + (KV)) {                                          \
-    case 2 * 16 + 1: return FN<2, 1>(__VA_ARGS__);                       \
-    case 2 * 16 + 2: return FN<2, 2>(__VA_ARGS__);                       \
-    case 2 * 16 + 3: return FN<2, 3>(__VA_ARGS__);                       \
-    case 2 * 16 + 4: return FN<2, 4>(__VA_ARGS__);                       \
-    case 2 * 16 + 5: return FN<2, 5>(__VA_ARGS__);                       \
-    case 2 * 16 + 6: return FN<2, 6>(__VA_ARGS__);                       \
-    case 2 * 16 + 7: return FN<2, 7>(__VA_ARGS__);                       \
-    case 2 * 16 + 8: return FN<2, 8>(__VA_ARGS__);                       \
-    case 3 * 16 + 1: return FN<3, 1>(__VA_ARGS__);                       \
-    case 3 * 16 + 2: return FN<3, 2>(__VA_ARGS__);                       \
-    case 3 * 16 + 3: return FN<3, 3>(__VA_ARGS__);                       \
-    case 3 * 16 + 4: return FN<3, 4>(__VA_ARGS__);                       \
-    case 3 * 16 + 5: return FN<3, 5>(__VA_ARGS__);                       \
-    case 3 * 16 + 6: return FN<3, 6>(__VA_ARGS__);                       \
-    case 3 * 16 + 7: return FN<3, 7>(__VA_ARGS__);                       \
-    case 3 * 16 + 8: return FN<3, 8>(__VA_ARGS__);                       \
-    default: return GMG_ERR_INVALID_ARG;                                 \
-  }
-
 static int upload(int k, const double* Mp, const double* Kp, const double* That, const double* Mc,
                   const double* Kc) {
   if (k < 1 || k > 8) return GMG_ERR_INVALID_ARG;
@@ -326,20 +157,9 @@ static int upload(int k, const double* Mp, const double* Kp, const double* That,
 template <>
 int upload_patch_tables<GMG_T>(int k, const double* Mp, const double* Kp, const double* That,
                                const double* Mc, const double* Kc, cudaStream_t) {
-  return GMG_NS::upload(k, Mp, Kp, That, Mc, Kc);
-}
-
-template <>
-int launch_patch_colour<GMG_T>(const PatchLaunch& pl, GMG_T* u, const GMG_T* b, const GMG_T* dinv,
-                               cudaStream_t s) {
-  GMG_DISPATCH(GMG_NS::patch_impl, pl.g.dim, pl.g.k, pl, u, b, dinv, s)
-}
-
-template <>
-int launch_patch_table<GMG_T>(int dim, int k, const PatchLaunch* pls, GMG_T* const* us,
-                              const GMG_T* const* bs, int n, const GMG_T* dinv, int ppc,
-                              cudaStream_t s) {
-  GMG_DISPATCH(GMG_NS::table_impl, dim, k, pls, us, bs, n, dinv, ppc, s)
+  const int st = GMG_NS::upload(k, Mp, Kp, That, Mc, Kc);
+  if (st != GMG_OK) return st;
+  return upload_closure_tables<GMG_T>(k, Mp, Kp, That);
 }
 
 template <>
