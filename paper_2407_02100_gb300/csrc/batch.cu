@@ -47,6 +47,11 @@ struct gmg_batch {
   Segments seg;
   int ppc = 0;                  // tuned patches per CTA of the batched sweep (0 = default)
   cudaStream_t cap_stream = nullptr;  // private stream the graph is captured on
+  // while capturing: streams that the problems' own operations are spread
+  // over, and the events that fork them from cap_stream and join them again
+  bool capturing = false;
+  std::vector<cudaStream_t> side;
+  std::vector<cudaEvent_t> side_ev;  // one per side stream, then the fork
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t vgraph = nullptr;
   size_t graph_nodes = 0;
@@ -114,37 +119,63 @@ int batch_smooth(gmg_batch* B, int depth, int reverse, bool finest_user, void* u
   return GMG_OK;
 }
 
+// The problems' own operations at one point of the V-cycle (residual,
+// transfers, coarse solve).  They are small and independent of one another,
+// each on its problem's vectors and temporaries, so that the captured graph
+// runs them as parallel branches; without capture they run in turn.
+template <typename F>
+int each_problem(gmg_batch* B, F&& f) {
+  const int S = B->capturing ? (int)B->side.size() : 0;
+  if (S < 2) {
+    for (int i = 0; i < B->n; ++i) CHECK(f(i, B->probs[i]));
+    return GMG_OK;
+  }
+  const int used = std::min(S, B->n);
+  if (cudaEventRecord(B->side_ev[S], B->stream) != cudaSuccess) return GMG_ERR_CUDA;
+  for (int j = 0; j < used; ++j)
+    if (cudaStreamWaitEvent(B->side[j], B->side_ev[S], 0) != cudaSuccess) return GMG_ERR_CUDA;
+  int st = GMG_OK;
+  for (int i = 0; i < B->n && st == GMG_OK; ++i) {
+    gmg_problem* p = B->probs[i];
+    p->stream = B->side[i % S];
+    st = f(i, p);
+    p->stream = B->stream;
+  }
+  for (int j = 0; j < used; ++j)  // (also after an error: every branch has to join before the capture ends)
+    if (cudaEventRecord(B->side_ev[j], B->side[j]) != cudaSuccess ||
+        cudaStreamWaitEvent(B->stream, B->side_ev[j], 0) != cudaSuccess)
+      return GMG_ERR_CUDA;
+  return st;
+}
+
 // V-cycle of every problem from `depth` down, x_0 = 0 (the same sequence of
 // operations as gmg_vcycle on each problem; the sweeps are batched).
 int batch_vcycle(gmg_batch* B, int depth) {
   bool any_smooth = false;
-  for (int i = 0; i < B->n; ++i) {
-    gmg_problem* p = B->probs[i];
+  CHECK(each_problem(B, [&](int, gmg_problem* p) -> int {
     const int l = level_of(p, depth);
-    if (l == 0) CHECK(coarse_solve(p, p->levels[0].b, p->levels[0].u));
+    if (l == 0) return coarse_solve(p, p->levels[0].b, p->levels[0].u);
     if (l >= 1) {
       any_smooth = true;
       Level& L = p->levels[l];
-      if (cudaMemsetAsync(L.u, 0, L.n_elems * B->esize, B->stream) != cudaSuccess) return GMG_ERR_CUDA;
+      if (cudaMemsetAsync(L.u, 0, L.n_elems * B->esize, p->stream) != cudaSuccess) return GMG_ERR_CUDA;
     }
-  }
+    return GMG_OK;
+  }));
   if (!any_smooth) return GMG_OK;
   CHECK(batch_smooth(B, depth, 0, false, nullptr, nullptr));
-  for (int i = 0; i < B->n; ++i) {
-    gmg_problem* p = B->probs[i];
+  CHECK(each_problem(B, [&](int, gmg_problem* p) -> int {
     const int l = level_of(p, depth);
-    if (l < 1) continue;
+    if (l < 1) return GMG_OK;
     Level& L = p->levels[l];
     CHECK(apply_level(p, l, L.u, L.r, L.b, -op_scale(L), 1.0));
-    CHECK(restrict_to(p, l, L.r, p->levels[l - 1].b));
-  }
+    return restrict_to(p, l, L.r, p->levels[l - 1].b);
+  }));
   CHECK(batch_vcycle(B, depth + 1));
-  for (int i = 0; i < B->n; ++i) {
-    gmg_problem* p = B->probs[i];
+  CHECK(each_problem(B, [&](int, gmg_problem* p) -> int {
     const int l = level_of(p, depth);
-    if (l < 1) continue;
-    CHECK(prolongate_add(p, l - 1, p->levels[l - 1].u, p->levels[l].u));
-  }
+    return l < 1 ? GMG_OK : prolongate_add(p, l - 1, p->levels[l - 1].u, p->levels[l].u);
+  }));
   return batch_smooth(B, depth, 1, false, nullptr, nullptr);
 }
 
@@ -167,6 +198,19 @@ int run_vcycle(gmg_batch* B) {
     if (!B->cap_stream &&
         cudaStreamCreateWithFlags(&B->cap_stream, cudaStreamNonBlocking) != cudaSuccess)
       return GMG_ERR_CUDA;
+    if (B->side.empty() && B->n > 1) {
+      constexpr int kSide = 8;
+      for (int j = 0; j < std::min(kSide, B->n); ++j) {
+        cudaStream_t st = nullptr;
+        if (cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking) != cudaSuccess) return GMG_ERR_CUDA;
+        B->side.push_back(st);
+      }
+      for (size_t j = 0; j <= B->side.size(); ++j) {
+        cudaEvent_t ev = nullptr;
+        if (cudaEventCreateWithFlags(&ev, cudaEventDisableTiming) != cudaSuccess) return GMG_ERR_CUDA;
+        B->side_ev.push_back(ev);
+      }
+    }
     cudaStream_t user = B->stream;
     auto set_streams = [&](cudaStream_t st) {
       B->stream = st;
@@ -177,7 +221,9 @@ int run_vcycle(gmg_batch* B) {
       set_streams(user);
       return GMG_ERR_CUDA;
     }
+    B->capturing = B->side_ev.size() == B->side.size() + 1;
     const int st = batch_vcycle(B, 0);
+    B->capturing = false;
     cudaGraph_t g = nullptr;
     const cudaError_t e = cudaStreamEndCapture(B->cap_stream, &g);
     set_streams(user);
@@ -246,6 +292,8 @@ int gmg_batch_destroy(gmg_batch* B) {
   cudaStreamSynchronize(B->stream);
   drop_graph(B);
   if (B->cap_stream) cudaStreamDestroy(B->cap_stream);
+  for (cudaStream_t st : B->side) cudaStreamDestroy(st);
+  for (cudaEvent_t ev : B->side_ev) cudaEventDestroy(ev);
   for (gmg_problem* p : B->probs) gmg_destroy(p);
   for (void* ptr : B->owned) cudaFree(ptr);
   delete B;

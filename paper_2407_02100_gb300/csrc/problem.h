@@ -56,9 +56,9 @@ struct gmg_problem {
   void* coef_prol = nullptr;
   void* coef_rest = nullptr;
   // host copies of the transfer tables, read by the double-float transfer
-  // passes of FP64 problems (xfer_df: the tables have the expected pattern)
+  // passes of FP64 problems (xfer_ok: the tables have the expected pattern)
   std::vector<double> prol_h, rest_h;
-  bool xfer_df = false;
+  bool xfer_ok = false;
   void* tmp1 = nullptr;  // transfer temporaries
   void* tmp2 = nullptr;
   // coarsest-level fast diagonalisation

@@ -1,4 +1,4 @@
-// Level transfers of FP64 problems in double-float arithmetic.
+// Level transfers: FP64 problems in double-float arithmetic, FP32 ones in FP32.
 //
 // Prolongation is the embedding of the coarse Q_k space into the fine one,
 // applied as a tensor product of the 1D cell interpolation (one axis per
@@ -7,7 +7,10 @@
 // (88-94 % busy at 5-20 % of the DRAM bandwidth), so FP64 problems run the
 // passes in double-float arithmetic on the FP32 pipe (df_arith.cuh): node
 // values are split once per load, the intermediate arrays between passes
-// hold float pairs, and only the last pass writes doubles.
+// hold float pairs, and only the last pass writes doubles.  FP32 problems run
+// the same kernel on floats: one output per thread (the general pass of the
+// coarse solve) reads every window again per output and spent 37 % of a
+// batched V-cycle of 16 Q3 meshes (2.43 ms) on its strided loads.
 //
 // Work per thread: all outputs of one coarse cell along the pass axis, which
 // share one input window kept in registers.
@@ -43,6 +46,27 @@ struct XferArgs {
   float2 c[kXferMaxTaps];  // coefficient table as float pairs (hi, lo), rows of W
 };
 
+// the arithmetic of a pass: double-float, or FP32 (coefficients (c, unused))
+struct Df {
+  using val = dfv;
+  using acc = df_acc;
+  static __device__ __forceinline__ val zero() { return {0.f, 0.f}; }
+  static __device__ __forceinline__ acc first(float2 c, val x) { return df_acc_first(c.x, c.y, x); }
+  static __device__ __forceinline__ void add(acc& a, float2 c, val x) { df_acc_add(a, c.x, c.y, x); }
+  static __device__ __forceinline__ val value(acc a) { return df_acc_value(a); }
+};
+struct F32 {
+  using val = float;
+  using acc = float;
+  static __device__ __forceinline__ val zero() { return 0.f; }
+  static __device__ __forceinline__ acc first(float2 c, val x) { return c.x * x; }
+  static __device__ __forceinline__ void add(acc& a, float2 c, val x) { a = fmaf(c.x, x, a); }
+  static __device__ __forceinline__ val value(acc a) { return a; }
+};
+template <typename TI>
+using Arith = std::conditional_t<std::is_same<TI, float>::value, F32, Df>;
+
+__device__ __forceinline__ float load_df(const float* p) { return __ldg(p); }
 template <typename TI>
 __device__ __forceinline__ dfv load_df(const TI* p) {
   if constexpr (sizeof(TI) == 8 && !std::is_same<TI, float2>::value) return df_from_double(__ldg(p));
@@ -52,6 +76,10 @@ __device__ __forceinline__ dfv load_df(const TI* p) {
   }
 }
 
+template <typename TO, bool ACC>
+__device__ __forceinline__ void store_df(float* p, float v) {
+  *p = ACC ? *p + v : v;
+}
 template <typename TO, bool ACC>
 __device__ __forceinline__ void store_df(TO* p, dfv v) {
   if constexpr (std::is_same<TO, float2>::value) {
@@ -63,8 +91,9 @@ __device__ __forceinline__ void store_df(TO* p, dfv v) {
 }
 
 template <int K, int AX, bool RESTRICT, typename TI, typename TO, bool ACC>
-__global__ void __launch_bounds__(256) transfer_df_kernel(const TI* __restrict__ in, TO* __restrict__ out,
+__global__ void __launch_bounds__(256) transfer_kernel(const TI* __restrict__ in, TO* __restrict__ out,
                                                           const __grid_constant__ XferArgs a) {
+  using A = Arith<TI>;
   constexpr int W = RESTRICT ? 4 * K - 1 : K + 1;  // window (= table row length)
   const AxisOp& op = a.op;
   const int ng = RESTRICT ? a.n_cells : a.n_cells + 1;  // groups along AX
@@ -93,43 +122,43 @@ __global__ void __launch_bounds__(256) transfer_df_kernel(const TI* __restrict__
                           (long long)(ob + op.out_off[LB]) * op.out_stride[LB];
   const long long sa = op.in_stride[AX], so = op.out_stride[AX];
   const int lim = op.in_dim[AX];
-  dfv x[W];
+  typename A::val x[W];
   if constexpr (RESTRICT) {
     const int start = 2 * K * j - (2 * K - 1);
 #pragma unroll
     for (int w = 0; w < W; ++w) {
       const int i = start + w;
-      x[w] = (i >= 0 && i < lim) ? load_df(in + ibase + (long long)i * sa) : dfv{0.f, 0.f};
+      x[w] = (i >= 0 && i < lim) ? load_df(in + ibase + (long long)i * sa) : A::zero();
     }
     // coarse node c = K j + r sits at output index c - 1 + out_off = c along AX
     if (j > 0) {
-      df_acc acc = df_acc_first(a.c[0].x, a.c[0].y, x[0]);
+      typename A::acc acc = A::first(a.c[0], x[0]);
 #pragma unroll
-      for (int w = 1; w < W; ++w) df_acc_add(acc, a.c[w].x, a.c[w].y, x[w]);
-      store_df<TO, ACC>(out + obase + (long long)(K * j) * so, df_acc_value(acc));
+      for (int w = 1; w < W; ++w) A::add(acc, a.c[w], x[w]);
+      store_df<TO, ACC>(out + obase + (long long)(K * j) * so, A::value(acc));
     }
 #pragma unroll
     for (int r = 1; r < K; ++r) {
-      df_acc acc = df_acc_first(a.c[r * W + 2 * K].x, a.c[r * W + 2 * K].y, x[2 * K]);
+      typename A::acc acc = A::first(a.c[r * W + 2 * K], x[2 * K]);
 #pragma unroll
-      for (int w = 2 * K + 1; w < W; ++w) df_acc_add(acc, a.c[r * W + w].x, a.c[r * W + w].y, x[w]);
-      store_df<TO, ACC>(out + obase + (long long)(K * j + r) * so, df_acc_value(acc));
+      for (int w = 2 * K + 1; w < W; ++w) A::add(acc, a.c[r * W + w], x[w]);
+      store_df<TO, ACC>(out + obase + (long long)(K * j + r) * so, A::value(acc));
     }
   } else {
     const int start = K * j;
 #pragma unroll
     for (int q = 0; q < W; ++q) {
       const int i = start + q;
-      x[q] = i < lim ? load_df(in + ibase + (long long)i * sa) : dfv{0.f, 0.f};
+      x[q] = i < lim ? load_df(in + ibase + (long long)i * sa) : A::zero();
     }
     const int nr = j < a.n_cells ? 2 * K : 1;  // the extra group: the last fine node only
 #pragma unroll
     for (int r = 0; r < 2 * K; ++r) {
       if (r < nr) {
-        df_acc acc = df_acc_first(a.c[r * W].x, a.c[r * W].y, x[0]);
+        typename A::acc acc = A::first(a.c[r * W], x[0]);
 #pragma unroll
-        for (int q = 1; q < W; ++q) df_acc_add(acc, a.c[r * W + q].x, a.c[r * W + q].y, x[q]);
-        store_df<TO, ACC>(out + obase + (long long)(2 * K * j + r) * so, df_acc_value(acc));
+        for (int q = 1; q < W; ++q) A::add(acc, a.c[r * W + q], x[q]);
+        store_df<TO, ACC>(out + obase + (long long)(2 * K * j + r) * so, A::value(acc));
       }
     }
   }
@@ -142,18 +171,28 @@ int launch_one(const XferArgs& a, const void* in, void* out, cudaStream_t s) {
   if (n <= 0) return GMG_OK;
   const long long blocks = (n + 255) / 256;
   if (blocks > 0x7FFFFFFFLL) return GMG_ERR_UNSUPPORTED;
-  transfer_df_kernel<K, AX, RESTRICT, TI, TO, ACC>
+  transfer_kernel<K, AX, RESTRICT, TI, TO, ACC>
       <<<(unsigned)blocks, 256, 0, s>>>(static_cast<const TI*>(in), static_cast<TO*>(out), a);
   count_launch();
   return cudaGetLastError() == cudaSuccess ? GMG_OK : GMG_ERR_CUDA;
 }
 
-// The passes run x, y (, z): the first reads doubles and writes float pairs,
+// The passes of FP64 problems run x, y (, z): the first reads doubles and writes float pairs,
 // a middle one (3D) float pairs to float pairs, the last float pairs to
 // doubles (added to the fine vector by the prolongation).
 template <int K, bool RESTRICT>
-int launch_k(const XferArgs& a, const void* in, bool in_df, void* out, bool out_df, cudaStream_t s) {
+int launch_k(const XferArgs& a, bool f32, const void* in, bool in_df, void* out, bool out_df, cudaStream_t s) {
   const bool acc = a.op.accumulate != 0;
+  if (f32) {  // floats throughout
+    if (acc && RESTRICT) return GMG_ERR_UNSUPPORTED;
+    switch (a.op.axis) {
+      case 0: return acc ? GMG_ERR_UNSUPPORTED : launch_one<K, 0, RESTRICT, float, float, false>(a, in, out, s);
+      case 1: return acc ? launch_one<K, 1, RESTRICT, float, float, !RESTRICT>(a, in, out, s)
+                         : launch_one<K, 1, RESTRICT, float, float, false>(a, in, out, s);
+      default: return acc ? launch_one<K, 2, RESTRICT, float, float, !RESTRICT>(a, in, out, s)
+                          : launch_one<K, 2, RESTRICT, float, float, false>(a, in, out, s);
+    }
+  }
   if (a.op.axis == 0 && !in_df && out_df && !acc)
     return launch_one<K, 0, RESTRICT, double, float2, false>(a, in, out, s);
   if (a.op.axis == 1 && in_df && out_df && !acc)
@@ -165,23 +204,24 @@ int launch_k(const XferArgs& a, const void* in, bool in_df, void* out, bool out_
 }
 
 template <bool RESTRICT>
-int launch_any(int k, const XferArgs& a, const void* in, bool in_df, void* out, bool out_df, cudaStream_t s) {
+int launch_any(int k, const XferArgs& a, bool f32, const void* in, bool in_df, void* out, bool out_df,
+               cudaStream_t s) {
   switch (k) {
-    case 1: return launch_k<1, RESTRICT>(a, in, in_df, out, out_df, s);
-    case 2: return launch_k<2, RESTRICT>(a, in, in_df, out, out_df, s);
-    case 3: return launch_k<3, RESTRICT>(a, in, in_df, out, out_df, s);
-    case 4: return launch_k<4, RESTRICT>(a, in, in_df, out, out_df, s);
-    case 5: return launch_k<5, RESTRICT>(a, in, in_df, out, out_df, s);
-    case 6: return launch_k<6, RESTRICT>(a, in, in_df, out, out_df, s);
-    case 7: return launch_k<7, RESTRICT>(a, in, in_df, out, out_df, s);
-    case 8: return launch_k<8, RESTRICT>(a, in, in_df, out, out_df, s);
+    case 1: return launch_k<1, RESTRICT>(a, f32, in, in_df, out, out_df, s);
+    case 2: return launch_k<2, RESTRICT>(a, f32, in, in_df, out, out_df, s);
+    case 3: return launch_k<3, RESTRICT>(a, f32, in, in_df, out, out_df, s);
+    case 4: return launch_k<4, RESTRICT>(a, f32, in, in_df, out, out_df, s);
+    case 5: return launch_k<5, RESTRICT>(a, f32, in, in_df, out, out_df, s);
+    case 6: return launch_k<6, RESTRICT>(a, f32, in, in_df, out, out_df, s);
+    case 7: return launch_k<7, RESTRICT>(a, f32, in, in_df, out, out_df, s);
+    case 8: return launch_k<8, RESTRICT>(a, f32, in, in_df, out, out_df, s);
     default: return GMG_ERR_UNSUPPORTED;
   }
 }
 
 }  // namespace
 
-int transfer_table_df_ok(int k, bool restrict_op, const double* table) {
+int transfer_table_ok(int k, bool restrict_op, const double* table) {
   if (k < 1 || k > 8 || !table) return 0;
   if (!restrict_op) return 1;  // prolongation rows are used in full
   const int W = 4 * k - 1;
@@ -191,8 +231,8 @@ int transfer_table_df_ok(int k, bool restrict_op, const double* table) {
   return 1;
 }
 
-int launch_transfer_df(const AxisOp& op, int k, int n_cells, bool restrict_op, const double* table,
-                       const void* in, bool in_df, void* out, bool out_df, cudaStream_t s) {
+int launch_transfer(const AxisOp& op, int k, int n_cells, bool restrict_op, const double* table, bool f32,
+                    const void* in, bool in_df, void* out, bool out_df, cudaStream_t s) {
   if (k < 1 || k > 8 || n_cells < 1 || !table || !in || !out) return GMG_ERR_INVALID_ARG;
   const int W = restrict_op ? 4 * k - 1 : k + 1, rows = restrict_op ? k : 2 * k;
   if (rows * W > kXferMaxTaps) return GMG_ERR_UNSUPPORTED;
@@ -207,8 +247,8 @@ int launch_transfer_df(const AxisOp& op, int k, int n_cells, bool restrict_op, c
     const float hi = (float)table[i];
     a.c[i] = make_float2(hi, (float)(table[i] - (double)hi));
   }
-  return restrict_op ? launch_any<true>(k, a, in, in_df, out, out_df, s)
-                     : launch_any<false>(k, a, in, in_df, out, out_df, s);
+  return restrict_op ? launch_any<true>(k, a, f32, in, in_df, out, out_df, s)
+                     : launch_any<false>(k, a, f32, in, in_df, out, out_df, s);
 }
 
 }  // namespace gmg
