@@ -204,7 +204,15 @@ PatchLaunch colour_launch(const Level& L, int colour, double omega) {
 int launch_colour(gmg_problem* p, const PatchLaunch& pl, void* u, const void* b) {
   if (pl.n_patches == 0) return GMG_OK;
   if (p->esize == 8) {
-    if (pl.n_patches <= p->small_patches) {  // a coarse level: one output per thread
+    // a coarse level: one output per thread.  Where the shared-face form would
+    // run (equal up to rounding, unlike the closure form and its slabs), the
+    // coarse-level kernel wins on larger colours too: 228 -> 152 us a sweep of
+    // 512 patches a colour at k = 4, 160 -> 100 us of 1000 at k = 3, even at
+    // 1728 (150 : 161 us) and behind above
+    const int k = pl.g.k;
+    const int small = p->faces && p->shared_faces && p->small_patches > 0
+                          ? std::max(p->small_patches, k == 3 ? 1536 : k == 4 ? 640 : 0) : p->small_patches;
+    if (pl.n_patches <= small) {
       const int st = launch_patch_small<double>(pl, (double*)u, (const double*)b, (const double*)p->dinv, p->stream);
       if (st != GMG_ERR_UNSUPPORTED) return st;
     }
@@ -232,11 +240,14 @@ int smooth_colour(gmg_problem* p, int level, void* u, const void* b, int colour)
     if (pl.n_patches == 0) return GMG_OK;
     const float* corr =
         p->local_solver == GMG_LOCAL_LEARNED && ((p->corr_levels >> level) & 1u) ? p->corr[level] : nullptr;
-    if (p->esize == 8)
-      return launch_patch_var<double>(pl, (double*)u, (const double*)b, (const double*)p->coef[level],
-                                      (const double*)p->vscale[level], (const double*)p->dinv, corr, p->corr_rank, p->stream);
-    return launch_patch_var<float>(pl, (float*)u, (const float*)b, (const float*)p->coef[level],
-                                   (const float*)p->vscale[level], (const float*)p->dinv, corr, p->corr_rank, p->stream);
+    if (p->esize == 8) {
+      const double *bd = (const double*)b, *co = (const double*)p->coef[level], *vs = (const double*)p->vscale[level];
+      if (!corr) return launch_patch_var_pair<double>(pl, (double*)u, bd, co, vs, (const double*)p->dinv, p->stream);
+      return launch_patch_var<double>(pl, (double*)u, bd, co, vs, (const double*)p->dinv, corr, p->corr_rank, p->stream);
+    }
+    const float *bf = (const float*)b, *co = (const float*)p->coef[level], *vs = (const float*)p->vscale[level];
+    if (!corr) return launch_patch_var_pair<float>(pl, (float*)u, bf, co, vs, (const float*)p->dinv, p->stream);
+    return launch_patch_var<float>(pl, (float*)u, bf, co, vs, (const float*)p->dinv, corr, p->corr_rank, p->stream);
   }
   return launch_colour(p, pl, u, b);
 }

@@ -125,6 +125,9 @@ struct PairDF {  // double-float (FP64 problems)
     const ulonglong2 v = reinterpret_cast<const ulonglong2&>(c);
     return {{v.x}, {v.y}};
   }
+  // a pair of values as a coefficient (one per patch)
+  static __device__ __forceinline__ coef weight(const mem& a) { return coefficient(a); }
+  static void make_tab(tab& c, double, float h, float l) { c = make_float4(h, h, l, l); }
   static __device__ __forceinline__ acc zero() { return {{0}, {0}}; }
   static __device__ __forceinline__ acc first(coef c, val x) { return df2_acc_first(c, x); }
   static __device__ __forceinline__ void add(acc& a, coef c, val x) { df2_acc_add(a, c, x); }
@@ -154,6 +157,8 @@ struct PairF32 {  // single precision
   static __device__ __forceinline__ val load(const mem& a) { return {reinterpret_cast<const unsigned long long&>(a)}; }
   static __device__ __forceinline__ void store(mem& a, val v) { reinterpret_cast<unsigned long long&>(a) = v.v; }
   static __device__ __forceinline__ coef coefficient(const tab& c) { return load(c); }
+  static __device__ __forceinline__ coef weight(const mem& a) { return load(a); }
+  static void make_tab(tab& c, double v, float, float) { c.x = c.y = (float)v; }
   static __device__ __forceinline__ acc zero() { return {0}; }
   static __device__ __forceinline__ acc first(coef c, val x) { return f2_fma(c, x, f2{0}); }
   static __device__ __forceinline__ void add(acc& a, coef c, val x) { a = f2_fma(c, x, a); }

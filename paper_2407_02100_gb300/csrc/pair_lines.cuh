@@ -118,50 +118,43 @@ __device__ __forceinline__ void pl_backward(const PA::val (&y)[2 * K - 1], F&& e
   emit(c, PA::value(e));
 }
 
+// fills this translation unit's transform of degree k
+inline int pl_upload_transform(int k, const double* That) {
+  const int M = 2 * k - 1;
+  std::vector<PA::tab> t(M * M);
+  for (int i = 0; i < M * M; ++i) {
+    float h, l;
+    split_pair(That[i], h, l);
+    PA::make_tab(t[i], That[i], h, l);
+  }
+  const size_t e = sizeof(PA::tab);
+  return cudaMemcpyToSymbol(p_T, t.data(), t.size() * e, pl_off_t(k) * e) == cudaSuccess ? GMG_OK : GMG_ERR_CUDA;
+}
+
 // fills this translation unit's tables of degree k
 inline int pl_upload(int k, const double* Mp, const double* Kp, const double* That) {
   const int C = 2 * k + 1, M = 2 * k - 1;
-  std::vector<PA::tab> m(M * C), s(M * C), t(M * M), end(2 * M);
-  if constexpr (sizeof(PA::tab) == 16) {
-    std::vector<float> kh, kl;
-    split_zero_sum_rows(Kp, M, C, kh, kl);
-    auto pair = [](PA::tab& c, float h, float l) { reinterpret_cast<float4&>(c) = make_float4(h, h, l, l); };
-    float h, l;
-    for (int i = 0; i < M * C; ++i) {
-      split_pair(Mp[i], h, l);
-      pair(m[i], h, l);
-      pair(s[i], kh[i], kl[i]);
-    }
-    for (int i = 0; i < M * M; ++i) {
-      split_pair(That[i], h, l);
-      pair(t[i], h, l);
-    }
-    for (int i = 0; i < M; ++i) {
-      const int o = i * C + (i < k ? 0 : C - 1);
-      split_pair(Mp[o], h, l);
-      pair(end[2 * i], -h, -l);
-      pair(end[2 * i + 1], -kh[o], -kl[o]);
-    }
-  } else {
-    auto pair = [](PA::tab& c, double v) { c.x = c.y = (float)v; };
-    for (int i = 0; i < M * C; ++i) {
-      pair(m[i], Mp[i]);
-      pair(s[i], Kp[i]);
-    }
-    for (int i = 0; i < M * M; ++i) pair(t[i], That[i]);
-    for (int i = 0; i < M; ++i) {
-      const int o = i * C + (i < k ? 0 : C - 1);
-      pair(end[2 * i], -Mp[o]);
-      pair(end[2 * i + 1], -Kp[o]);
-    }
+  std::vector<PA::tab> m(M * C), s(M * C), end(2 * M);
+  std::vector<float> kh, kl;
+  split_zero_sum_rows(Kp, M, C, kh, kl);
+  float h, l;
+  for (int i = 0; i < M * C; ++i) {
+    split_pair(Mp[i], h, l);
+    PA::make_tab(m[i], Mp[i], h, l);
+    PA::make_tab(s[i], Kp[i], kh[i], kl[i]);
+  }
+  for (int i = 0; i < M; ++i) {
+    const int o = i * C + (i < k ? 0 : C - 1);
+    split_pair(Mp[o], h, l);
+    PA::make_tab(end[2 * i], -Mp[o], -h, -l);
+    PA::make_tab(end[2 * i + 1], -Kp[o], -kh[o], -kl[o]);
   }
   const size_t e = sizeof(PA::tab);
   if (cudaMemcpyToSymbol(p_M, m.data(), m.size() * e, pl_off_patch(k) * e) != cudaSuccess ||
       cudaMemcpyToSymbol(p_K, s.data(), s.size() * e, pl_off_patch(k) * e) != cudaSuccess ||
-      cudaMemcpyToSymbol(p_E, end.data(), end.size() * e, pl_off_end(k) * e) != cudaSuccess ||
-      cudaMemcpyToSymbol(p_T, t.data(), t.size() * e, pl_off_t(k) * e) != cudaSuccess)
+      cudaMemcpyToSymbol(p_E, end.data(), end.size() * e, pl_off_end(k) * e) != cudaSuccess)
     return GMG_ERR_CUDA;
-  return GMG_OK;
+  return pl_upload_transform(k, That);
 }
 
 }  // namespace

@@ -6,7 +6,8 @@
 //  * apply_var_kernel: y += alpha * sum_c a_c A_c x_c, cell by cell by sum
 //    factorisation (App. A.1), accumulated with atomics (a node is shared
 //    by up to 2^d cells); the caller initialises y.
-//  * patch_var_kernel: one colour of the patch smoother (Algorithm 4) whose
+//  * patch_var_kernel: one colour of the patch smoother (Algorithm 4) on
+//    levels with a learned correction (the others: pair_var.cuh); the
 //    local residual is evaluated cell by cell with the cell coefficients
 //    (Sec. 3.1, eq. "main:4"), and whose local solver is the fast
 //    diagonalisation of the constant-coefficient patch scaled by the

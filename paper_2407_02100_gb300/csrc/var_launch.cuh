@@ -125,7 +125,8 @@ int upload_var_tables<GMG_T>(int k, const double* Mc, const double* Kc, const do
     if (e == cudaSuccess) e = cudaMemcpyToSymbol(c_Thi, h.data(), tb, to);
     if (e == cudaSuccess) e = cudaMemcpyToSymbol(c_Tlo, l.data(), tb, to);
   }
-  return e == cudaSuccess ? GMG_OK : GMG_ERR_CUDA;
+  if (e != cudaSuccess) return GMG_ERR_CUDA;
+  return upload_var_pair_tables<GMG_T>(k, Mc, Kc, That);
 }
 
 template <>
