@@ -126,9 +126,6 @@ int launch_patch_small(const PatchLaunch& pl, T* u, const T* b, const T* dinv, c
 template <typename T>
 int launch_patch_table(int dim, int k, const PatchLaunch* pls, T* const* us, const T* const* bs,
                        int n, const T* dinv, int ppc, cudaStream_t s);
-// the FP64 3D closure form at degrees 7 and 8, one patch per thread (patch_f64.cu)
-int launch_line_table(int k, const PatchLaunch* pls, double* const* us, const double* const* bs, int n,
-                      const double* dinv, cudaStream_t s);
 // Tensor-core sweep (patch_tc.cu): 3D, FP32 data, degrees 4..7, combined
 // mode only (GMG_ERR_UNSUPPORTED otherwise).
 bool tc_supported(int dim, int k);

@@ -3,12 +3,12 @@
 // problems, patch lists (slabs, Algorithm 5) and the solve-only mode of
 // Algorithm 3, in 2D and 3D.  With one patch per thread the FP32 kernel issued
 // two instructions beside each multiply-add; per sweep, before -> now (us):
-// FP32 Q4 64^3 934 -> 582, FP64 2D Q3 1024^2 967 -> 693, FP64 closure form Q4
-// 64^3 4930 -> 4220.
+// FP32 Q4 64^3 934 -> 599, FP64 2D Q3 1024^2 967 -> 544, FP64 closure form Q4
+// 64^3 4930 -> 3180.
 //
 // Patch local_update (Sec. 3.1; Algorithm 4 runs it for every patch of one
 // colour per launch):
-//   gather    closure bar u_j ((2k+1)^d nodes) into shared memory
+//   gather    closure bar u_j ((2k+1)^d nodes)
 //   evaluate  r = h^{2-d} b_j - [A_ref bar u_j]_interior by sum factorisation
 //             over the patch: the patch operator is a sum of tensor products
 //             of the two-cell 1D matrices M_p, K_p (interior rows x closure
@@ -20,15 +20,12 @@
 #include <algorithm>
 #include <type_traits>
 
-#include <cuda.h>
 #include <cuda_runtime.h>
 
 #include "../../include/gmg.h"
-#include "async.cuh"
 #include "kernels.h"
 #include "pair_lines.cuh"
 #include "patch_dispatch.h"
-#include "tma_host.h"
 
 namespace gmg {
 namespace {
@@ -40,39 +37,20 @@ constexpr bool DF = sizeof(T) == 8;
 
 __host__ __device__ constexpr int cmax(int a, int b) { return a > b ? a : b; }
 
-// Shared memory: per patch IN, its closure of u and its interior
-// of b in rows of XU / XB elements of T ([z][y][x]; with the TMA gather a row
-// is the box width: C (resp. M + 1) plus the alignment shift, rounded up to
-// 16 bytes, and each box starts on 128 bytes); per pair W, entries of E: the
-// two fields of the first contraction, in rows of R entries.  Every later
-// stage works in place: a thread reads the whole line it writes.
-template <int DIM, int K, bool TMA>
+// Shared memory per pair, entries of E: the two fields of the first
+// contraction, in rows of R entries.  Every later stage works in place: a
+// thread reads the whole line it writes.  u and b go from global memory
+// straight to registers (lanes along x): without room for the closures more
+// than twice as many CTAs fit on an SM, which overlap one another's loads and
+// barriers (FP32 Q4 64^3: 9 KB a pair against 22 KB with TMA boxes).
+template <int DIM, int K>
 struct ClosureSmem {
   static constexpr int C = 2 * K + 1, M = 2 * K - 1;
-  static constexpr int A = 16 / (int)sizeof(T);  // elements per 16 bytes
-  static constexpr int XU = TMA ? (C + A - 1 + A - 1) / A * A : C;
-  static constexpr int XB = TMA ? XU : M;
-  static constexpr int R128 = 128 / (int)sizeof(T);
-  static constexpr int rnd(int n) { return (n + R128 - 1) / R128 * R128; }
-  static constexpr int NCLO = rnd(DIM == 3 ? C * C * XU : C * XU);
-  static constexpr int NBIN = rnd(DIM == 3 ? M * M * XB : M * XB);
   static constexpr int NINT = DIM == 3 ? M * M * M : M * M;
-  static constexpr int IN = NCLO + NBIN;
   static constexpr int R = DIM == 3 ? C : M;             // row of W (x)
   static constexpr int F = DIM == 3 ? C * M * R : C * R;  // one field: [z][y][x], z in C, y in M (2D: [y][x])
-  static constexpr int bytes(int pp) { return pp * 2 * (IN * (int)sizeof(T) + F * (int)sizeof(E)) + 128; }
-  // TMA box bytes of the closure of u and of the interior rows of b
-  static constexpr int BOX_U = (DIM == 3 ? C * C * XU : C * XU) * (int)sizeof(T);
-  static constexpr int BOX_B = (DIM == 3 ? M * M * XB : M * XB) * (int)sizeof(T);
+  static constexpr int bytes(int pp) { return pp * 2 * F * (int)sizeof(E); }
 };
-
-// Tensor maps of the u and b vectors of each table entry (TMA gather).
-template <int ME>
-struct ClosureMaps {
-  CUtensorMap u[ME], b[ME];
-};
-template <>
-struct ClosureMaps<0> {};
 
 // One contraction of a line of C closure values: row(i, M x, K x) per interior
 // row i, with the line's values loaded by get(closure index) one cell at a
@@ -149,13 +127,9 @@ __device__ __forceinline__ void closure_line_residual(G&& get1, H&& get2, PA::ac
 
 // One colour of the sweep.  A CTA takes one group of 2 PP consecutive patches
 // of a table entry; a thread carries the same line of patches 2q and 2q + 1.
-// Small CTAs, several to an SM, overlap one another's gathers and barriers,
-// and the hardware hands them out as SMs become free (persistent CTAs with a
-// fixed share: 0.63 against 0.60 ms per FP32 Q4 64^3 sweep, a second input
-// buffer 0.66).  The gather is one TMA box per patch and vector (ME > 0:
-// tiled cp.async.bulk.tensor loads completing on an mbarrier; the box starts
-// at the closure origin rounded down to 16 bytes and the shift is kept per
-// patch) or one cp.async per element (ME = 0).  The last contraction runs along the slowest
+// Small CTAs, several to an SM, overlap one another's loads and barriers, and
+// the hardware hands them out as SMs become free (persistent CTAs with a fixed
+// share: 0.63 against 0.60 ms per FP32 Q4 64^3 sweep).  The last contraction runs along the slowest
 // axis, as does the scatter: consecutive lanes then hold consecutive x, and
 // loads and stores touch whole sectors.  Stages, 3D (2D: without z; y takes
 // the part of z):
@@ -168,30 +142,20 @@ __device__ __forceinline__ void closure_line_residual(G&& get1, H&& get2, PA::ac
 // zero interior and the scatter writes omega d + (1 - omega) u_j.  (FP32 keeps
 // the correction form: recomputing the interior would cost a factor
 // cond(A_j) in single precision.)
-// Same-colour patches never write each other's closure, so the buffered
-// closure values are the values the gather (eq. "gather") reads.
-template <int DIM, int K, int NT, int PP, int CTAS, int ME>
+// Same-colour patches never write each other's closure, so the order in which
+// they run does not matter.
+template <int DIM, int K, int NT, int PP, int CTAS>
 __global__ void __launch_bounds__(NT, CTAS) pair_closure_kernel(const __grid_constant__ PatchTable tab,
-                                                                const T* __restrict__ dinv,
-                                                                const __grid_constant__ ClosureMaps<ME> maps,
-                                                                int* __restrict__ err) {
-  constexpr bool TMA = ME > 0;
+                                                                const T* __restrict__ dinv) {
   constexpr bool EXACT = DF && DIM == 3;
-  using Z = ClosureSmem<DIM, K, TMA>;
-  constexpr int C = Z::C, M = Z::M, XU = Z::XU, XB = Z::XB, R = Z::R, F = Z::F, NP = 2 * PP;
+  using Z = ClosureSmem<DIM, K>;
+  constexpr int C = Z::C, M = Z::M, R = Z::R, F = Z::F, NP = 2 * PP;
   constexpr int LINES = DIM == 3 ? M * M : M;  // interior lines per axis
-  static_assert(NP <= NT, "one lane issues the copies of one patch");
+  static_assert(NP <= NT, "one thread sets up one patch");
   extern __shared__ __align__(128) unsigned char smem_raw[];
-  T* const IN = reinterpret_cast<T*>(smem_raw + ((128 - (async::smem_u32(smem_raw) & 127)) & 127));  // [NP][IN]
-  E* const W = reinterpret_cast<E*>(IN + NP * Z::IN);  // [PP][2][F]
+  E* const W = reinterpret_cast<E*>(smem_raw);  // [PP][2][F]
   __shared__ long long s_origin[NP];
-  __shared__ int s_shift[NP];  // of the closure inside its TMA box
-  __shared__ __align__(8) uint64_t s_bar;
   const int mode = tab.mode, grp = blockIdx.x;
-  // element offsets inside a patch's input: closure of u, interior of b
-  auto uo = [](int x, int y, int z) { return DIM == 3 ? (z * C + y) * XU + x : y * XU + x; };
-  auto bo = [](int x, int y, int z) { return DIM == 3 ? (z * M + y) * XB + x : y * XB + x; };
-
   int entry = 0, hi = tab.n - 1;  // last table entry with group_begin <= grp
   while (entry < hi) {
     const int mid = (entry + hi + 1) >> 1;
@@ -200,71 +164,37 @@ __global__ void __launch_bounds__(NT, CTAS) pair_closure_kernel(const __grid_con
   }
   const PatchEntry& e = tab.e[entry];
   const int g = grp - e.group_begin, nv = min(NP, e.n_patches - g * NP), npair = (nv + 1) / 2;
-  T* __restrict__ const u = static_cast<T*>(e.u);
-  const long long py = e.py, pz = e.pz;
+  T* const u = static_cast<T*>(e.u);
+  const T* __restrict__ const b = static_cast<const T*>(e.b);
+  const long long py = e.py, pz = e.pz, ps = DIM == 3 ? pz : py;  // ps: the slowest axis
   const float sb = (float)e.sb;  // h^{2-d}: n in 3D, 1 in 2D, exact in float
-  if (TMA) {
-    if (threadIdx.x == 0) {
-      async::mbar_init(&s_bar, 1);
-      async::mbar_arrive_expect_tx(&s_bar, (uint32_t)(nv * ((mode == 0 ? Z::BOX_U : 0) + Z::BOX_B)));
-    }
-    __syncthreads();
-  }
-  {
-    // patch origins and copies: the patches are spread over the warps, as a
-    // warp issues its lanes' copies one after the other
-    const int q = threadIdx.x / 32 + (threadIdx.x % 32) * (NT / 32);
-    if (q < nv) {
-      int pid = g * NP + q;
-      if (e.plist) pid = e.plist[pid];
-      const int i0 = pid % e.count[0], rest = pid / e.count[0];
-      const int i1 = rest % e.count[1], i2 = DIM == 3 ? rest / e.count[1] : 0;
-      const int o0 = (e.first[0] + 2 * i0 - 1) * K, o1 = (e.first[1] + 2 * i1 - 1) * K;
-      const int o2 = DIM == 3 ? (e.first[2] + 2 * i2 - 1) * K : 0;
-      s_origin[q] = o0 + py * o1 + pz * o2;
-      s_shift[q] = TMA ? o0 % Z::A : 0;
-      if constexpr (TMA) {
-        T* const dst = IN + q * Z::IN;
-        const int xa = o0 - o0 % Z::A;
-        if (DIM == 3) {
-          if (mode == 0) async::tma_load_3d(dst, &maps.u[entry], xa, o1, o2, &s_bar);
-          async::tma_load_3d(dst + Z::NCLO, &maps.b[entry], xa, o1 + 1, o2 + 1, &s_bar);
-        } else {
-          if (mode == 0) async::tma_load_2d(dst, &maps.u[entry], xa, o1, &s_bar);
-          async::tma_load_2d(dst + Z::NCLO, &maps.b[entry], xa, o1 + 1, &s_bar);
-        }
-      }
-    }
+  if ((int)threadIdx.x < NP) {  // (a lone last patch is carried twice and stored once)
+    int pid = g * NP + min((int)threadIdx.x, nv - 1);
+    if (e.plist) pid = e.plist[pid];
+    const int i0 = pid % e.count[0], rest = pid / e.count[0];
+    const int i1 = rest % e.count[1], i2 = DIM == 3 ? rest / e.count[1] : 0;
+    s_origin[threadIdx.x] = (e.first[0] + 2 * i0 - 1) * K + py * ((e.first[1] + 2 * i1 - 1) * K) +
+                            (DIM == 3 ? pz * ((e.first[2] + 2 * i2 - 1) * K) : 0);
   }
   __syncthreads();
-  bool wait_ok = true;  // an expired wait is recorded and the kernel carries on
-  if constexpr (TMA) {
-    wait_ok = async::mbar_wait(&s_bar, 0);
-  } else {
-    const T* __restrict__ b = static_cast<const T*>(e.b);
-    constexpr int NC = DIM == 3 ? C * C * C : C * C;
-    auto copy = [](T* d, const T* s) {
-      asm volatile("cp.async.ca.shared.global [%0], [%1], %2;\n" ::"r"(async::smem_u32(d)), "l"(s), "n"(sizeof(T)) : "memory");
-    };
-    // the solve-only mode needs no closure: only the residual's interior
-    for (int t = threadIdx.x; t < (mode == 0 ? nv * NC : 0); t += NT) {
-      const int p = t / NC, l = t % NC, x = l % C, row = l / C;
-      copy(IN + p * Z::IN + l, u + s_origin[p] + x + py * (row % C) + (DIM == 3 ? pz * (row / C) : 0));
-    }
-    for (int t = threadIdx.x; t < nv * Z::NINT; t += NT) {
-      const int p = t / Z::NINT, l = t % Z::NINT, x = l % M, row = l / M;
-      copy(IN + p * Z::IN + Z::NCLO + l, b + s_origin[p] + 1 + x + py * (row % M + 1) + (DIM == 3 ? pz * (row / M + 1) : 0));
-    }
-    async::copy_wait_all();
-    __syncthreads();
-  }
-  // both patches' inputs, shifted to the closure origin (a lone last patch
-  // has whatever the buffer holds beside it; nothing of that is stored)
-  auto input = [&](int q, int second) -> const T* {
-    const int p = 2 * q + second;
-    return IN + p * Z::IN + (p < nv ? s_shift[p] : 0);
-  };
 
+  // The rows of b are on their way from the start where the registers allow it
+  // (FP64 Q3 64^3 1107 -> 1029 us, Q4 3273 -> 3172; Q5 48^3 5895 -> 6271; Q2
+  // 96^3 fits one CTA per SM less, 821 -> 854).
+  constexpr bool EARLY = K <= 4 && (DIM == 2 || K >= 3) && PP * LINES <= NT;
+  T eb[EARLY ? 2 * M : 1];
+  auto rhs = [&](int t, int p) -> const T* {
+    const int ln = t % LINES;
+    return b + s_origin[2 * (t / LINES) + p] + 1 + ln % M + (DIM == 3 ? py * (1 + ln / M) : 0) + ps;
+  };
+  if constexpr (EARLY) {
+    const int t = (int)threadIdx.x < npair * LINES ? threadIdx.x : 0;
+#pragma unroll
+    for (int l = 0; l < M; ++l) {
+      eb[l] = __ldg(rhs(t, 0) + ps * l);
+      eb[M + l] = __ldg(rhs(t, 1) + ps * l);
+    }
+  }
   if (mode == 0) {
     if (DIM == 3) {
       // ---- y: P = M_y u, Q = K_y u on lines (x, z), from -u ----
@@ -292,10 +222,9 @@ __global__ void __launch_bounds__(NT, CTAS) pair_closure_kernel(const __grid_con
           x = t % (C * C) % C;
           z = t % (C * C) / C;
         }
-        const T* const a = input(q, 0) + uo(x, 0, z);
-        const T* const b = input(q, 1) + uo(x, 0, z);
+        const T *const ua = u + s_origin[2 * q] + x + pz * z, *const ub = u + s_origin[2 * q + 1] + x + pz * z;
         E* const P = W + q * 2 * F + z * M * R + x;
-        auto get = [&](int y) -> V { return PA::pack_neg(a[y * XU], b[y * XU]); };
+        auto get = [&](int y) -> V { return PA::pack_neg(ua[py * y], ub[py * y]); };
         auto put = [&](int j, V m, V k) {
           PA::store(P[j * R], m);
           PA::store(P[F + j * R], k);
@@ -343,10 +272,9 @@ __global__ void __launch_bounds__(NT, CTAS) pair_closure_kernel(const __grid_con
       // ---- x: P = M_x u, Q = K_x u on rows y, from -u ----
       for (int t = threadIdx.x; t < npair * C; t += NT) {
         const int q = t / C, y = t % C;
-        const T* const a = input(q, 0) + uo(0, y, 0);
-        const T* const b = input(q, 1) + uo(0, y, 0);
+        const T *const ua = u + s_origin[2 * q] + py * y, *const ub = u + s_origin[2 * q + 1] + py * y;
         E* const P = W + q * 2 * F + y * R;
-        closure_line<K>([&](int x) -> V { return PA::pack_neg(a[x], b[x]); },
+        closure_line<K>([&](int x) -> V { return PA::pack_neg(ua[x], ub[x]); },
                         [&](int i, V m, V k) {
                           PA::store(P[i], m);
                           PA::store(P[F + i], k);
@@ -362,14 +290,12 @@ __global__ void __launch_bounds__(NT, CTAS) pair_closure_kernel(const __grid_con
   auto line = [&](int q, int ln) -> E* { return W + q * 2 * F + (DIM == 3 ? ln / M * R + ln % M : ln); };
   for (int t = threadIdx.x; t < npair * LINES; t += NT) {
     const int q = t / LINES, ln = t % LINES;  // 3D: x + M y; 2D: x
-    const int bofs = Z::NCLO + (TMA ? 1 : 0) + (DIM == 3 ? bo(ln % M, ln / M, 0) : ln);
-    const T* const ba = input(q, 0) + bofs;
-    const T* const bb = input(q, 1) + bofs;
+    const T *const ba = rhs(t, 0), *const bb = rhs(t, 1);
     PA::acc acc[M];
 #pragma unroll
     for (int l = 0; l < M; ++l) {
-      const int o = (DIM == 3 ? M * XB : XB) * l;
-      acc[l] = PA::scaled(sb, PA::pack(ba[o], bb[o]));
+      if constexpr (EARLY) acc[l] = PA::scaled(sb, PA::pack(eb[l], eb[M + l]));
+      else acc[l] = PA::scaled(sb, PA::pack(__ldg(ba + ps * l), __ldg(bb + ps * l)));
     }
     if (mode == 0) {
       const E* const A = line(q, ln);
@@ -414,7 +340,7 @@ __global__ void __launch_bounds__(NT, CTAS) pair_closure_kernel(const __grid_con
   if (DIM == 3) line_y(std::false_type());
   // ---- backward along the slowest axis and scatter (eq. "scatter") ----
   const T om = (T)tab.omega;
-  const long long ps = DIM == 3 ? pz : py;
+  const bool fresh = EXACT && mode == 0 && om == T(1);  // nothing of the old value is left
   for (int t = threadIdx.x; t < npair * LINES; t += NT) {
     const int q = t / LINES, ln = t % LINES;
     const E* const w = line(q, ln);
@@ -422,22 +348,27 @@ __global__ void __launch_bounds__(NT, CTAS) pair_closure_kernel(const __grid_con
 #pragma unroll
     for (int l = 0; l < M; ++l) v[l] = PA::load(w[l * SL]);
     const bool two = 2 * q + 1 < nv;
-    const int x = 1 + ln % M, y = DIM == 3 ? 1 + ln / M : 0;
-    const long long ofs = x + (DIM == 3 ? py * y : 0) + ps;
-    const int uofs = DIM == 3 ? uo(x, y, 1) : uo(x, 1, 0);
-    constexpr int US = DIM == 3 ? C * XU : XU;  // the slow stride of the closure
-    T* const ga = u + s_origin[2 * q] + ofs;
-    T* const gb = two ? u + s_origin[2 * q + 1] + ofs : ga;
-    const T *const ia = input(q, 0) + uofs, *const ib = input(q, 1) + uofs;
-    pl_backward<K>(v, [&](int l, V d) {
-      auto one = [&](T* g, const T* i, T dv) {
-        *g = EXACT && mode == 0 ? fma(om, dv, (T(1) - om) * *i) : fma(om, dv, mode == 0 ? *i : *g);
-      };
-      one(ga + ps * l, ia + US * l, PA::x(d));
-      if (two) one(gb + ps * l, ib + US * l, PA::y(d));
-    });
+    const long long ofs = 1 + ln % M + (DIM == 3 ? py * (1 + ln / M) : 0) + ps;
+    T *const ga = u + s_origin[2 * q] + ofs, *const gb = u + s_origin[2 * q + 1] + ofs;
+    if (EXACT && fresh) {
+      pl_backward<K>(v, [&](int l, V d) {
+        ga[ps * l] = PA::x(d);
+        if (two) gb[ps * l] = PA::y(d);
+      });
+    } else {
+      T oa[M], ob[M];
+#pragma unroll
+      for (int l = 0; l < M; ++l) {
+        oa[l] = ga[ps * l];
+        ob[l] = gb[ps * l];
+      }
+      const T keep = EXACT && mode == 0 ? T(1) - om : T(1);
+      pl_backward<K>(v, [&](int l, V d) {
+        ga[ps * l] = fma(om, PA::x(d), EXACT ? keep * oa[l] : oa[l]);
+        if (two) gb[ps * l] = fma(om, PA::y(d), EXACT ? keep * ob[l] : ob[l]);
+      });
+    }
   }
-  if (!wait_ok) atomicExch(err, GMG_ERR_TIMEOUT);
 }
 
 // ---- host side ----
@@ -445,30 +376,25 @@ __global__ void __launch_bounds__(NT, CTAS) pair_closure_kernel(const __grid_con
 // Patch pairs and threads per CTA, and the CTAs per SM that the registers are
 // limited for.  A pair has LINES lines in most stages, and a CTA as many pairs
 // as fill its threads with them.  Measured per sweep (us), the shape taken
-// first: FP32 Q3 64^3 1 pair in 32 threads 279, 2 in 64 296, 5 in 128 361; Q4
-// 64^3 1 in 64 582, 2 in 128 630, 4 in 224 787; Q6 40^3 with registers for 3
-// CTAs 594, without 770; FP64 Q3 64^3 5 in 128 1536, 1 in 32 1826; FP64 2D Q3
-// 1024^2 25 in 128 697, 12 in 64 756; FP32 2D Q3 6 in 32 201, 25 in 128 238.
+// first: FP32 Q4 64^3 1 pair in 64 threads 599, 2 in 128 630, 5 in 256 644;
+// Q6 40^3 with registers for 4 CTAs 552, for 1 772; FP64 Q3 64^3 10 in 256
+// with registers for 2 CTAs 1030, 5 in 128 for 4 1265, 1 in 32 2251; FP64 2D
+// Q3 1024^2 25 in 128 for 5 CTAs 544, for 1 938, 12 in 64 for 8 710.
 template <int DIM, int K>
 struct ClosureCfg {
   static constexpr int M = 2 * K - 1, LINES = DIM == 3 ? M * M : M;
-  static constexpr int NT = DIM == 2 ? (!DF ? 32 : K == 2 ? 64 : 128)
-                          : K <= 3 ? (DF ? 128 : 32) : K >= 7 ? 256 : (LINES + 31) / 32 * 32;
-  static constexpr int PP = cmax(1, std::min(NT / LINES, 3 * NT / 8));
-  static constexpr int CTAS = DIM == 2 ? (DF && K == 3 ? 4 : 1) : !DF && K == 5 ? 6 : !DF && K == 6 ? 3 : 1;
+  static constexpr int NT = DIM == 2 || K <= 2 ? 128 : DF ? 256 : K == 3 ? 128 : K == 8 ? 256 : (LINES + 31) / 32 * 32;
+  static constexpr int PP = cmax(1, std::min(NT / LINES, 48));
+  static constexpr int CTAS = DIM == 2 ? (!DF || K <= 2 ? 1 : K == 3 ? 5 : 4)
+                            : DF ? (K == 1 ? 1 : K == 2 ? 5 : K == 6 || K == 8 ? 1 : 2)
+                                 : (K == 4 ? 14 : K == 6 ? 4 : K >= 7 ? 2 : 1);
 };
-// a pair of the largest FP64 patches does not fit in the shared memory of a CTA
-template <int DIM, int K>
-constexpr bool closure_pairs() {
-  return ClosureSmem<DIM, K, true>::bytes(1) <= 227 * 1024;
-}
 
-template <int DIM, int K, int PP, int NT, int CTAS, int ME>
+template <int DIM, int K, int PP, int NT, int CTAS>
 int closure_launch(PatchTable& tab, const T* dinv, cudaStream_t s) {
-  using Z = ClosureSmem<DIM, K, (ME > 0)>;
-  constexpr int SMEM = Z::bytes(PP);
+  constexpr int SMEM = ClosureSmem<DIM, K>::bytes(PP);
   static_assert(SMEM <= 227 * 1024, "sweep kernel shared memory exceeds the per-CTA limit");
-  auto kern = pair_closure_kernel<DIM, K, NT, PP, CTAS, ME>;
+  auto kern = pair_closure_kernel<DIM, K, NT, PP, CTAS>;
   static PerDevice<bool> ready_dev;  // attribute set once per device
   bool* const ready = ready_dev.get();
   if (!ready) return GMG_ERR_CUDA;
@@ -484,36 +410,9 @@ int closure_launch(PatchTable& tab, const T* dinv, cudaStream_t s) {
   }
   tab.total_groups = groups;
   if (groups <= 0) return GMG_OK;
-  ClosureMaps<ME> maps;
-  if constexpr (ME > 0) {
-    for (int i = 0; i < tab.n; ++i) {
-      const PatchEntry& e = tab.e[i];
-      if (!tma_encode(&maps.u[i], e.u, (int)sizeof(T), DIM, e.N, e.py, e.pz, Z::XU, Z::C) ||
-          !tma_encode(&maps.b[i], e.b, (int)sizeof(T), DIM, e.N, e.py, e.pz, Z::XB, Z::M))
-        return GMG_ERR_CUDA;
-    }
-  }
-  int* const flag = device_wait_flag();
-  if (!flag) return GMG_ERR_CUDA;
-  kern<<<groups, NT, SMEM, s>>>(tab, dinv, maps, flag);
+  kern<<<groups, NT, SMEM, s>>>(tab, dinv);
   count_launch();
   return cudaGetLastError() == cudaSuccess ? GMG_OK : GMG_ERR_CUDA;
-}
-
-// the TMA gather when every vector of the table allows the boxes, else one
-// cp.async per element
-template <int DIM, int K, int PP, int NT, int CTAS>
-int closure_gather(PatchTable& tab, const T* dinv, cudaStream_t s) {
-  bool tma = true;
-  for (int i = 0; i < tab.n; ++i) {
-    const PatchEntry& e = tab.e[i];
-    if (e.N < 2 || !tma_vector_ok(e.u, (int)sizeof(T), DIM, e.py, e.pz) ||
-        !tma_vector_ok(e.b, (int)sizeof(T), DIM, e.py, e.pz))
-      tma = false;
-  }
-  if (!tma) return closure_launch<DIM, K, PP, NT, CTAS, 0>(tab, dinv, s);
-  if (tab.n == 1) return closure_launch<DIM, K, PP, NT, CTAS, 1>(tab, dinv, s);
-  return closure_launch<DIM, K, PP, NT, CTAS, kMaxTable>(tab, dinv, s);
 }
 
 template <int DIM, int K>
@@ -521,11 +420,11 @@ int closure_table(PatchTable& tab, const T* dinv, int ppc, cudaStream_t s) {
   using Cfg = ClosureCfg<DIM, K>;
   // tuned patches-per-CTA variants of the batched sweep (patches come in pairs)
   if constexpr (DIM == 3 && !DF && K <= 4) {
-    if (ppc == 1) return closure_gather<DIM, K, 1, 32, 1>(tab, dinv, s);
-    if (ppc == 2) return closure_gather<DIM, K, 1, 64, 1>(tab, dinv, s);
-    if (ppc == 4) return closure_gather<DIM, K, 2, 128, 1>(tab, dinv, s);
+    if (ppc == 1) return closure_launch<DIM, K, 1, 32, 1>(tab, dinv, s);
+    if (ppc == 2) return closure_launch<DIM, K, 1, 64, 1>(tab, dinv, s);
+    if (ppc == 4) return closure_launch<DIM, K, 2, 128, 1>(tab, dinv, s);
   }
-  return closure_gather<DIM, K, Cfg::PP, Cfg::NT, Cfg::CTAS>(tab, dinv, s);
+  return closure_launch<DIM, K, Cfg::PP, Cfg::NT, Cfg::CTAS>(tab, dinv, s);
 }
 
 }  // namespace

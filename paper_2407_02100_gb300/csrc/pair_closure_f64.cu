@@ -8,24 +8,18 @@ namespace {
 template <int DIM, int K>
 int table_launches(const PatchLaunch* pls, T* const* us, const T* const* bs, int n, const T* dinv, int ppc,
                    cudaStream_t s) {
-  // a pair of the largest patches does not fit in shared memory: one patch
-  // per thread for those
-  if constexpr (!closure_pairs<DIM, K>()) {
-    return launch_line_table(K, pls, us, bs, n, dinv, s);
-  } else {
-    for (int i0 = 0; i0 < n; i0 += kMaxTable) {
-      PatchTable tab;
-      tab.n = 0;
-      tab.mode = pls[i0].mode;
-      tab.omega = pls[i0].omega;
-      for (int i = i0; i < std::min(n, i0 + kMaxTable); ++i)
-        if (pls[i].n_patches > 0) fill_entry(tab.e[tab.n++], pls[i], us[i], bs[i]);
-      if (tab.n == 0) continue;
-      const int st = closure_table<DIM, K>(tab, dinv, ppc, s);
-      if (st != GMG_OK) return st;
-    }
-    return GMG_OK;
+  for (int i0 = 0; i0 < n; i0 += kMaxTable) {
+    PatchTable tab;
+    tab.n = 0;
+    tab.mode = pls[i0].mode;
+    tab.omega = pls[i0].omega;
+    for (int i = i0; i < std::min(n, i0 + kMaxTable); ++i)
+      if (pls[i].n_patches > 0) fill_entry(tab.e[tab.n++], pls[i], us[i], bs[i]);
+    if (tab.n == 0) continue;
+    const int st = closure_table<DIM, K>(tab, dinv, ppc, s);
+    if (st != GMG_OK) return st;
   }
+  return GMG_OK;
 }
 
 }  // namespace

@@ -1,5 +1,5 @@
 // Patch sweep on the 5th-generation tensor cores (3D, FP32 data, degree
-// 4..7): the same local_update as patch_colour_kernel (Sec. 3.1; gather,
+// 4..7): the same local_update as pair_closure.cuh (Sec. 3.1; gather,
 // local residual by sum factorisation over the patch, fast-diagonalisation
 // solve of App. A.3, scatter), with every 1D contraction executed as a TF32
 // tcgen05.mma with FP32 accumulation in tensor memory.

@@ -297,7 +297,7 @@ __global__ void init_interior_kernel(T* __restrict__ y, const T* __restrict__ b,
 
 // One colour of the variable-coefficient patch smoother: persistent CTAs,
 // one patch at a time.  With TMA the closure of u and the interior of b of
-// the CTA's next patch arrive by two TMA boxes (as in patch_colour_kernel)
+// the CTA's next patch arrive by two TMA boxes
 // into the other input slot while the current patch is computed; without it
 // they are read element by element into the same layout.
 template <int DIM, int K, int NT, bool TMA>
