@@ -16,14 +16,11 @@
 #include <algorithm>
 #include <type_traits>
 
-#include <cuda.h>
 #include <cuda_runtime.h>
 
 #include "../../include/gmg.h"
-#include "async.cuh"
 #include "kernels.h"
 #include "pair_lines.cuh"
-#include "tma_host.h"
 
 namespace gmg {
 namespace {
@@ -51,29 +48,18 @@ __device__ __forceinline__ void var_row(int p, const V (&x)[K + 1], PA::acc& acc
   }
 }
 
-// Shared memory per patch: closure of u, interior of b (TMA boxes, or rows of
-// C and M elements without TMA); per pair the two fields of a contraction,
-// [z][y][x] with 2k rows per contracted axis; stages work in place.
-template <int DIM, int K, bool TMA>
+// Shared memory per pair: the two fields of a contraction, [z][y][x] with 2k
+// rows per contracted axis; stages work in place.  u and b go from global
+// memory straight to registers (lanes along x): without room for them twice
+// as many CTAs fit on an SM, which overlap one another's loads and barriers.
+template <int DIM, int K>
 struct VarSmem {
   static constexpr int C = 2 * K + 1, M = 2 * K - 1, H = 2 * K;
-  static constexpr int A = 16 / (int)sizeof(T);
-  static constexpr int XU = TMA ? (C + A - 1 + A - 1) / A * A : C;
-  static constexpr int XB = TMA ? XU : M;
-  static constexpr int R128 = 128 / (int)sizeof(T);
-  static constexpr int rnd(int n) { return (n + R128 - 1) / R128 * R128; }
-  static constexpr int NCLO = rnd(DIM == 3 ? C * C * XU : C * XU);
-  static constexpr int NBIN = rnd(DIM == 3 ? M * M * XB : M * XB);
   static constexpr int NINT = DIM == 3 ? M * M * M : M * M;
-  static constexpr int IN = NCLO + NBIN;
   static constexpr int R = DIM == 3 ? C : H;             // row (x)
   static constexpr int F = DIM == 3 ? C * H * R : C * R;  // one field
   static constexpr int NCELL = 1 << DIM;
-  static constexpr int bytes(int pp) {
-    return pp * (2 * IN * (int)sizeof(T) + (2 * F + NCELL) * (int)sizeof(E)) + 128;
-  }
-  static constexpr int BOX_U = (DIM == 3 ? C * C * XU : C * XU) * (int)sizeof(T);
-  static constexpr int BOX_B = (DIM == 3 ? M * M * XB : M * XB) * (int)sizeof(T);
+  static constexpr int bytes(int pp) { return pp * (2 * F + NCELL) * (int)sizeof(E); }
 };
 
 struct VarArgs {
@@ -83,10 +69,6 @@ struct VarArgs {
   const T* coef;
   const T* vscale;  // abar, theta per interior vertex
   const T* dinv;
-  int* err;
-};
-struct VarMaps {
-  CUtensorMap u, b;
 };
 
 // A CTA takes 2 PP consecutive patches of the colour, a thread the same line
@@ -96,93 +78,53 @@ struct VarMaps {
 //   z: r = h^{2-d} b + the columns of a node (1, 2 or 4), forward transform |
 //   y: forward | x: forward, diagonal, backward | y: backward |
 //   z: backward, u += omega theta / abar d
-template <int DIM, int K, int NT, int PP, bool TMA>
-__global__ void __launch_bounds__(NT) pair_var_kernel(const __grid_constant__ VarArgs va,
-                                                      const __grid_constant__ VarMaps maps) {
-  using Z = VarSmem<DIM, K, TMA>;
-  constexpr int C = Z::C, M = Z::M, H = Z::H, XU = Z::XU, XB = Z::XB, R = Z::R, F = Z::F, NP = 2 * PP;
+template <int DIM, int K, int NT, int PP, int CTAS, bool PRE>
+__global__ void __launch_bounds__(NT, CTAS) pair_var_kernel(const __grid_constant__ VarArgs va) {
+  using Z = VarSmem<DIM, K>;
+  constexpr int C = Z::C, M = Z::M, H = Z::H, R = Z::R, F = Z::F, NP = 2 * PP;
   constexpr int LINES = DIM == 3 ? M * M : M, NCELL = Z::NCELL;
-  static_assert(NP <= NT, "one lane issues the copies of one patch");
+  static_assert(NP <= NT, "one thread sets up one patch");
   extern __shared__ __align__(128) unsigned char smem_raw[];
-  T* const IN = reinterpret_cast<T*>(smem_raw + ((128 - (async::smem_u32(smem_raw) & 127)) & 127));  // [NP][IN]
-  E* const W = reinterpret_cast<E*>(IN + NP * Z::IN);  // [PP][2][F]
-  E* const CO = W + PP * 2 * F;                         // [PP][NCELL] cell coefficients of both patches
-  __shared__ long long s_origin[NP];
-  __shared__ int s_shift[NP], s_vert[NP][3];
+  E* const W = reinterpret_cast<E*>(smem_raw);  // [PP][2][F]
+  E* const CO = W + PP * 2 * F;                  // [PP][NCELL] cell coefficients of both patches
+  __shared__ long long s_origin[NP], s_cell[NP];
   __shared__ T s_scale[NP];
-  __shared__ __align__(8) uint64_t s_bar;
   const PatchLaunch& pl = va.pl;
   const long long py = pl.g.py, pz = pl.g.pz;
   const int g0 = blockIdx.x * NP, nv = min(NP, pl.n_patches - g0), npair = (nv + 1) / 2, n = pl.g.n;
   const float sb = (float)pl.sb;  // an integer power of the cell count, exact in float
-  auto uo = [](int x, int y, int z) { return DIM == 3 ? (z * C + y) * XU + x : y * XU + x; };
-  auto bo = [](int x, int y, int z) { return DIM == 3 ? (z * M + y) * XB + x : y * XB + x; };
-  if (TMA) {
-    if (threadIdx.x == 0) {
-      async::mbar_init(&s_bar, 1);
-      async::mbar_arrive_expect_tx(&s_bar, (uint32_t)(nv * (Z::BOX_U + Z::BOX_B)));
-    }
-    __syncthreads();
-  }
-  {
-    const int q = threadIdx.x / 32 + (threadIdx.x % 32) * (NT / 32);  // the patches are spread over the warps
-    if (q < nv) {
-      const int pid = g0 + q;
-      const int i0 = pid % pl.count[0], rest = pid / pl.count[0];
-      const int i1 = rest % pl.count[1], i2 = DIM == 3 ? rest / pl.count[1] : 0;
-      const int v0 = pl.first[0] + 2 * i0, v1 = pl.first[1] + 2 * i1, v2 = DIM == 3 ? pl.first[2] + 2 * i2 : 1;
-      const int o0 = (v0 - 1) * K, o1 = (v1 - 1) * K, o2 = (v2 - 1) * K;
-      s_origin[q] = o0 + py * o1 + (DIM == 3 ? pz * o2 : 0);
-      s_shift[q] = TMA ? o0 % Z::A : 0;
-      s_vert[q][0] = v0 - 1;
-      s_vert[q][1] = v1 - 1;
-      s_vert[q][2] = v2 - 1;
-      if constexpr (TMA) {
-        T* const dst = IN + q * Z::IN;
-        const int xa = o0 - o0 % Z::A;
-        if (DIM == 3) {
-          async::tma_load_3d(dst, &maps.u, xa, o1, o2, &s_bar);
-          async::tma_load_3d(dst + Z::NCLO, &maps.b, xa, o1 + 1, o2 + 1, &s_bar);
-        } else {
-          async::tma_load_2d(dst, &maps.u, xa, o1, &s_bar);
-          async::tma_load_2d(dst + Z::NCLO, &maps.b, xa, o1 + 1, &s_bar);
-        }
-      }
-      const long long vid = (v0 - 1) + (long long)(n - 1) * ((v1 - 1) + (DIM == 3 ? (long long)(n - 1) * (v2 - 1) : 0));
-      s_scale[q] = (T)pl.omega * va.vscale[2 * vid + 1] / va.vscale[2 * vid];
-    }
+  if ((int)threadIdx.x < NP) {  // (a lone last patch is carried twice and stored once)
+    const int q = threadIdx.x, pid = g0 + min(q, nv - 1);
+    const int i0 = pid % pl.count[0], rest = pid / pl.count[0];
+    const int i1 = rest % pl.count[1], i2 = DIM == 3 ? rest / pl.count[1] : 0;
+    const int v0 = pl.first[0] + 2 * i0, v1 = pl.first[1] + 2 * i1, v2 = DIM == 3 ? pl.first[2] + 2 * i2 : 1;
+    s_origin[q] = (v0 - 1) * K + py * ((v1 - 1) * K) + (DIM == 3 ? pz * ((v2 - 1) * K) : 0);
+    s_cell[q] = (v0 - 1) + (long long)n * ((v1 - 1) + (DIM == 3 ? (long long)n * (v2 - 1) : 0));
+    const long long vid = (v0 - 1) + (long long)(n - 1) * ((v1 - 1) + (DIM == 3 ? (long long)(n - 1) * (v2 - 1) : 0));
+    s_scale[q] = (T)pl.omega * va.vscale[2 * vid + 1] / va.vscale[2 * vid];
   }
   __syncthreads();
   for (int t = threadIdx.x; t < npair * NCELL; t += NT) {
     const int q = t / NCELL, c = t % NCELL;
-    auto cell = [&](int p) -> T {
-      return va.coef[s_vert[p][0] + (c & 1) + (long long)n * ((s_vert[p][1] + ((c >> 1) & 1)) +
-                                                             (DIM == 3 ? (long long)n * (s_vert[p][2] + (c >> 2)) : 0))];
-    };
-    PA::store(CO[t], PA::pack(cell(2 * q), cell(2 * q + 1 < nv ? 2 * q + 1 : 2 * q)));
+    const long long o = (c & 1) + (long long)n * (((c >> 1) & 1) + (DIM == 3 ? (long long)n * (c >> 2) : 0));
+    PA::store(CO[t], PA::pack(va.coef[s_cell[2 * q] + o], va.coef[s_cell[2 * q + 1] + o]));
   }
-  bool wait_ok = true;  // an expired wait is recorded and the kernel carries on
-  if constexpr (TMA) {
-    wait_ok = async::mbar_wait(&s_bar, 0);
-  } else {  // element by element
-    constexpr int NC = DIM == 3 ? C * C * C : C * C;
-    for (int t = threadIdx.x; t < nv * NC; t += NT) {
-      const int p = t / NC, l = t % NC, x = l % C, row = l / C;
-      IN[p * Z::IN + l] = va.u[s_origin[p] + x + py * (row % C) + (DIM == 3 ? pz * (row / C) : 0)];
-    }
-    for (int t = threadIdx.x; t < nv * Z::NINT; t += NT) {
-      const int p = t / Z::NINT, l = t % Z::NINT, x = l % M, row = l / M;
-      IN[p * Z::IN + Z::NCLO + l] =
-          va.b[s_origin[p] + 1 + x + py * (row % M + 1) + (DIM == 3 ? pz * (row / M + 1) : 0)];
-    }
-  }
-  __syncthreads();  // (also the coefficients)
-  // (a lone last patch has whatever the buffer holds beside it; nothing of
-  // that is stored)
-  auto input = [&](int q, int second) -> const T* {
-    const int p = 2 * q + second;
-    return IN + p * Z::IN + (p < nv ? s_shift[p] : 0);
+  // the rows of b are on their way from the start
+  constexpr bool EARLY = PRE && PP * LINES <= NT;
+  const long long ps = DIM == 3 ? pz : py;
+  T eb[EARLY ? 2 * M : 1];
+  auto rhs = [&](int t, int p) -> const T* {
+    const int ln = t % LINES;
+    return va.b + s_origin[2 * (t / LINES) + p] + 1 + ln % M + (DIM == 3 ? py * (1 + ln / M) : 0) + ps;
   };
+  if constexpr (EARLY) {
+    const int t = (int)threadIdx.x < npair * LINES ? threadIdx.x : 0;
+#pragma unroll
+    for (int l = 0; l < M; ++l) {
+      eb[l] = __ldg(rhs(t, 0) + ps * l);
+      eb[M + l] = __ldg(rhs(t, 1) + ps * l);
+    }
+  }
   // row of a cell-wise axis that holds interior node i (the first of the two
   // at the vertex)
   auto pos = [](int i) { return i + (i >= K ? 1 : 0); };
@@ -206,9 +148,9 @@ __global__ void __launch_bounds__(NT) pair_var_kernel(const __grid_constant__ Va
     // ---- y: P = M_y u, Q = K_y u on lines (x, z), from -u ----
     for (int t = threadIdx.x; t < npair * C * C; t += NT) {
       const int q = t / (C * C), x = t % C, z = t % (C * C) / C;
-      const T *const a = input(q, 0) + uo(x, 0, z), *const b = input(q, 1) + uo(x, 0, z);
+      const T *const a = va.u + s_origin[2 * q] + x + pz * z, *const b = va.u + s_origin[2 * q + 1] + x + pz * z;
       E* const P = W + q * 2 * F + z * H * R + x;
-      line_rows([&](int y) -> V { return PA::pack_neg(a[y * XU], b[y * XU]); },
+      line_rows([&](int y) -> V { return PA::pack_neg(a[py * y], b[py * y]); },
                 [&](int j, V m, V k) {
                   PA::store(P[j * R], m);
                   PA::store(P[F + j * R], k);
@@ -247,7 +189,7 @@ __global__ void __launch_bounds__(NT) pair_var_kernel(const __grid_constant__ Va
     // ---- x: P = M_x u, Q = K_x u on rows y, from -u ----
     for (int t = threadIdx.x; t < npair * C; t += NT) {
       const int q = t / C, y = t % C;
-      const T *const a = input(q, 0) + uo(0, y, 0), *const b = input(q, 1) + uo(0, y, 0);
+      const T *const a = va.u + s_origin[2 * q] + py * y, *const b = va.u + s_origin[2 * q + 1] + py * y;
       E* const P = W + q * 2 * F + y * R;
       line_rows([&](int x) -> V { return PA::pack_neg(a[x], b[x]); },
                 [&](int i, V m, V k) {
@@ -296,8 +238,7 @@ __global__ void __launch_bounds__(NT) pair_var_kernel(const __grid_constant__ Va
   };
   for (int t = threadIdx.x; t < npair * LINES; t += NT) {
     const int q = t / LINES, ln = t % LINES, i = ln % M, j = ln / M;
-    const int bofs = Z::NCLO + (TMA ? 1 : 0) + (DIM == 3 ? bo(i, j, 0) : i);
-    const T *const ba = input(q, 0) + bofs, *const bb = input(q, 1) + bofs;
+    const T *const ba = rhs(t, 0), *const bb = rhs(t, 1);
     E* const w = column(q, ln);
     const bool two_x = i == K - 1, two_y = DIM == 3 && j == K - 1;
     V r[M];
@@ -310,8 +251,10 @@ __global__ void __launch_bounds__(NT) pair_var_kernel(const __grid_constant__ Va
         if (two_x) s2 = PA::sum(s2, PA::load(w[l * SL + R + 1]));
         s = PA::sum(s, s2);
       }
-      const int o = (DIM == 3 ? M * XB : XB) * l;
-      r[l] = PA::sum(PA::value(PA::scaled(sb, PA::pack(ba[o], bb[o]))), s);
+      V rb;
+      if constexpr (EARLY) rb = PA::pack(eb[l], eb[M + l]);
+      else rb = PA::pack(__ldg(ba + ps * l), __ldg(bb + ps * l));
+      r[l] = PA::sum(PA::value(PA::scaled(sb, rb)), s);
     }
     pl_forward<K>(r, [&](int l, V v) { PA::store(w[l * SL], v); });
   }
@@ -344,7 +287,6 @@ __global__ void __launch_bounds__(NT) pair_var_kernel(const __grid_constant__ Va
   __syncthreads();
   if (DIM == 3) line_y(std::false_type());
   // ---- backward along the slowest axis and scatter ----
-  const long long ps = DIM == 3 ? pz : py;
   for (int t = threadIdx.x; t < npair * LINES; t += NT) {
     const int q = t / LINES, ln = t % LINES;
     const E* const w = column(q, ln);
@@ -354,41 +296,30 @@ __global__ void __launch_bounds__(NT) pair_var_kernel(const __grid_constant__ Va
     const bool two = 2 * q + 1 < nv;
     const int x = 1 + ln % M, y = DIM == 3 ? 1 + ln / M : 0;
     const long long ofs = x + (DIM == 3 ? py * y : 0) + ps;
-    const int uofs = DIM == 3 ? uo(x, y, 1) : uo(x, 1, 0);
-    constexpr int US = DIM == 3 ? C * XU : XU;
-    T* const ga = va.u + s_origin[2 * q] + ofs;
-    T* const gb = two ? va.u + s_origin[2 * q + 1] + ofs : ga;
-    const T *const ia = input(q, 0) + uofs, *const ib = input(q, 1) + uofs;
-    const T sa = s_scale[2 * q], sc = two ? s_scale[2 * q + 1] : T(0);
+    T *const ga = va.u + s_origin[2 * q] + ofs, *const gb = va.u + s_origin[2 * q + 1] + ofs;
+    const T sa = s_scale[2 * q], sc = s_scale[2 * q + 1];
+    T oa[M], ob[M];
+#pragma unroll
+    for (int l = 0; l < M; ++l) {
+      oa[l] = ga[ps * l];
+      ob[l] = gb[ps * l];
+    }
     pl_backward<K>(v, [&](int l, V d) {
-      ga[ps * l] = fma(sa, PA::x(d), ia[US * l]);
-      if (two) gb[ps * l] = fma(sc, PA::y(d), ib[US * l]);
+      ga[ps * l] = fma(sa, PA::x(d), oa[l]);
+      if (two) gb[ps * l] = fma(sc, PA::y(d), ob[l]);
     });
   }
-  if (!wait_ok) atomicExch(va.err, GMG_ERR_TIMEOUT);
 }
 
 // ---- host side ----
 
-// patch pairs and threads per CTA: as many pairs as fill the threads with the
-// interior lines of a stage
-template <int DIM, int K>
-struct VarPairCfg {
-  static constexpr int LINES = DIM == 3 ? (2 * K - 1) * (2 * K - 1) : 2 * K - 1;
-#ifdef VPP
-  static constexpr int NT = VNT, PP = VPP;
-#else
-  static constexpr int NT = DF || DIM == 2 ? 128 : 32;
-  static constexpr int PP = std::max(1, std::min(NT / LINES, 3 * NT / 8));
-#endif
-};
-
-template <int DIM, int K, bool TMA>
-int var_launch(const VarArgs& va, const VarMaps& maps, cudaStream_t s) {
-  using Cfg = VarPairCfg<DIM, K>;
-  constexpr int SMEM = VarSmem<DIM, K, TMA>::bytes(Cfg::PP);
+template <int DIM, int K, int NT, int PP, int CTAS, bool PRE>
+int var_pair_launch(const PatchLaunch& pl, T* u, const T* b, const T* coef, const T* vscale, const T* dinv,
+                    cudaStream_t s) {
+  if (pl.n_patches <= 0) return GMG_OK;
+  constexpr int SMEM = VarSmem<DIM, K>::bytes(PP);
   static_assert(SMEM <= 227 * 1024, "sweep kernel shared memory exceeds the per-CTA limit");
-  auto kern = pair_var_kernel<DIM, K, Cfg::NT, Cfg::PP, TMA>;
+  auto kern = pair_var_kernel<DIM, K, NT, PP, CTAS, PRE>;
   static PerDevice<bool> ready_dev;  // attribute set once per device
   bool* const ready = ready_dev.get();
   if (!ready) return GMG_ERR_CUDA;
@@ -397,26 +328,33 @@ int var_launch(const VarArgs& va, const VarMaps& maps, cudaStream_t s) {
       return GMG_ERR_CUDA;
     *ready = true;
   }
-  kern<<<(va.pl.n_patches + 2 * Cfg::PP - 1) / (2 * Cfg::PP), Cfg::NT, SMEM, s>>>(va, maps);
+  const VarArgs va{pl, u, b, coef, vscale, dinv};
+  kern<<<(pl.n_patches + 2 * PP - 1) / (2 * PP), NT, SMEM, s>>>(va);
   count_launch();
   return cudaGetLastError() == cudaSuccess ? GMG_OK : GMG_ERR_CUDA;
 }
 
+// Patch pairs and threads per CTA, and the CTAs per SM that the registers are
+// limited for; PRE: the rows of b are loaded before the first stage.  As many
+// pairs as fill the threads with the interior lines of a stage.  Measured per
+// sweep (us), the shape taken first: FP64 Q3 64^3 10 pairs in 256 threads with
+// registers for 2 CTAs 1384 (without PRE 1474), 5 in 128 for 4 1617, for 1
+// 2070; Q2 96^3 14 in 128 for 5 1168 (1235), for 1 1504; 2D Q3 1024^2 25 in 128
+// for 5 717, for 1 1131; FP32 Q3 64^3 5 in 128 317, 1 in 32 341.
+template <int DIM, int K>
+struct VarPairCfg {
+  static constexpr int LINES = DIM == 3 ? (2 * K - 1) * (2 * K - 1) : 2 * K - 1;
+  static constexpr int NT = DF && DIM == 3 && K == 3 ? 256 : 128;
+  static constexpr int PP = std::max(1, std::min(NT / LINES, 3 * NT / 8));
+  static constexpr int CTAS = !DF || K == 1 ? 1 : DIM == 3 && K == 3 ? 2 : 5;
+  static constexpr bool PRE = DF || DIM == 2;
+};
+
 template <int DIM, int K>
 int var_pair_impl(const PatchLaunch& pl, T* u, const T* b, const T* coef, const T* vscale, const T* dinv,
                   cudaStream_t s) {
-  if (pl.n_patches <= 0) return GMG_OK;
-  VarArgs va{pl, u, b, coef, vscale, dinv, device_wait_flag()};
-  if (!va.err) return GMG_ERR_CUDA;
-  VarMaps maps{};
-  constexpr int es = (int)sizeof(T);
-  if (!tma_vector_ok(u, es, DIM, pl.g.py, pl.g.pz) || !tma_vector_ok(b, es, DIM, pl.g.py, pl.g.pz))
-    return var_launch<DIM, K, false>(va, maps, s);
-  using Z = VarSmem<DIM, K, true>;
-  if (!tma_encode(&maps.u, u, es, DIM, pl.g.N, pl.g.py, pl.g.pz, Z::XU, Z::C) ||
-      !tma_encode(&maps.b, b, es, DIM, pl.g.N, pl.g.py, pl.g.pz, Z::XB, Z::M))
-    return GMG_ERR_CUDA;
-  return var_launch<DIM, K, true>(va, maps, s);
+  using Cfg = VarPairCfg<DIM, K>;
+  return var_pair_launch<DIM, K, Cfg::NT, Cfg::PP, Cfg::CTAS, Cfg::PRE>(pl, u, b, coef, vscale, dinv, s);
 }
 
 }  // namespace
