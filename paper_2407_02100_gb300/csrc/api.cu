@@ -758,10 +758,10 @@ int gmg::detail::create_problem(const gmg_desc* d, gmg_problem* p, const CreateO
     if (fe > 0 && dalloc(p, &p->faces, fe * p->esize) != GMG_OK) p->faces = nullptr;
   }
   // workspace of the three-pass FP64 operator (also used by the FP64 CG of
-  // single-precision problems): four finest-level vectors; without memory
+  // single-precision problems): two finest-level vectors; without memory
   // for it the tile kernel is used
   if (staged_apply_preferred(dim, k) && !opt.no_faces &&
-      dalloc(p, &p->apply_ws, 4 * p->levels[L - 1].n_elems * 8) != GMG_OK)
+      dalloc(p, &p->apply_ws, 2 * p->levels[L - 1].n_elems * 8) != GMG_OK)
     p->apply_ws = nullptr;
   // transfer tables
   std::vector<double> P1;

@@ -359,7 +359,7 @@ int gmg_batch_create(const gmg_desc* desc, int n_problems, const int* n_cells, g
   if (staged_apply_preferred(desc->dim, desc->degree)) {
     long long lmax = 0;
     for (long long l : B->len) lmax = std::max(lmax, l);
-    if (balloc(B, &B->apply_ws, 4 * lmax * 8) != GMG_OK) B->apply_ws = nullptr;
+    if (balloc(B, &B->apply_ws, 2 * lmax * 8) != GMG_OK) B->apply_ws = nullptr;
   }
   std::vector<long long> cstart;
   std::vector<int> clen, cowner, cbegin;

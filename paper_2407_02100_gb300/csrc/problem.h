@@ -109,7 +109,7 @@ struct gmg_problem {
   // FP64 colour steps of at most this many patches use the coarse-level
   // kernel (gmg_set_small_sweep; 0: never; set by gmg_create)
   int small_patches = 0;
-  // workspace of the three-pass FP64 3D operator (four finest-level
+  // workspace of the three-pass FP64 3D operator (two finest-level
   // vectors), null where the tile kernel is used
   void* apply_ws = nullptr;
   bool three_pass = true;  // gmg_set_three_pass_operator

@@ -1,237 +1,189 @@
-// Halo-free FP64 form of the 3D level operator: three passes over the
-// level, one per axis, each a 1D contraction with the global 1D matrices
-// (unit-cell mass M and stiffness K assembled along one axis), through two
-// pairs of workspace vectors:
+// FP64 form of the 3D level operator in three passes, one per axis, each a 1D
+// contraction with the global 1D matrices (unit-cell mass M and stiffness K
+// assembled along one axis), through two workspace vectors:
 //   pass z: P = M_z u,  Q = K_z u
 //   pass y: A1 = M_y P, A2 = K_y P + M_y Q
 //   pass x: y = alpha (K_x A1 + M_x A2) + beta b     (interior nodes)
 // which is A = K (x) M (x) M + M (x) K (x) M + M (x) M (x) K by sum
 // factorisation (Sec. 2, App. A.1 with the cell integrals summed into
 // global rows).  The tile kernel recomputes a halo of up to K + 1 nodes per
-// direction in its first two stages; here every output row is evaluated
-// once, for ten passes of level vectors through HBM.  Included by
-// patch_f64.cu after patch_kernels.cuh (T = double).
+// direction in its first two stages; here only the y rows of a tile's left
+// columns are evaluated twice, for six passes of level vectors through HBM.
+// Included by patch_f64.cu after patch_kernels.cuh (T = double).
 #pragma once
 
 namespace gmg {
 namespace GMG_NS {
 
-// One thread evaluates the K global rows of nodes c K .. c K + K - 1 along
-// AX (cell c of that axis) at one position of the other two axes, from the
-// 2K + 1 inputs c K - K .. c K + K of each input vector (zero outside the
-// lattice).  Row c K (a vertex) is row K of cell c - 1 plus row 0 of cell c;
-// row c K + p (0 < p < K) is row p of cell c.
-//   AX 2: positions all (x, y), rows z interior;  in0 = u -> out0 = M in0, out1 = K in0
-//   AX 1: positions all x, z interior, rows y interior;
-//         in0 = P, in1 = Q -> out0 = M P, out1 = K P + M Q
-//   AX 0: positions y, z interior, rows x interior;
-//         in0 = A1, in1 = A2 -> out0 = alpha (K A1 + M A2) + beta b
-template <int K, int AX>
-__global__ void __launch_bounds__(128) axis_pass_kernel(const T* __restrict__ in0, const T* __restrict__ in1,
-                                                        T* __restrict__ out0, T* __restrict__ out1,
-                                                        const T* __restrict__ bvec, const LevelGeom g, T alpha,
-                                                        T beta) {
-  constexpr int W = 2 * K + 1;
-  const int N = g.N, n = g.n;
-  const long long py = g.py, pz = g.pz;
-  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  int x, y, z, c;
-  long long stride;
-  if (AX == 2) {
-    if (t >= (long long)N * N * n) return;
-    x = (int)(t % N);
-    const long long r = t / N;
-    y = (int)(r % N);
-    c = (int)(r / N);
-    z = 0;
-    stride = pz;
-  } else if (AX == 1) {
-    if (t >= (long long)N * (N - 2) * n) return;
-    x = (int)(t % N);
-    const long long r = t / N;
-    z = 1 + (int)(r % (N - 2));
-    c = (int)(r / (N - 2));
-    y = 0;
-    stride = py;
-  } else {
-    if (t >= (long long)n * (N - 2) * (N - 2)) return;
-    c = (int)(t % n);
-    const long long r = t / n;
-    y = 1 + (int)(r % (N - 2));
-    z = 1 + (int)(r / (N - 2));
-    x = 0;
-    stride = 1;
-  }
-  // element offset of node c K - K of the thread's line
-  const long long base = x + py * y + pz * z + stride * ((long long)c * K - K);
-  auto E = [](int kind, int r, int q) -> T {
-    return kind == 0 ? c_Mc[off_cell(K) + r * (K + 1) + q] : c_Kc[off_cell(K) + r * (K + 1) + q];
-  };
-  T a[W], b[AX == 2 ? 1 : W];
+// A thread evaluates the K global rows of nodes c K .. c K + K - 1 along an
+// axis (cell c of that axis) from the 2K + 1 inputs c K - K .. c K + K (zero
+// outside the lattice).  Row c K (a vertex) is row K of cell c - 1 plus row 0
+// of cell c; row c K + p (0 < p < K) is row p of cell c.
+//
+// acc += (FIRST: =) global row p of a segment (row c K + p, see above), matrix
+// KIND, applied to the 2K + 1 window v, in double-float (Dot2)
+template <int K, int KIND, bool FIRST>
+__device__ __forceinline__ void segment_row_df(int p, const dfv (&v)[2 * K + 1], df_acc& acc) {
+  auto eh = [](int r, int q) { return KIND == 0 ? c_Mchi[off_cell(K) + r * (K + 1) + q] : c_Kchi[off_cell(K) + r * (K + 1) + q]; };
+  auto el = [](int r, int q) { return KIND == 0 ? c_Mclo[off_cell(K) + r * (K + 1) + q] : c_Kclo[off_cell(K) + r * (K + 1) + q]; };
+  if (p == 0) {
 #pragma unroll
-  for (int w = 0; w < W; ++w) {
-    const int node = c * K - K + w;
-    const bool ok = node >= 0 && node < N;
-    a[w] = ok ? in0[base + stride * w] : T(0);
-    if constexpr (AX != 2) b[w] = ok ? in1[base + stride * w] : T(0);
-  }
-  // global row p of the segment, matrix kind, applied to the window v
-  auto row = [&](int p, int kind, const T (&v)[W], T acc) -> T {
-    if (p == 0) {
-#pragma unroll
-      for (int q = 0; q <= K; ++q) acc = fma(E(kind, K, q), v[q], acc);
+    for (int q = 0; q <= K; ++q) {
+      if (FIRST && q == 0) acc = df_acc_first(eh(K, q), el(K, q), v[q]);
+      else df_acc_add(acc, eh(K, q), el(K, q), v[q]);
     }
+  }
 #pragma unroll
-    for (int q = 0; q <= K; ++q) acc = fma(E(kind, p, q), v[K + q], acc);
-    return acc;
-  };
-#pragma unroll
-  for (int p = 0; p < K; ++p) {
-    const int node = c * K + p;
-    if (node < 1 || node > N - 2) continue;
-    const long long o = base + stride * (K + p);
-    if constexpr (AX == 2) {
-      out0[o] = row(p, 0, a, T(0));
-      out1[o] = row(p, 1, a, T(0));
-    } else if constexpr (AX == 1) {
-      out0[o] = row(p, 0, a, T(0));
-      out1[o] = row(p, 0, b, row(p, 1, a, T(0)));
-    } else {
-      T v = alpha * row(p, 0, b, row(p, 1, a, T(0)));
-      if (bvec) v = fma(beta, bvec[o], v);
-      out0[o] = v;
-    }
+  for (int q = 0; q <= K; ++q) {
+    if (FIRST && p > 0 && q == 0) acc = df_acc_first(eh(p, q), el(p, q), v[K + q]);
+    else df_acc_add(acc, eh(p, q), el(p, q), v[K + q]);
   }
 }
 
-// The same three passes in double-float arithmetic (FP64 problems; GB300
-// runs FP64 at about 1/74 of its FP32 rate): the workspace vectors hold
-// float pairs (hi, lo) in the 8 bytes of a double, the rows accumulate in
-// Dot2 form with the float-pair cell matrices, and the x pass forms
-// alpha (K A1 + M A2) + beta b in FP64 from the pair's value (two FP64
-// operations per node).
-template <int K, int AX>
-__global__ void __launch_bounds__(128) axis_pass_df_kernel(const void* __restrict__ in0v,
-                                                           const float2* __restrict__ in1,
-                                                           float2* __restrict__ out0, float2* __restrict__ out1,
-                                                           double* __restrict__ yout, const double* __restrict__ bvec,
-                                                           const LevelGeom g, double alpha, double beta) {
+// The same in double-float arithmetic (FP64 problems; GB300 runs FP64 at about
+// 1/74 of its FP32 rate), in two launches: the workspace vectors hold float
+// pairs (hi, lo) in the 8 bytes of a double, the rows accumulate in Dot2 form
+// with the float-pair cell matrices, and alpha (K A1 + M A2) + beta b is formed
+// in FP64 from the pair's value (two FP64 operations per node).
+//
+// Pass z.  A CTA takes 128 consecutive x positions of one y and one cell layer.
+template <int K>
+__global__ void __launch_bounds__(128) pass_z_df_kernel(const double* __restrict__ in, float2* __restrict__ P,
+                                                        float2* __restrict__ Q, const LevelGeom g) {
   constexpr int W = 2 * K + 1;
-  const int N = g.N, n = g.n;
+  const int N = g.N;
   const long long py = g.py, pz = g.pz;
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  int x, y, z, c;
-  long long stride;
-  if (AX == 2) {
-    if (t >= (long long)N * N * n) return;
-    x = (int)(t % N);
-    const long long r = t / N;
-    y = (int)(r % N);
-    c = (int)(r / N);
-    z = 0;
-    stride = pz;
-  } else if (AX == 1) {
-    if (t >= (long long)N * (N - 2) * n) return;
-    x = (int)(t % N);
-    const long long r = t / N;
-    z = 1 + (int)(r % (N - 2));
-    c = (int)(r / (N - 2));
-    y = 0;
-    stride = py;
-  } else {
-    if (t >= (long long)n * (N - 2) * (N - 2)) return;
-    c = (int)(t % n);
-    const long long r = t / n;
-    y = 1 + (int)(r % (N - 2));
-    z = 1 + (int)(r / (N - 2));
-    x = 0;
-    stride = 1;
-  }
-  const long long base = x + py * y + pz * z + stride * ((long long)c * K - K);
-  dfv a[W], b[AX == 2 ? 1 : W];
+  if (t >= (long long)N * N * g.n) return;
+  const int x = (int)(t % N);
+  const long long r = t / N;
+  const int y = (int)(r % N), c = (int)(r / N);
+  const long long base = x + py * y + pz * ((long long)c * K - K);
+  dfv a[W];
 #pragma unroll
   for (int w = 0; w < W; ++w) {
-    const int node = c * K - K + w;
-    const bool ok = node >= 0 && node < N;
-    if constexpr (AX == 2) {
-      a[w] = ok ? df_from_double(static_cast<const double*>(in0v)[base + stride * w]) : dfv{0.f, 0.f};
-    } else {
-      const float2 va = ok ? static_cast<const float2*>(in0v)[base + stride * w] : make_float2(0.f, 0.f);
-      const float2 vb = ok ? in1[base + stride * w] : make_float2(0.f, 0.f);
+    const bool ok = w >= K || c > 0;
+    a[w] = ok ? df_from_double(in[base + pz * w]) : dfv{0.f, 0.f};
+  }
+#pragma unroll
+  for (int p = 0; p < K; ++p) {
+    if (p == 0 && c == 0) continue;  // a Dirichlet node
+    const long long o = base + pz * (K + p);
+    df_acc r0, r1;
+    segment_row_df<K, 0, true>(p, a, r0);
+    segment_row_df<K, 1, true>(p, a, r1);
+    const dfv v0 = df_acc_value(r0), v1 = df_acc_value(r1);
+    P[o] = make_float2(v0.hi, v0.lo);
+    Q[o] = make_float2(v1.hi, v1.lo);
+  }
+}
+
+// Passes y and x together on a tile of BX x BY cells of one z plane: A1 and A2
+// of the tile (with the K + 1 columns to its left) stay in shared memory, so
+// that four of the ten passes over level vectors are not made: Q4 64^3 403 ->
+// 367 us with pass z (140 us), Q3 51^3 121 -> 102.  Both launches are bound by the
+// FP32 pipe (Dot2 terms of 10 operations); limits on the registers only made
+// them slower (Q4 3 CTAs per SM 403 us, Q7 32^3 2 CTAs 509 against 444).  The y
+// rows are evaluated for ((BX + 1) K + 1) / (BX K) of the columns that are needed.
+template <int K>
+struct PlanePass {
+  static constexpr int BX = 64 / K, BY = 4, NT = 256;
+  static constexpr int EX = (BX + 1) * K + 1, EY = BY * K;
+  static constexpr int EXP = EX | 1;  // odd row: lanes of the x stage lie K entries apart
+  static constexpr int BYTES = 2 * EY * EXP * (int)sizeof(float2);
+};
+
+template <int K>
+__global__ void __launch_bounds__(PlanePass<K>::NT) pass_yx_df_kernel(
+    const float2* __restrict__ P, const float2* __restrict__ Q, double* __restrict__ yout,
+    const double* __restrict__ bvec, const LevelGeom g, double alpha, double beta, int tx, int ty) {
+  using D = PlanePass<K>;
+  constexpr int BX = D::BX, BY = D::BY, EX = D::EX, EXP = D::EXP, NT = D::NT, W = 2 * K + 1;
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  float2* const A1 = reinterpret_cast<float2*>(smem_raw);
+  float2* const A2 = A1 + D::EY * EXP;
+  const int N = g.N, n = g.n;
+  const long long py = g.py;
+  const int t0 = blockIdx.x % tx, t1 = blockIdx.x / tx % ty, z = 1 + blockIdx.x / (tx * ty);
+  const long long plane = g.pz * z;
+  const int x0 = (t0 * BX - 1) * K, c1 = t1 * BY;
+  for (int t = threadIdx.x; t < EX * BY; t += NT) {
+    const int xi = t % EX, x = x0 + xi, cy = t / EX, c = c1 + cy;
+    const bool in = x >= 0 && x < N && c < n;
+    const long long base = plane + x + py * ((long long)c * K - K);
+    dfv a[W], b[W];
+#pragma unroll
+    for (int w = 0; w < W; ++w) {
+      const bool ok = in && (w >= K || c > 0);
+      const float2 va = ok ? P[base + py * w] : make_float2(0.f, 0.f);
+      const float2 vb = ok ? Q[base + py * w] : make_float2(0.f, 0.f);
       a[w] = {va.x, va.y};
       b[w] = {vb.x, vb.y};
     }
+#pragma unroll
+    for (int p = 0; p < K; ++p) {
+      df_acc r0, r1;
+      segment_row_df<K, 0, true>(p, a, r0);
+      segment_row_df<K, 1, true>(p, a, r1);
+      segment_row_df<K, 0, false>(p, b, r1);
+      const dfv v0 = df_acc_value(r0), v1 = df_acc_value(r1);
+      const int o = (cy * K + p) * EXP + xi;
+      A1[o] = make_float2(v0.hi, v0.lo);
+      A2[o] = make_float2(v1.hi, v1.lo);
+    }
   }
-  // acc += (first: =) global row p of the cell matrix `kind` applied to the window v
-  auto row = [&](int p, int kind, const dfv (&v)[W], df_acc& acc, bool first) {
-    auto eh = [&](int r, int q) { return kind == 0 ? c_Mchi[off_cell(K) + r * (K + 1) + q] : c_Kchi[off_cell(K) + r * (K + 1) + q]; };
-    auto el = [&](int r, int q) { return kind == 0 ? c_Mclo[off_cell(K) + r * (K + 1) + q] : c_Kclo[off_cell(K) + r * (K + 1) + q]; };
-    if (p == 0) {
+  __syncthreads();
+  // one thread per cell of a row, rows along the lanes (odd row stride); the
+  // results go back through shared memory, so that the rows of b and y are
+  // read and written with lanes along x
+  static_assert(BX * D::EY <= NT, "one thread per cell row");
+  const int r = threadIdx.x % D::EY, cx = threadIdx.x / D::EY;
+  dfv v[K];
+  if (cx < BX) {
+    dfv a[W], b[W];
 #pragma unroll
-      for (int q = 0; q <= K; ++q) {
-        if (first && q == 0) acc = df_acc_first(eh(K, q), el(K, q), v[q]);
-        else df_acc_add(acc, eh(K, q), el(K, q), v[q]);
-      }
+    for (int w = 0; w < W; ++w) {
+      const float2 va = A1[r * EXP + cx * K + w], vb = A2[r * EXP + cx * K + w];
+      a[w] = {va.x, va.y};
+      b[w] = {vb.x, vb.y};
     }
 #pragma unroll
-    for (int q = 0; q <= K; ++q) {
-      if (first && p > 0 && q == 0) acc = df_acc_first(eh(p, q), el(p, q), v[K + q]);
-      else df_acc_add(acc, eh(p, q), el(p, q), v[K + q]);
+    for (int p = 0; p < K; ++p) {
+      df_acc acc;
+      segment_row_df<K, 1, true>(p, a, acc);
+      segment_row_df<K, 0, false>(p, b, acc);
+      v[p] = df_acc_value(acc);
     }
-  };
+  }
+  __syncthreads();
+  if (cx < BX) {
 #pragma unroll
-  for (int p = 0; p < K; ++p) {
-    const int node = c * K + p;
-    if (node < 1 || node > N - 2) continue;
-    const long long o = base + stride * (K + p);
-    df_acc r0, r1;
-    if constexpr (AX == 2) {
-      row(p, 0, a, r0, true);
-      row(p, 1, a, r1, true);
-      const dfv v0 = df_acc_value(r0), v1 = df_acc_value(r1);
-      out0[o] = make_float2(v0.hi, v0.lo);
-      out1[o] = make_float2(v1.hi, v1.lo);
-    } else if constexpr (AX == 1) {
-      row(p, 0, a, r0, true);
-      row(p, 1, a, r1, true);
-      row(p, 0, b, r1, false);
-      const dfv v0 = df_acc_value(r0), v1 = df_acc_value(r1);
-      out0[o] = make_float2(v0.hi, v0.lo);
-      out1[o] = make_float2(v1.hi, v1.lo);
-    } else {
-      row(p, 1, a, r0, true);
-      row(p, 0, b, r0, false);
-      double v = alpha * df_to_double(df_acc_value(r0));
-      if (bvec) v = fma(beta, bvec[o], v);
-      yout[o] = v;
-    }
+    for (int p = 0; p < K; ++p) A1[r * EXP + cx * K + p] = make_float2(v[p].hi, v[p].lo);
+  }
+  __syncthreads();
+  for (int t = threadIdx.x; t < BX * K * D::EY; t += NT) {
+    const int xi = t % (BX * K), yr = t / (BX * K), x = x0 + K + xi, y = c1 * K + yr;
+    if (x < 1 || x > N - 2 || y < 1 || y > N - 2) continue;
+    const float2 f = A1[yr * EXP + xi];
+    const long long o = plane + py * y + x;
+    double d = alpha * df_to_double(dfv{f.x, f.y});
+    if (bvec) d = fma(beta, bvec[o], d);
+    yout[o] = d;
   }
 }
 
 template <int K>
-static int staged_apply_impl(const ApplyLaunch& al, const T* x, T* y, const T* bvec, cudaStream_t s) {
+static int staged_apply_impl(const ApplyLaunch& al, const double* x, double* y, const double* bvec, cudaStream_t s) {
+  using D = PlanePass<K>;
+  static_assert(D::BYTES <= 48 * 1024, "tile exceeds the default shared memory of a CTA");
   const LevelGeom& g = al.g;
-  const long long ne = g.pz * g.N;
-  T* P = static_cast<T*>(al.ws);
-  T* Q = P + ne;
-  T* A1 = Q + ne;
-  T* A2 = A1 + ne;
-  const long long N = g.N, n = g.n;
-  const long long t2 = N * N * n, t1 = N * (N - 2) * n, t0 = n * (N - 2) * (N - 2);
-  auto blocks = [](long long t) { return (unsigned)((t + 127) / 128); };
-  if constexpr (sizeof(T) == 8) {  // double-float passes (pairs in the workspace)
-    float2 *P2 = reinterpret_cast<float2*>(P), *Q2 = reinterpret_cast<float2*>(Q);
-    float2 *A12 = reinterpret_cast<float2*>(A1), *A22 = reinterpret_cast<float2*>(A2);
-    axis_pass_df_kernel<K, 2><<<blocks(t2), 128, 0, s>>>(x, nullptr, P2, Q2, nullptr, nullptr, g, 0.0, 0.0);
-    axis_pass_df_kernel<K, 1><<<blocks(t1), 128, 0, s>>>(P2, Q2, A12, A22, nullptr, nullptr, g, 0.0, 0.0);
-    axis_pass_df_kernel<K, 0><<<blocks(t0), 128, 0, s>>>(A12, A22, nullptr, nullptr, y, bvec, g, al.alpha,
-                                                        al.beta);
-  } else {
-    axis_pass_kernel<K, 2><<<blocks(t2), 128, 0, s>>>(x, nullptr, P, Q, nullptr, g, T(0), T(0));
-    axis_pass_kernel<K, 1><<<blocks(t1), 128, 0, s>>>(P, Q, A1, A2, nullptr, g, T(0), T(0));
-    axis_pass_kernel<K, 0><<<blocks(t0), 128, 0, s>>>(A1, A2, y, nullptr, bvec, g, (T)al.alpha, (T)al.beta);
-  }
-  count_launch(3);
+  float2* const P = static_cast<float2*>(al.ws);
+  float2* const Q = P + g.pz * g.N;
+  const long long N = g.N, tx = (g.n + D::BX - 1) / D::BX, ty = (g.n + D::BY - 1) / D::BY;
+  pass_z_df_kernel<K><<<(unsigned)((N * N * g.n + 127) / 128), 128, 0, s>>>(x, P, Q, g);
+  pass_yx_df_kernel<K><<<(unsigned)(tx * ty * (N - 2)), D::NT, D::BYTES, s>>>(P, Q, y, bvec, g, al.alpha, al.beta,
+                                                                              (int)tx, (int)ty);
+  count_launch(2);
   return cudaGetLastError() == cudaSuccess ? GMG_OK : GMG_ERR_CUDA;
 }
 
