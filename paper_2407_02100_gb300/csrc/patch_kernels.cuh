@@ -386,33 +386,38 @@ __global__ void __launch_bounds__(NT) apply_kernel(const T* __restrict__ xin, T*
         }
       }
     } else {
+      // one thread per line and cell: with a thread per line a tile kept 16
+      // to 20 threads busy on chains of up to 100 FP64 operations
       // stage y: P = M_y x, Q = K_y x   (x:EIX, y:EOY)
-      for (int l = threadIdx.x; l < EIX; l += NT) {
-        T v[EIY];
+      for (int t = threadIdx.x; t < EIX * BY; t += NT) {
+        const int l = t % EIX, c = t / EIX;
+        T v[2 * K + 1];
 #pragma unroll
-        for (int j = 0; j < EIY; ++j) v[j] = A[l + j * EIX];
+        for (int j = 0; j <= 2 * K; ++j) v[j] = A[l + (c * K + j) * EIX];
 #pragma unroll
-        for (int o = 0; o < EOY; ++o) {
-          B[l + o * EIX] = cell_row<K, EIY, 0>(o, v);
-          B[EIX * EOY + l + o * EIX] = cell_row<K, EIY, 1>(o, v);
+        for (int p = 0; p < K; ++p) {
+          B[l + (c * K + p) * EIX] = cell_row<K, 2 * K + 1, 0>(p, v);
+          B[EIX * EOY + l + (c * K + p) * EIX] = cell_row<K, 2 * K + 1, 1>(p, v);
         }
       }
       __syncthreads();
-      for (int l = threadIdx.x; l < EOY; l += NT) {
-        int gy = g1 + K + l;
+      // stage x and write
+      for (int t = threadIdx.x; t < EOY * BX; t += NT) {
+        const int c = t % BX, l = t / BX;
+        const int gy = g1 + K + l;
         if (gy <= 0 || gy >= N - 1) continue;
-        T p[EIX], q[EIX];
+        T p[2 * K + 1], q[2 * K + 1];
 #pragma unroll
-        for (int j = 0; j < EIX; ++j) {
-          p[j] = B[j + EIX * l];
-          q[j] = B[EIX * EOY + j + EIX * l];
+        for (int j = 0; j <= 2 * K; ++j) {
+          p[j] = B[c * K + j + EIX * l];
+          q[j] = B[EIX * EOY + c * K + j + EIX * l];
         }
         const long long row = py * gy;
 #pragma unroll
-        for (int o = 0; o < EOX; ++o) {
-          int gx = g0 + K + o;
+        for (int o = 0; o < K; ++o) {
+          const int gx = g0 + K + c * K + o;
           if (gx <= 0 || gx >= N - 1) continue;
-          T v = alpha * (cell_row<K, EIX, 1>(o, p) + cell_row<K, EIX, 0>(o, q));
+          T v = alpha * (cell_row<K, 2 * K + 1, 1>(o, p) + cell_row<K, 2 * K + 1, 0>(o, q));
           if (bvec) v += beta * bvec[row + gx];
           y[row + gx] = v;
         }
