@@ -600,6 +600,15 @@ int coarse_solve(gmg_problem* p, const void* b, void* x) {
       return launch_dense_solve<double>(g, p->coarse_inv, p->coarse_n, (const double*)b, (double*)x, p->stream);
     return launch_dense_solve<float>(g, p->coarse_inv, p->coarse_n, (const float*)b, (float*)x, p->stream);
   }
+  if (coarse_fd_fits(g.dim, p->m0)) {
+    if (p->esize == 4)
+      return launch_coarse_fd<float>(g, p->m0, (const double*)p->c64_fwd, (const double*)p->c64_bwd,
+                                     (const double*)p->c64_dinv, (const float*)b, (float*)x, p->levels[0].n_elems,
+                                     p->stream);
+    return launch_coarse_fd<double>(g, p->m0, (const double*)p->coef_c_fwd, (const double*)p->coef_c_bwd,
+                                    (const double*)p->dinv0, (const double*)b, (double*)x, p->levels[0].n_elems,
+                                    p->stream);
+  }
   if (p->esize == 4) {  // single-precision problem: the coarse solve runs in FP64
     const long long n0 = p->levels[0].n_elems;
     CHECK(launch_convert_f32_f64(n0, (const float*)b, (double*)p->c64_b, p->stream));

@@ -170,6 +170,14 @@ template <typename T>
 int launch_patch_var_pair(const PatchLaunch& pl, T* u, const T* b, const T* coef, const T* vscale, const T* dinv,
                           cudaStream_t s);
 
+// Coarsest-level solve by global fast diagonalisation in one launch (FP64
+// arithmetic, m unknowns per direction, tables of m x m entries), for the sizes
+// that coarse_fd_fits accepts.
+bool coarse_fd_fits(int dim, int m);
+template <typename T>
+int launch_coarse_fd(const LevelGeom& g, int m, const double* fwd, const double* bwd, const double* dinv, const T* b,
+                     T* x, long long n_elems, cudaStream_t s);
+
 // x = Ainv b on the interior nodes of a level (Ainv dense FP64, interior
 // nodes numbered x fastest); the coarse solve of variable-coefficient problems
 template <typename T>

@@ -108,6 +108,26 @@ __global__ void __launch_bounds__(NT) patch_wide_df_kernel(const PatchLaunch pl,
   const long long origin = (long long)(pl.first[0] + 2 * i0 - 1) * K + py * ((pl.first[1] + 2 * i1 - 1) * K) +
                            (DIM == 3 ? pz * ((pl.first[2] + 2 * i2 - 1) * K) : 0);
   auto st = [](const dfv a) -> float2 { return make_float2(a.hi, a.lo); };
+  // b, the old u and the diagonal of the thread's interior nodes are on their
+  // way from the start (a step is one chain of latencies: a CTA has its SM
+  // nearly to itself)
+  constexpr int PER = (NINT + NT - 1) / NT;
+  constexpr bool EARLY = PER <= 2;
+  double eb[EARLY ? PER : 1], eu[EARLY ? PER : 1];
+  float2 ed[EARLY ? PER : 1];
+  auto interior = [&](int t) -> long long {
+    return origin + 1 + t % M + py * (t / M % M + 1) + (DIM == 3 ? pz * (t / (M * M) + 1) : 0);
+  };
+  if constexpr (EARLY) {
+#pragma unroll
+    for (int r = 0; r < PER; ++r) {
+      const int t = min((int)threadIdx.x + r * NT, NINT - 1);
+      const long long gi = interior(t);
+      eb[r] = b[gi];
+      eu[r] = u[gi];
+      ed[r] = __ldg(dd + t);
+    }
+  }
   for (int t = threadIdx.x; t < M * C; t += NT) {
     Mp[t] = make_float2(c_Mphi[off_patch(K) + t], c_Mplo[off_patch(K) + t]);
     Kp[t] = make_float2(c_Kphi[off_patch(K) + t], c_Kplo[off_patch(K) + t]);
@@ -161,10 +181,15 @@ __global__ void __launch_bounds__(NT) patch_wide_df_kernel(const PatchLaunch pl,
     float2* const R = DIM == 3 ? Y : X;
     constexpr int PLANE = DIM == 3 ? C * M * M : C * M;
     const float sbf = (float)pl.sb;  // h^{2-d}: the cell count in 3D, 1 in 2D, exact in float
-    for (int t = threadIdx.x; t < NINT; t += NT) {
+#pragma unroll
+    for (int r = 0; r < PER; ++r) {
+      const int t = threadIdx.x + r * NT;
+      if (t >= NINT) break;
       const int i = t % M, l = t / M;  // x, and the line (y, z)
-      const long long row = origin + 1 + py * ((DIM == 3 ? l % M : l) + 1) + (DIM == 3 ? pz * (l / M + 1) : 0);
-      const dfv bb = df_mul(df_from_double(b[row + i]), {sbf, 0.f});
+      double bv;
+      if constexpr (EARLY) bv = eb[r];
+      else bv = b[interior(t)];
+      const dfv bb = df_mul(df_from_double(bv), {sbf, 0.f});
       df_acc acc;
       wide_row<K, true>(acc, i, Kp, S1 + C * l, 1);
       wide_row<K, false>(acc, i, Mp, S1 + PLANE + C * l, 1);
@@ -177,14 +202,19 @@ __global__ void __launch_bounds__(NT) patch_wide_df_kernel(const PatchLaunch pl,
   float2* A = DIM == 3 ? Y : X;  // holds the residual
   float2* B = DIM == 3 ? X : Y;
   auto pass = [&](int axis, bool forward, bool scale) {
-    for (int t = threadIdx.x; t < NINT; t += NT) {
+#pragma unroll
+    for (int r = 0; r < PER; ++r) {
+      const int t = threadIdx.x + r * NT;
+      if (t >= NINT) break;
       const int x = t % M, y = (t / M) % M, z = DIM == 3 ? t / (M * M) : 0;
       const int i = axis == 0 ? x : axis == 1 ? y : z;                      // output index on the line
       const int s = axis == 0 ? 1 : axis == 1 ? M : M * M;                   // line stride
       const float2* line = A + t - i * s;
       dfv v = forward ? wide_fd<K, true>(i, Tt, line, s) : wide_fd<K, false>(i, Tt, line, s);
       if (scale) {
-        const float2 d = __ldg(dd + t);
+        float2 d;
+        if constexpr (EARLY) d = ed[r];
+        else d = __ldg(dd + t);
         v = df_mul(v, {d.x, d.y});
       }
       B[t] = st(v);
@@ -207,11 +237,16 @@ __global__ void __launch_bounds__(NT) patch_wide_df_kernel(const PatchLaunch pl,
   pass(0, false, false);
   // ---- scatter: u += omega d on the patch interior ----
   const double om = pl.omega;
-  for (int t = threadIdx.x; t < NINT; t += NT) {
-    const int x = t % M, y = (t / M) % M, z = DIM == 3 ? t / (M * M) : 0;
-    const long long gi = origin + 1 + x + py * (y + 1) + (DIM == 3 ? pz * (z + 1) : 0);
+#pragma unroll
+  for (int r = 0; r < PER; ++r) {
+    const int t = threadIdx.x + r * NT;
+    if (t >= NINT) break;
+    const long long gi = interior(t);
     const float2 d = A[t];
-    u[gi] = fma(om, df_to_double({d.x, d.y}), u[gi]);
+    double old;
+    if constexpr (EARLY) old = eu[r];
+    else old = u[gi];
+    u[gi] = fma(om, df_to_double({d.x, d.y}), old);
   }
 }
 

@@ -149,6 +149,56 @@ __global__ void dense_solve_kernel(LevelGeom g, const double* __restrict__ Ainv,
   if (lane == 0) x[node(warp)] = (T)acc;
 }
 
+// Coarsest-level solve x = (T x .. x T) diag(dinv) (T x .. x T)^T b in one
+// launch of one CTA, the m^dim unknowns in shared memory: FP64, summed in the
+// order of the axis passes (axis_op_kernel, scale_kernel), which give the same
+// bits in 5 (2D) or 7 (3D) launches, and 2 more for the conversions of a
+// single-precision problem.  x is written on the interior; of a
+// single-precision vector the rest becomes zero.
+constexpr int kCoarseThreads = 512;
+template <typename T>
+__global__ void __launch_bounds__(kCoarseThreads)
+    coarse_fd_kernel(LevelGeom g, int m, const double* __restrict__ fwd, const double* __restrict__ bwd,
+                     const double* __restrict__ dinv, const T* __restrict__ b, T* __restrict__ x, long long n_elems) {
+  extern __shared__ double coarse_smem[];
+  const int mm = m * m, nm = g.dim == 3 ? mm * m : mm;
+  double *in = coarse_smem, *out = in + nm;
+  double *const F = out + nm, *const B = F + mm;
+  auto node = [&](int i) -> long long {
+    return i % m + 1 + (long long)g.py * (i / m % m + 1) + (g.dim == 3 ? g.pz * (i / mm + 1) : 0);
+  };
+  for (int t = threadIdx.x; t < mm; t += kCoarseThreads) {
+    F[t] = fwd[t];
+    B[t] = bwd[t];
+  }
+  for (int t = threadIdx.x; t < nm; t += kCoarseThreads) in[t] = (double)b[node(t)];
+  __syncthreads();
+  for (int pass = 0; pass < 2 * g.dim; ++pass) {
+    const int ax = pass % g.dim, st = ax == 0 ? 1 : ax == 1 ? m : mm;
+    const double* const M = pass < g.dim ? F : B;
+    for (int t = threadIdx.x; t < nm; t += kCoarseThreads) {
+      const int o = t / st % m;
+      const double *const c = M + o * m, *const v = in + t - o * st;
+      double acc = 0.0;
+      for (int w = 0; w < m; ++w) acc += c[w] * v[w * st];
+      out[t] = pass == g.dim - 1 ? acc * dinv[t] : acc;
+    }
+    __syncthreads();
+    double* const tmp = in;
+    in = out;
+    out = tmp;
+  }
+  if constexpr (sizeof(T) == 4) {
+    for (long long e = threadIdx.x; e < n_elems; e += kCoarseThreads) {
+      const int ix = (int)(e % g.py), iy = (int)(e / g.py % g.N), iz = g.dim == 3 ? (int)(e / g.pz) : 1;
+      const bool ok = ix >= 1 && ix <= m && iy >= 1 && iy <= m && iz >= 1 && (g.dim == 2 || iz <= m);
+      x[e] = ok ? (T)in[ix - 1 + m * (iy - 1) + (g.dim == 3 ? mm * (iz - 1) : 0)] : T(0);
+    }
+  } else {
+    for (int t = threadIdx.x; t < nm; t += kCoarseThreads) x[node(t)] = in[t];
+  }
+}
+
 constexpr int kSegThreads = 256;
 
 __global__ void seg_dot_kernel(Segments sg, const double* __restrict__ x, const double* __restrict__ y,
@@ -229,6 +279,24 @@ int launch_axis_op(const AxisOp& op, const T* in, T* out, const T* coef, cudaStr
 }
 template int launch_axis_op<double>(const AxisOp&, const double*, double*, const double*, cudaStream_t);
 template int launch_axis_op<float>(const AxisOp&, const float*, float*, const float*, cudaStream_t);
+
+// One CTA does 2 dim m multiply-adds per unknown at about two a clock, so the
+// line is drawn where that takes as long as the launches it saves.
+bool coarse_fd_fits(int dim, int m) {
+  const long long nm = (long long)m * m * (dim == 3 ? m : 1);
+  return m <= 64 && nm * m * 2 * dim <= 40000;
+}
+template <typename T>
+int launch_coarse_fd(const LevelGeom& g, int m, const double* fwd, const double* bwd, const double* dinv, const T* b,
+                     T* x, long long n_elems, cudaStream_t s) {
+  const size_t smem = 2 * ((size_t)m * m * (g.dim == 3 ? m : 1) + m * m) * sizeof(double);
+  coarse_fd_kernel<T><<<1, kCoarseThreads, smem, s>>>(g, m, fwd, bwd, dinv, b, x, n_elems);
+  return status();
+}
+template int launch_coarse_fd<double>(const LevelGeom&, int, const double*, const double*, const double*, const double*,
+                                      double*, long long, cudaStream_t);
+template int launch_coarse_fd<float>(const LevelGeom&, int, const double*, const double*, const double*, const float*,
+                                     float*, long long, cudaStream_t);
 
 template <typename T>
 int launch_dense_solve(const LevelGeom& g, const double* Ainv, int n_int, const T* b, T* x,
