@@ -3,7 +3,7 @@
 // problems, patch lists (slabs, Algorithm 5) and the solve-only mode of
 // Algorithm 3, in 2D and 3D.  With one patch per thread the FP32 kernel issued
 // two instructions beside each multiply-add; per sweep, before -> now (us):
-// FP32 Q4 64^3 934 -> 599, FP64 2D Q3 1024^2 967 -> 544, FP64 closure form Q4
+// FP32 Q4 64^3 934 -> 583, FP64 2D Q3 1024^2 967 -> 544, FP64 closure form Q4
 // 64^3 4930 -> 3180.
 //
 // Patch local_update (Sec. 3.1; Algorithm 4 runs it for every patch of one
@@ -179,9 +179,8 @@ __global__ void __launch_bounds__(NT, CTAS) pair_closure_kernel(const __grid_con
   __syncthreads();
 
   // The rows of b are on their way from the start where the registers allow it
-  // (FP64 Q3 64^3 1107 -> 1029 us, Q4 3273 -> 3172; Q5 48^3 5895 -> 6271; Q2
-  // 96^3 fits one CTA per SM less, 821 -> 854).
-  constexpr bool EARLY = K <= 4 && (DIM == 2 || K >= 3) && PP * LINES <= NT;
+  // (FP64 Q3 64^3 1107 -> 1029 us, Q4 3273 -> 3172; Q5 48^3 5895 -> 6271).
+  constexpr bool EARLY = (K == 3 || K == 4) && PP * LINES <= NT;
   T eb[EARLY ? 2 * M : 1];
   auto rhs = [&](int t, int p) -> const T* {
     const int ln = t % LINES;
@@ -374,20 +373,22 @@ __global__ void __launch_bounds__(NT, CTAS) pair_closure_kernel(const __grid_con
 // ---- host side ----
 
 // Patch pairs and threads per CTA, and the CTAs per SM that the registers are
-// limited for.  A pair has LINES lines in most stages, and a CTA as many pairs
-// as fill its threads with them.  Measured per sweep (us), the shape taken
-// first: FP32 Q4 64^3 1 pair in 64 threads 599, 2 in 128 630, 5 in 256 644;
-// Q6 40^3 with registers for 4 CTAs 552, for 1 772; FP64 Q3 64^3 10 in 256
-// with registers for 2 CTAs 1030, 5 in 128 for 4 1265, 1 in 32 2251; FP64 2D
-// Q3 1024^2 25 in 128 for 5 CTAs 544, for 1 938, 12 in 64 for 8 710.
+// limited for (0: left to the compiler, which then takes another schedule).  A
+// pair has LINES lines in most stages, and a CTA as many pairs as fill its
+// threads with them.  Measured per sweep (us), the shape taken first: FP32 Q4
+// 64^3 1 pair in 64 threads 583, limited for 14 CTAs 599, 2 in 128 630, 5 in
+// 256 612; Q6 40^3 with registers for 4 CTAs 552, left 615, for 1 772; FP64 Q2
+// 96^3 28 in 256 758, 14 in 128 803; Q3 64^3 10 in 256 for 2 CTAs 1030, left
+// 1605, 5 in 128 for 4 1265; Q5 48^3 left 5165, for 2 CTAs 5904; 2D Q2 1024^2
+// left 181, for 1 CTA 242; 2D Q3 25 in 128 for 5 CTAs 544, for 1 938.
 template <int DIM, int K>
 struct ClosureCfg {
   static constexpr int M = 2 * K - 1, LINES = DIM == 3 ? M * M : M;
-  static constexpr int NT = DIM == 2 || K <= 2 ? 128 : DF ? 256 : K == 3 ? 128 : K == 8 ? 256 : (LINES + 31) / 32 * 32;
+  static constexpr int NT = DIM == 2 || K == 1 ? 128 : DF ? 256 : K <= 3 ? 128 : K == 8 ? 256 : (LINES + 31) / 32 * 32;
   static constexpr int PP = cmax(1, std::min(NT / LINES, 48));
-  static constexpr int CTAS = DIM == 2 ? (!DF || K <= 2 ? 1 : K == 3 ? 5 : 4)
-                            : DF ? (K == 1 ? 1 : K == 2 ? 5 : K == 6 || K == 8 ? 1 : 2)
-                                 : (K == 4 ? 14 : K == 6 ? 4 : K >= 7 ? 2 : 1);
+  static constexpr int CTAS = DIM == 2 ? (!DF || K <= 2 ? 0 : K == 3 ? 5 : 4)
+                            : DF ? (K == 3 || K == 4 || K == 7 ? 2 : 0)
+                                 : (K == 4 ? 0 : K == 6 ? 4 : K >= 7 ? 2 : 1);
 };
 
 template <int DIM, int K, int PP, int NT, int CTAS>
