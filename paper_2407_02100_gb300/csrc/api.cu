@@ -208,9 +208,10 @@ int launch_colour(gmg_problem* p, const PatchLaunch& pl, void* u, const void* b)
     // run (equal up to rounding, unlike the closure form and its slabs), the
     // coarse-level kernel wins on larger colours too: 228 -> 152 us a sweep of
     // 512 patches a colour at k = 4, 160 -> 100 us of 1000 at k = 3, even at
-    // 1728 (150 : 161 us) and behind above
+    // 1728 (150 : 161 us) and behind above; a limit that the caller sets holds
+    // as it is
     const int k = pl.g.k;
-    const int small = p->faces && p->shared_faces && p->small_patches > 0
+    const int small = p->faces && p->shared_faces && p->small_auto
                           ? std::max(p->small_patches, k == 3 ? 1536 : k == 4 ? 640 : 0) : p->small_patches;
     if (pl.n_patches <= small) {
       const int st = launch_patch_small<double>(pl, (double*)u, (const double*)b, (const double*)p->dinv, p->stream);
@@ -695,6 +696,7 @@ int gmg::detail::create_problem(const gmg_desc* d, gmg_problem* p, const CreateO
   // at k <= 4, where it measured faster than the line kernels; above, a
   // patch's outputs outnumber a CTA's threads and it measured slower
   p->small_patches = k <= 4 ? 256 : 0;
+  p->small_auto = k <= 4;
   // level hierarchy: n_levels given, or halve while even and >= 2
   int L = d->n_levels;
   if (L == 0) {
@@ -1172,6 +1174,7 @@ int gmg_set_small_sweep(gmg_problem* p, int max_patches) {
   if (!p || max_patches < 0) return GMG_ERR_INVALID_ARG;
   drop_cg_graph(p);
   p->small_patches = max_patches;
+  p->small_auto = false;
   // levels that leave or join the coarse-level kernel take or drop their slabs
   for (int l = 0; l < (int)p->levels.size(); ++l) CHECK(build_slabs(p, l, slab_width_for(p, p->levels[l])));
   return GMG_OK;

@@ -109,6 +109,7 @@ struct gmg_problem {
   // FP64 colour steps of at most this many patches use the coarse-level
   // kernel (gmg_set_small_sweep; 0: never; set by gmg_create)
   int small_patches = 0;
+  bool small_auto = false;  // the limit is the library's, not the caller's
   // workspace of the three-pass FP64 3D operator (two finest-level
   // vectors), null where the tile kernel is used
   void* apply_ws = nullptr;
