@@ -55,19 +55,21 @@ FP64_PEAK_DERIVED_TFLOPS = 152 * 4 * 2.07e9 / 1e12
 # The FP64 sweep runs each colour as two launches, the face kernel and the
 # patch kernel (shared-face form), both in double-float arithmetic on the
 # FP32 pipe; "per launch" figures below are per colour step (both kernels).
-# From ncu over every launch of 7 sweeps of the current kernels at this
-# workload (profiles/face_sweep_fp64_q4_64.md), per average colour step of
+# A thread carries two patches in packed arithmetic: a packed instruction is
+# one issued instruction and two cycles of the FP32 pipe.  From ncu over every
+# launch of a sweep of the current kernels at this workload
+# (profiles/face_sweep_fp64_q4_64.md), per average colour step of
 # 31,256 patches: DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum)
 # and warp instructions issued (smsp__inst_executed.sum), face + patch kernel.
-TRAFFIC_PER_LAUNCH = (151.86e6 + 16.79e6) + (221.64e6 + 69.60e6)
-WARP_INST_PER_PATCH = (90.91e6 + 212.46e6) / (250047 / 8)
-EXECUTED_SOURCE = ("profiles/face_sweep_fp64_q4_64.md: ncu smsp__inst_executed.sum over every launch of 7 sweeps "
-                   "(face_kernel_df + patch_face_kernel), per patch")
+TRAFFIC_PER_LAUNCH = (153.86e6 + 18.47e6) + (219.91e6 + 70.64e6)
+WARP_INST_PER_PATCH = (40.46e6 + 112.15e6) / (250047 / 8)
+EXECUTED_SOURCE = ("profiles/face_sweep_fp64_q4_64.md: ncu smsp__inst_executed.sum over every launch of a sweep "
+                   "(face_pair_kernel + pair_sweep_kernel), per patch")
 # issue slots of GB300: 152 SMs x 4 schedulers, one warp instruction each per clock
 ISSUE_SLOTS_PER_CLOCK = 152 * 4
-# FP32 pipe activity of the two kernels (ncu --set full, one colour step each)
-PIPE_ACTIVE = {"face_kernel_df": {"fma": 0.468, "alu": 0.283, "issue": 0.697},
-               "patch_face_kernel": {"fma": 0.457, "alu": 0.232, "issue": 0.672}}
+# FP32 pipe and issue activity of the two kernels (ncu, averages over a sweep)
+PIPE_ACTIVE = {"face_pair_kernel": {"fma": 0.448, "issue": 0.440},
+               "pair_sweep_kernel": {"fma": 0.573, "issue": 0.516}}
 CPU_SAMPLE = dict(dim=3, degree=4, n_cells=8, n_levels=3)
 BLAS_THREAD_VARS = ("OMP_NUM_THREADS", "OPENBLAS_NUM_THREADS", "MKL_NUM_THREADS", "BLIS_NUM_THREADS")
 # further workloads of the method, measured in the same run (one timed solve each)
@@ -531,7 +533,7 @@ def run_ours(args):
                                                  "against the measured FP64 FMA peak; the kernels compute the sweep "
                                                  "in double-float arithmetic on the FP32 pipe with a regrouped "
                                                  "(banded, even/odd, shared-face) operation count"},
-                     "kernel": "face_kernel_df<4,128> + patch_face_kernel<4,256,5,1> (FP64 shared-face sweep in "
+                     "kernel": "face_pair_kernel<4> + pair_sweep_kernel<4> (FP64 shared-face sweep in packed "
                                "double-float arithmetic), one pair of launches per colour; timed as whole sweeps"},
         "cpu_baseline": cpu,
         "e2e": {"value": e2e_value, "unit": "MDoF/s", "h2d_bytes_per_step": n_elems * 8,

@@ -327,8 +327,8 @@ int gmg_batch_cg_solve(gmg_batch* b, double* u, const double* rhs, double rtol, 
                        int* iterations, double* rel_residual);
 
 /* Choose, by timing batched sweeps on the GPU, the number of patches per CTA
- * of the batched sweep kernel (0 = the default configuration, or 1, 2, 4;
- * the variants exist for 3D FP32 up to degree 4).  The choice never changes
+ * of the batched sweep kernel (0 = the default configuration, or 1, 2, 4; one
+ * is rounded up to a pair; the variants exist for 3D FP32 up to degree 4).  The choice never changes
  * results: every patch is computed the same way whatever the grouping.
  * *ppc_out (may be NULL) receives the choice. */
 int gmg_batch_autotune(gmg_batch* b, int* ppc_out);
@@ -497,7 +497,9 @@ int gmg_shared_faces(const gmg_problem* p);
  * and colour order; results agree with the other forms up to rounding.
  * Levels swept by it take no slab schedule.
  * gmg_set_small_sweep: max_patches >= 0 (0 turns the kernel off; gmg_create
- *   sets 256 for degrees up to 4 and 0 above); GMG_ERR_INVALID_ARG for a
+ *   sets 256 for degrees up to 4 and 0 above, and where the shared-face form
+ *   would take a larger colour, up to 1536 patches at degree 3 and 640 at
+ *   degree 4; a limit set here holds as it is); GMG_ERR_INVALID_ARG for a
  *   null problem or a negative count.  Single-precision and variable-
  *   coefficient problems ignore it.
  * gmg_small_sweep: the current max_patches, GMG_ERR_INVALID_ARG for a null
@@ -511,10 +513,10 @@ int gmg_small_sweep(const gmg_problem* p);
  * gmg_apply_operator(_f64), the V-cycle residuals of FP64 problems and the
  * FP64 CG of every problem) runs as three passes over the level, one 1D
  * contraction per axis with the
- * global 1D mass and stiffness matrices (z, then y, then x), through four
- * workspace vectors of the finest level (FP64, allocated by gmg_create).
- * Every output row is evaluated once; the tile kernel recomputes a halo of
- * up to k + 1 nodes per direction.  Same operator, results equal up to
+ * global 1D mass and stiffness matrices (z in one launch, y and x in another),
+ * through two workspace vectors of the finest level (FP64, allocated by
+ * gmg_create).  Only the y rows of a tile's left columns are evaluated twice;
+ * the tile kernel recomputes a halo of up to k + 1 nodes per direction.  Same operator, results equal up to
  * rounding.  If the workspace cannot be allocated the tile kernel is used.
  * gmg_set_three_pass_operator: enable (default) or disable the form (the
  *   workspace stays allocated); GMG_ERR_INVALID_ARG for a null problem.
@@ -530,13 +532,11 @@ int gmg_three_pass_operator(const gmg_problem* p);
  * fast-diagonalisation solve of App. A.3, scatter), with each 1D
  * contraction executed as a TF32 tcgen05 MMA over the lines of the patch
  * tensor.  Device-side waits are bounded: on the tensor cores' completion,
- * and on the TMA gathers of the sweep kernels (every sweep gathers a patch's
- * closure with one TMA box per vector when the vectors' base addresses are
- * 16-byte aligned and their pitches multiples of 16 bytes, else with one
- * cp.async per element).  An expired wait makes the kernel finish early and
- * set a device flag (one per device).  This covers every sweep kernel of the
- * library (gmg_smooth and its variants, gmg_smooth_noalloc, the V-cycle and
- * CG, batches, the variable-coefficient sweep) and the tensor-core sweep.
+ * and on the bulk copies of the sweep kernels that use them (the shared-face
+ * sweep: the faces and the interior of b; the variable-coefficient sweep with
+ * a learned correction: the closures of u and b; the other sweeps load straight
+ * to registers).  An expired wait makes the kernel finish early and set a
+ * device flag (one per device).
  * gmg_tc_status synchronises the device, returns GMG_OK or the recorded
  * status (GMG_ERR_TIMEOUT) of the current device and clears it. */
 int gmg_tc_status(void);
