@@ -81,13 +81,17 @@ __global__ void __launch_bounds__(128) pass_z_df_kernel(const double* __restrict
 // Passes y and x together on a tile of BX x BY cells of one z plane: A1 and A2
 // of the tile (with the K + 1 columns to its left) stay in shared memory, so
 // that four of the ten passes over level vectors are not made: Q4 64^3 403 ->
-// 367 us with pass z (140 us), Q3 51^3 121 -> 102.  Both launches are bound by the
+// 368 us with pass z (140 us), Q3 51^3 108 -> 91.  Both launches are bound by the
 // FP32 pipe (Dot2 terms of 10 operations); limits on the registers only made
-// them slower (Q4 3 CTAs per SM 403 us, Q7 32^3 2 CTAs 509 against 444).  The y
+// them slower (Q4 3 CTAs per SM 403 us, Q7 32^3 2 CTAs 509 against 444 with 9-cell tiles).  The y
 // rows are evaluated for ((BX + 1) K + 1) / (BX K) of the columns that are needed.
 template <int K>
 struct PlanePass {
-  static constexpr int BX = 64 / K, BY = 4, NT = 256;
+  // the widest tile whose columns with their halo, 4 cells high, take one round
+  // of the threads (Q7 48^3 1449 -> 1179 us, Q3 51^3 102 -> 91, against 64 / K
+  // cells); at K = 4 16 cells, which split the usual meshes evenly, are better
+  // than 14 (Q4 64^3 368 : 410 us)
+  static constexpr int BX = K == 4 ? 16 : (63 - K) / K, BY = 4, NT = 256;
   static constexpr int EX = (BX + 1) * K + 1, EY = BY * K;
   static constexpr int EXP = EX | 1;  // odd row: lanes of the x stage lie K entries apart
   static constexpr int BYTES = 2 * EY * EXP * (int)sizeof(float2);
