@@ -498,8 +498,8 @@ int gmg_shared_faces(const gmg_problem* p);
  * Levels swept by it take no slab schedule.
  * gmg_set_small_sweep: max_patches >= 0 (0 turns the kernel off; gmg_create
  *   sets 256 for degrees up to 4 and 0 above, and where the shared-face form
- *   would take a larger colour, up to 1536 patches at degree 3 and 640 at
- *   degree 4; a limit set here holds as it is); GMG_ERR_INVALID_ARG for a
+ *   would take a larger colour, up to 1536 patches at degree 3, 640 at
+ *   degree 4 and 128 above; a limit set here holds as it is); GMG_ERR_INVALID_ARG for a
  *   null problem or a negative count.  Single-precision and variable-
  *   coefficient problems ignore it.
  * gmg_small_sweep: the current max_patches, GMG_ERR_INVALID_ARG for a null

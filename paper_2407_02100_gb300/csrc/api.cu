@@ -208,11 +208,12 @@ int launch_colour(gmg_problem* p, const PatchLaunch& pl, void* u, const void* b)
     // run (equal up to rounding, unlike the closure form and its slabs), the
     // coarse-level kernel wins on larger colours too: 228 -> 152 us a sweep of
     // 512 patches a colour at k = 4, 160 -> 100 us of 1000 at k = 3, even at
-    // 1728 (150 : 161 us) and behind above; a limit that the caller sets holds
-    // as it is
+    // 1728 (150 : 161 us) and behind above; at k >= 5 while each patch has an SM
+    // to itself (us a sweep of 6^3: Q5 306 : 115, Q7 504 : 293, Q8 648 : 425);
+    // a limit that the caller sets holds as it is
     const int k = pl.g.k;
     const int small = p->faces && p->shared_faces && p->small_auto
-                          ? std::max(p->small_patches, k == 3 ? 1536 : k == 4 ? 640 : 0) : p->small_patches;
+                          ? std::max(p->small_patches, k == 3 ? 1536 : k == 4 ? 640 : k >= 5 ? 128 : 0) : p->small_patches;
     if (pl.n_patches <= small) {
       const int st = launch_patch_small<double>(pl, (double*)u, (const double*)b, (const double*)p->dinv, p->stream);
       if (st != GMG_ERR_UNSUPPORTED) return st;
@@ -696,7 +697,7 @@ int gmg::detail::create_problem(const gmg_desc* d, gmg_problem* p, const CreateO
   // at k <= 4, where it measured faster than the line kernels; above, a
   // patch's outputs outnumber a CTA's threads and it measured slower
   p->small_patches = k <= 4 ? 256 : 0;
-  p->small_auto = k <= 4;
+  p->small_auto = true;
   // level hierarchy: n_levels given, or halve while even and >= 2
   int L = d->n_levels;
   if (L == 0) {

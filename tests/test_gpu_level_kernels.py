@@ -79,8 +79,9 @@ def test_operator_2d(gmg, k, n):
     assert rel(P.from_device(y), m.assemble() @ x) < 1e-12
 
 
-# colours on both sides of the coarse-level kernel's line (1536 patches at k = 3, 640 at k = 4)
-@pytest.mark.parametrize("k,n", [(3, 13), (3, 24), (4, 14), (4, 18)])
+# colours on both sides of the coarse-level kernel's line (1536 patches at k = 3, 640 at k = 4, 128
+# above)
+@pytest.mark.parametrize("k,n", [(3, 13), (3, 24), (4, 14), (4, 18), (5, 4), (6, 11), (7, 5), (8, 3)])
 def test_mid_size_colours(gmg, k, n):
     out = []
     for kw in ({}, {"small_sweep": 0}):
