@@ -16,9 +16,11 @@ inline void split_pair(double v, float& hi, float& lo) {
 // that a sweep repeats everywhere with the same sign and a V-cycle then
 // amplifies.  So what a row of pairs is short of zero goes to its entries,
 // largest first, each taking the multiple of its own last place (2^-48 of
-// its binade) that comes nearest: no entry moves by more than half of the
-// last place of the next larger one, and what is left is below the last
-// place of the smallest.
+// its binade) that comes nearest.  The largest entry takes up what the FP64
+// row was short of zero itself and the rounding of every entry, at most
+// (cols + 1) / 2 of its last places in all; any other moves by at most half of
+// the last place of the next larger one and one of its own.  What is left is
+// below the last place of the smallest.
 inline void split_zero_sum_rows(const double* a, int rows, int cols, std::vector<float>& hi, std::vector<float>& lo) {
   hi.resize((size_t)rows * cols);
   lo.resize((size_t)rows * cols);
@@ -39,6 +41,33 @@ inline void split_zero_sum_rows(const double* a, int rows, int cols, std::vector
     }
     for (int c = 0; c < cols; ++c) split_pair(q[c], hi[(size_t)r * cols + c], lo[(size_t)r * cols + c]);
   }
+}
+
+// The interior rows of the two-cell patch matrix Kp (2k - 1 rows, 2k + 1
+// columns), as the sweeps read them: from the rows of the first cell alone, the
+// second cell being its mirror image.  The vertex row is that cell's last row
+// and its mirror image, which meet in the vertex entry, so it is split as the
+// cell's row, with half of the vertex entry; corrected as one row of 2k + 1
+// entries, mirrored ones would take different corrections, and the sum that is
+// applied, twice the left half and the vertex, would not be zero (k = 8: -7e-14,
+// -3e-14 split entry by entry).
+inline void split_patch_stiffness(const double* Kp, int k, std::vector<float>& hi, std::vector<float>& lo) {
+  const int C = 2 * k + 1, M = 2 * k - 1, n = k + 1;
+  std::vector<double> cell((size_t)k * n);  // rows 1..k of the first cell
+  for (int p = 0; p < k; ++p)
+    for (int q = 0; q < n; ++q) cell[(size_t)p * n + q] = Kp[p * C + q];
+  cell[(size_t)k * n - 1] *= 0.5;
+  std::vector<float> h, l;
+  split_zero_sum_rows(cell.data(), k, n, h, l);
+  hi.assign((size_t)M * C, 0.f);
+  lo.assign((size_t)M * C, 0.f);
+  for (int p = 0; p < k; ++p)
+    for (int q = 0; q < n; ++q) {
+      const float both = p == k - 1 && q == k ? 2.f : 1.f;  // the vertex entry, of both cells
+      const int o = p * C + q;
+      hi[o] = hi[M * C - 1 - o] = both * h[p * n + q];
+      lo[o] = lo[M * C - 1 - o] = both * l[p * n + q];
+    }
 }
 
 }  // namespace gmg

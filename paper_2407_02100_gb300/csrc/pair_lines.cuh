@@ -136,7 +136,7 @@ inline int pl_upload(int k, const double* Mp, const double* Kp, const double* Th
   const int C = 2 * k + 1, M = 2 * k - 1;
   std::vector<PA::tab> m(M * C), s(M * C), end(2 * M);
   std::vector<float> kh, kl;
-  split_zero_sum_rows(Kp, M, C, kh, kl);
+  split_patch_stiffness(Kp, k, kh, kl);
   float h, l;
   for (int i = 0; i < M * C; ++i) {
     split_pair(Mp[i], h, l);

@@ -138,7 +138,7 @@ static int upload(int k, const double* Mp, const double* Kp, const double* That,
     mhi[i] = (float)Mp[i];
     mlo[i] = (float)(Mp[i] - (double)mhi[i]);
   }
-  split_zero_sum_rows(Kp, M, C, khi, klo);
+  split_patch_stiffness(Kp, k, khi, klo);
   const size_t po = off_patch(k) * sizeof(float), pb = mhi.size() * sizeof(float);
   e = e == cudaSuccess ? cudaMemcpyToSymbol(c_Mphi, mhi.data(), pb, po) : e;
   e = e == cudaSuccess ? cudaMemcpyToSymbol(c_Mplo, mlo.data(), pb, po) : e;

@@ -53,3 +53,79 @@ def test_stiffness_rows_sum_to_zero_as_pairs(tmp_path):
                     os.path.join(CSRC, "setup.cpp"), "-o", str(exe)], check=True, capture_output=True)
     res = subprocess.run([str(exe)], capture_output=True, text=True, timeout=60)
     assert res.returncode == 0 and res.stdout == "ok\n", res.stdout
+
+
+# the sums of the two-cell rows as the two-patch kernels read them: a cell's
+# row for either cell, the vertex row as twice its left half and the vertex
+# entry, the end columns from the table of negated end entries.  Exact, in
+# units of 2^-90.  No entry may move by more than the header of coef_split.h
+# says: half of the last place of the next larger one and one of its own, the
+# largest by (k + 2) / 2 of its own, and what the FP64 row itself is short of
+# zero.
+PATCH = r'''
+#include "coef_split.h"
+#include "setup.h"
+#include <cstdio>
+using namespace gmg;
+typedef __int128 I;
+static I unit(float v) { return (I)std::ldexp((double)v, 90); }
+int main() {
+  for (int k = 1; k <= 8; ++k) {
+    const int C = 2 * k + 1, M = 2 * k - 1;
+    std::vector<double> Mp, Kp;
+    assembled_1d(k, 2, 1, M, 0, C, Mp, Kp);
+    std::vector<float> h, l;
+    split_patch_stiffness(Kp.data(), k, h, l);
+    auto pair = [&](int i, int c) { return unit(h[i * C + c]) + unit(l[i * C + c]); };
+    for (int i = 0; i < k; ++i) {  // row i, from its left half
+      I sum = 0;
+      for (int c = 0; c <= k; ++c) sum += pair(i, c) * (i == k - 1 && c < k ? 2 : 1);
+      if (sum != 0) { std::printf("sum %d %d %g\n", k, i, std::ldexp((double)sum, -90)); return 1; }
+    }
+    for (int i = 0; i < M; ++i) {
+      I whole = 0;
+      for (int c = 0; c < C; ++c) whole += pair(i, c);
+      if (whole != 0) { std::printf("whole row %d %d\n", k, i); return 1; }
+      for (int c = 0; c < C; ++c)
+        if (h[i * C + c] != h[(M - 1 - i) * C + C - 1 - c] || l[i * C + c] != l[(M - 1 - i) * C + C - 1 - c]) {
+          std::printf("mirror %d %d %d\n", k, i, c);
+          return 1;
+        }
+    }
+    for (int i = 0; i < k; ++i) {
+      std::vector<double> row(k + 1);
+      double defect = 0;
+      for (int c = 0; c <= k; ++c) {
+        row[c] = Kp[i * C + c] * (i == k - 1 && c == k ? 0.5 : 1.0);
+        defect += row[c];
+      }
+      auto place = [&](double v) { return std::ldexp(1.0, std::ilogb(v) - 48); };
+      for (int c = 0; c <= k; ++c) {
+        double next = 0;  // the next larger entry
+        for (int d = 0; d <= k; ++d)
+          if (d != c && std::fabs(row[d]) >= std::fabs(row[c]) && (next == 0 || std::fabs(row[d]) < next)) next = std::fabs(row[d]);
+        const double both = i == k - 1 && c == k ? 2.0 : 1.0;
+        const double q = ((double)h[i * C + c] + (double)l[i * C + c]) / both;
+        const double bound = next == 0 ? (k + 2) / 2.0 * place(row[c]) + std::fabs(defect) + 1e-15 * std::fabs(row[c])
+                                       : place(next) / 2 + place(row[c]);
+        if (!(std::fabs(q - row[c]) <= bound)) { std::printf("entry %d %d %d: %g above %g\n", k, i, c, q - row[c], bound); return 1; }
+        if (!(std::fabs(l[i * C + c]) <= std::ldexp(std::fabs(h[i * C + c]), -24))) { std::printf("pair %d %d %d\n", k, i, c); return 1; }
+      }
+    }
+  }
+  std::printf("ok\n");
+  return 0;
+}
+'''
+
+
+def test_patch_rows_sum_to_zero_as_the_sweeps_read_them(tmp_path):
+    gxx = shutil.which("g++")
+    if not gxx:
+        pytest.skip("needs g++")
+    src, exe = tmp_path / "patch.cpp", tmp_path / "patch"
+    src.write_text(PATCH)
+    subprocess.run([gxx, "-std=c++17", "-O2", "-ffp-contract=off", f"-I{CSRC}", "-I/usr/local/cuda/include", str(src),
+                    os.path.join(CSRC, "setup.cpp"), "-o", str(exe)], check=True, capture_output=True)
+    res = subprocess.run([str(exe)], capture_output=True, text=True, timeout=60)
+    assert res.returncode == 0 and res.stdout == "ok\n", res.stdout
