@@ -114,6 +114,10 @@ int upload_patch_tables(int k, const double* Mp, const double* Kp, const double*
 // tables of the closure form of the sweep (called by upload_patch_tables)
 template <typename T>
 int upload_closure_tables(int k, const double* Mp, const double* Kp, const double* That);
+// the form with one patch per thread of FP64 problems (pair_solo_f64.cu); fills
+// the table's group ranges
+int upload_closure_solo_tables(int k, const double* Mp, const double* Kp, const double* That);
+int launch_closure_solo(int dim, int k, PatchTable& tab, const double* dinv, cudaStream_t s);
 template <typename T>
 int launch_patch_colour(const PatchLaunch& pl, T* u, const T* b, const T* dinv, cudaStream_t s);
 // one colour of a coarse level with the one-output-per-thread kernel (FP64 problems,

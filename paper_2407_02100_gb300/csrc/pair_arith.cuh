@@ -105,9 +105,12 @@ __device__ __forceinline__ void df2_acc_add(df2_acc& a, df2_coef c, df2 x) {
 }
 __device__ __forceinline__ df2 df2_acc_value(df2_acc a) { return df2_norm(a.s, a.e); }
 
-// The two arithmetics of the pair kernels, under the same names: a value, an
-// accumulator, a coefficient and their forms in shared and constant memory.
+// The arithmetics of the pair kernels, under the same names: a value, an
+// accumulator, a coefficient and their forms in shared and constant memory, and
+// the patches W that a thread carries.  SoloDF does the operations of a lane of
+// PairDF in the same order, bit for bit.
 struct PairDF {  // double-float (FP64 problems)
+  static constexpr int W = 2;
   using T = double;
   using val = df2;
   using acc = df2_acc;
@@ -147,7 +150,39 @@ struct PairDF {  // double-float (FP64 problems)
   static __device__ __forceinline__ T x(val v) { return df_to_double(df2_x(v)); }
   static __device__ __forceinline__ T y(val v) { return df_to_double(df2_y(v)); }
 };
+struct SoloDF {  // double-float, one patch
+  static constexpr int W = 1;
+  using T = double;
+  using val = dfv;
+  using acc = df_acc;
+  struct coef {
+    float h, l;
+  };
+  using mem = float2;  // (hi, lo)
+  using tab = float2;  // (h, l)
+  static __device__ __forceinline__ val load(const mem& a) { return {a.x, a.y}; }
+  static __device__ __forceinline__ void store(mem& a, val v) { a = make_float2(v.hi, v.lo); }
+  static __device__ __forceinline__ coef coefficient(const tab& c) { return {c.x, c.y}; }
+  static __device__ __forceinline__ coef weight(const mem& a) { return {a.x, a.y}; }
+  static void make_tab(tab& c, double, float h, float l) { c = make_float2(h, l); }
+  static __device__ __forceinline__ acc zero() { return {0.f, 0.f}; }
+  static __device__ __forceinline__ acc first(coef c, val x) { return df_acc_first(c.h, c.l, x); }
+  static __device__ __forceinline__ void add(acc& a, coef c, val x) { df_acc_add(a, c.h, c.l, x); }
+  static __device__ __forceinline__ val value(acc a) { return df_acc_value(a); }
+  static __device__ __forceinline__ val sum(val a, val b) { return df_add(a, b); }
+  static __device__ __forceinline__ val diff(val a, val b) { return df_add(a, df_neg(b)); }
+  static __device__ __forceinline__ acc scaled(float c, val x) { return df_acc_scaled(c, x); }
+  static __device__ __forceinline__ val pack(T a, T) { return df_from_double(a); }
+  static __device__ __forceinline__ val pack_neg(T a, T) { return df_neg(df_from_double(a)); }
+  static __device__ __forceinline__ val diagonal(const T* dinv, int n, int i, val v) {
+    const float2 d = __ldg(reinterpret_cast<const float2*>(dinv + n) + i);
+    return value(first({d.x, d.y}, v));
+  }
+  static __device__ __forceinline__ T x(val v) { return df_to_double(v); }
+  static __device__ __forceinline__ T y(val v) { return df_to_double(v); }
+};
 struct PairF32 {  // single precision
+  static constexpr int W = 2;
   using T = float;
   using val = f2;
   using acc = f2;

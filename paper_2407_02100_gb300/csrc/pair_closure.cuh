@@ -1,10 +1,9 @@
-// Closure form of the patch sweep, two patches per thread (pair_arith.cuh),
-// for the arithmetic PA of the including file: whole colours, batches of
-// problems, patch lists (slabs, Algorithm 5) and the solve-only mode of
-// Algorithm 3, in 2D and 3D.  With one patch per thread the FP32 kernel issued
+// Closure form of the patch sweep, PA::W patches per thread (pair_arith.cuh: two,
+// or one where that is faster, see SoloCfg), for the arithmetic PA of the
+// including file: whole colours, batches of problems, patch lists (slabs,
+// Algorithm 5) and the solve-only mode of Algorithm 3, in 2D and 3D.  With one patch per thread the FP32 kernel issued
 // two instructions beside each multiply-add; per sweep, before -> now (us):
-// FP32 Q4 64^3 934 -> 583, FP64 2D Q3 1024^2 967 -> 544, FP64 closure form Q4
-// 64^3 4930 -> 3180.
+// FP32 Q4 64^3 934 -> 583, FP64 closure form Q4 64^3 4930 -> 3180.
 //
 // Patch local_update (Sec. 3.1; Algorithm 4 runs it for every patch of one
 // colour per launch):
@@ -37,7 +36,7 @@ constexpr bool DF = sizeof(T) == 8;
 
 __host__ __device__ constexpr int cmax(int a, int b) { return a > b ? a : b; }
 
-// Shared memory per pair, entries of E: the two fields of the first
+// Shared memory per pair (one patch with W = 1), entries of E: the two fields of the first
 // contraction, in rows of R entries.  Every later stage works in place: a
 // thread reads the whole line it writes.  u and b go from global memory
 // straight to registers (lanes along x): without room for the closures more
@@ -125,8 +124,9 @@ __device__ __forceinline__ void closure_line_residual(G&& get1, H&& get2, PA::ac
   }
 }
 
-// One colour of the sweep.  A CTA takes one group of 2 PP consecutive patches
-// of a table entry; a thread carries the same line of patches 2q and 2q + 1.
+// One colour of the sweep.  A CTA takes one group of W PP consecutive patches
+// of a table entry; a thread carries the same line of patches 2q and 2q + 1
+// (W = 2; the text below says pair for what a thread carries).
 // Small CTAs, several to an SM, overlap one another's loads and barriers, and
 // the hardware hands them out as SMs become free (persistent CTAs with a fixed
 // share: 0.63 against 0.60 ms per FP32 Q4 64^3 sweep).  The last contraction runs along the slowest
@@ -149,11 +149,11 @@ __global__ void __launch_bounds__(NT, CTAS) pair_closure_kernel(const __grid_con
                                                                 const T* __restrict__ dinv) {
   constexpr bool EXACT = DF && DIM == 3;
   using Z = ClosureSmem<DIM, K>;
-  constexpr int C = Z::C, M = Z::M, R = Z::R, F = Z::F, NP = 2 * PP;
+  constexpr int C = Z::C, M = Z::M, R = Z::R, F = Z::F, W = PA::W, NP = W * PP;
   constexpr int LINES = DIM == 3 ? M * M : M;  // interior lines per axis
   static_assert(NP <= NT, "one thread sets up one patch");
   extern __shared__ __align__(128) unsigned char smem_raw[];
-  E* const W = reinterpret_cast<E*>(smem_raw);  // [PP][2][F]
+  E* const S = reinterpret_cast<E*>(smem_raw);  // [PP][2][F]
   __shared__ long long s_origin[NP];
   const int mode = tab.mode, grp = blockIdx.x;
   int entry = 0, hi = tab.n - 1;  // last table entry with group_begin <= grp
@@ -163,7 +163,7 @@ __global__ void __launch_bounds__(NT, CTAS) pair_closure_kernel(const __grid_con
     else hi = mid - 1;
   }
   const PatchEntry& e = tab.e[entry];
-  const int g = grp - e.group_begin, nv = min(NP, e.n_patches - g * NP), npair = (nv + 1) / 2;
+  const int g = grp - e.group_begin, nv = min(NP, e.n_patches - g * NP), npair = (nv + W - 1) / W;
   T* const u = static_cast<T*>(e.u);
   const T* __restrict__ const b = static_cast<const T*>(e.b);
   const long long py = e.py, pz = e.pz, ps = DIM == 3 ? pz : py;  // ps: the slowest axis
@@ -184,14 +184,14 @@ __global__ void __launch_bounds__(NT, CTAS) pair_closure_kernel(const __grid_con
   T eb[EARLY ? 2 * M : 1];
   auto rhs = [&](int t, int p) -> const T* {
     const int ln = t % LINES;
-    return b + s_origin[2 * (t / LINES) + p] + 1 + ln % M + (DIM == 3 ? py * (1 + ln / M) : 0) + ps;
+    return b + s_origin[W * (t / LINES) + p] + 1 + ln % M + (DIM == 3 ? py * (1 + ln / M) : 0) + ps;
   };
   if constexpr (EARLY) {
     const int t = (int)threadIdx.x < npair * LINES ? threadIdx.x : 0;
 #pragma unroll
     for (int l = 0; l < M; ++l) {
       eb[l] = __ldg(rhs(t, 0) + ps * l);
-      eb[M + l] = __ldg(rhs(t, 1) + ps * l);
+      eb[M + l] = __ldg(rhs(t, W - 1) + ps * l);
     }
   }
   if (mode == 0) {
@@ -221,8 +221,8 @@ __global__ void __launch_bounds__(NT, CTAS) pair_closure_kernel(const __grid_con
           x = t % (C * C) % C;
           z = t % (C * C) / C;
         }
-        const T *const ua = u + s_origin[2 * q] + x + pz * z, *const ub = u + s_origin[2 * q + 1] + x + pz * z;
-        E* const P = W + q * 2 * F + z * M * R + x;
+        const T *const ua = u + s_origin[W * q] + x + pz * z, *const ub = u + s_origin[W * q + W - 1] + x + pz * z;
+        E* const P = S + q * 2 * F + z * M * R + x;
         auto get = [&](int y) -> V { return PA::pack_neg(ua[py * y], ub[py * y]); };
         auto put = [&](int j, V m, V k) {
           PA::store(P[j * R], m);
@@ -254,7 +254,7 @@ __global__ void __launch_bounds__(NT, CTAS) pair_closure_kernel(const __grid_con
       __syncthreads();
       // ---- x: A1 = M_x P, A2 = K_x P + M_x Q on rows (y, z), in place ----
       for (int t = threadIdx.x; t < npair * C * M; t += NT) {
-        E* const P = W + t / (C * M) * 2 * F + t % (C * M) * R;
+        E* const P = S + t / (C * M) * 2 * F + t % (C * M) * R;
         V a1[M], a2[M];
         closure_line2<K>([&](int x) -> V { return PA::load(P[x]); }, [&](int x) -> V { return PA::load(P[F + x]); },
                          [&](int i, V m, V k) {
@@ -271,8 +271,8 @@ __global__ void __launch_bounds__(NT, CTAS) pair_closure_kernel(const __grid_con
       // ---- x: P = M_x u, Q = K_x u on rows y, from -u ----
       for (int t = threadIdx.x; t < npair * C; t += NT) {
         const int q = t / C, y = t % C;
-        const T *const ua = u + s_origin[2 * q] + py * y, *const ub = u + s_origin[2 * q + 1] + py * y;
-        E* const P = W + q * 2 * F + y * R;
+        const T *const ua = u + s_origin[W * q] + py * y, *const ub = u + s_origin[W * q + W - 1] + py * y;
+        E* const P = S + q * 2 * F + y * R;
         closure_line<K>([&](int x) -> V { return PA::pack_neg(ua[x], ub[x]); },
                         [&](int i, V m, V k) {
                           PA::store(P[i], m);
@@ -286,10 +286,10 @@ __global__ void __launch_bounds__(NT, CTAS) pair_closure_kernel(const __grid_con
   // ---- residual on interior lines of the slowest axis (z in 3D, y in 2D),
   // then the forward transform along it, in place of the first field ----
   constexpr int SL = DIM == 3 ? M * R : R;  // stride of the line in W
-  auto line = [&](int q, int ln) -> E* { return W + q * 2 * F + (DIM == 3 ? ln / M * R + ln % M : ln); };
+  auto line = [&](int q, int ln) -> E* { return S + q * 2 * F + (DIM == 3 ? ln / M * R + ln % M : ln); };
   for (int t = threadIdx.x; t < npair * LINES; t += NT) {
     const int q = t / LINES, ln = t % LINES;  // 3D: x + M y; 2D: x
-    const T *const ba = rhs(t, 0), *const bb = rhs(t, 1);
+    const T *const ba = rhs(t, 0), *const bb = rhs(t, W - 1);
     PA::acc acc[M];
 #pragma unroll
     for (int l = 0; l < M; ++l) {
@@ -312,7 +312,7 @@ __global__ void __launch_bounds__(NT, CTAS) pair_closure_kernel(const __grid_con
   auto line_y = [&](auto forward) {
     for (int t = threadIdx.x; t < npair * LINES; t += NT) {
       const int q = t / LINES, ln = t % LINES;
-      E* const w = W + q * 2 * F + ln % M + ln / M * M * R;
+      E* const w = S + q * 2 * F + ln % M + ln / M * M * R;
       V v[M];
 #pragma unroll
       for (int j = 0; j < M; ++j) v[j] = PA::load(w[j * R]);
@@ -325,7 +325,7 @@ __global__ void __launch_bounds__(NT, CTAS) pair_closure_kernel(const __grid_con
   if (DIM == 3) line_y(std::true_type());
   for (int t = threadIdx.x; t < npair * LINES; t += NT) {
     const int q = t / LINES, ln = t % LINES;  // 3D: y + M z; 2D: y
-    E* const w = W + q * 2 * F + ln * R;
+    E* const w = S + q * 2 * F + ln * R;
     V v[M];
 #pragma unroll
     for (int i = 0; i < M; ++i) v[i] = PA::load(w[i]);
@@ -346,9 +346,9 @@ __global__ void __launch_bounds__(NT, CTAS) pair_closure_kernel(const __grid_con
     V v[M];
 #pragma unroll
     for (int l = 0; l < M; ++l) v[l] = PA::load(w[l * SL]);
-    const bool two = 2 * q + 1 < nv;
+    const bool two = W == 2 && 2 * q + 1 < nv;
     const long long ofs = 1 + ln % M + (DIM == 3 ? py * (1 + ln / M) : 0) + ps;
-    T *const ga = u + s_origin[2 * q] + ofs, *const gb = u + s_origin[2 * q + 1] + ofs;
+    T *const ga = u + s_origin[W * q] + ofs, *const gb = u + s_origin[W * q + W - 1] + ofs;
     if (EXACT && fresh) {
       pl_backward<K>(v, [&](int l, V d) {
         ga[ps * l] = PA::x(d);
@@ -379,16 +379,52 @@ __global__ void __launch_bounds__(NT, CTAS) pair_closure_kernel(const __grid_con
 // 64^3 1 pair in 64 threads 583, limited for 14 CTAs 599, 2 in 128 630, 5 in
 // 256 612; Q6 40^3 with registers for 4 CTAs 552, left 615, for 1 772; FP64 Q2
 // 96^3 28 in 256 758, 14 in 128 803; Q3 64^3 10 in 256 for 2 CTAs 1030, left
-// 1605, 5 in 128 for 4 1265; Q5 48^3 left 5165, for 2 CTAs 5904; 2D Q2 1024^2
-// left 181, for 1 CTA 242; 2D Q3 25 in 128 for 5 CTAs 544, for 1 938.
+// 1605, 5 in 128 for 4 1265; Q5 48^3 left 5165, for 2 CTAs 5904; 2D Q7 320^2 9
+// in 128 for 4 CTAs 874, left 935; Q8 320^2 8 in 128 for 4 1392, left 1783.
 template <int DIM, int K>
 struct ClosureCfg {
   static constexpr int M = 2 * K - 1, LINES = DIM == 3 ? M * M : M;
   static constexpr int NT = DIM == 2 || K == 1 ? 128 : DF ? 256 : K <= 3 ? 128 : K == 8 ? 256 : (LINES + 31) / 32 * 32;
   static constexpr int PP = cmax(1, std::min(NT / LINES, 48));
-  static constexpr int CTAS = DIM == 2 ? (!DF || K <= 2 ? 0 : K == 3 ? 5 : 4)
+  static constexpr int CTAS = DIM == 2 ? (DF ? 4 : 0)
                             : DF ? (K == 3 || K == 4 || K == 7 ? 2 : 0)
                                  : (K == 4 ? 0 : K == 6 ? 4 : K >= 7 ? 2 : 1);
+};
+
+// FP64, one patch per thread (SoloDF), the same results bit for bit: shapes and
+// the largest launch (patches) that takes it.  Two patches per thread halve the
+// issue slots of a chip that is full; on a small colour they only lengthen each
+// thread's chain, fill half of the CTAs and, on the longer lines, spill.  As many
+// patches as fill the threads with the lines of the first stage.  Measured per
+// sweep (us), two patches -> one, for colours of the stated patches: 3D Q1 512
+// 76 -> 49 (32768: 82 -> 80); Q2 512 130 -> 66, 8000 131 -> 101 (13824: 163 ->
+// 153); Q3 64 149 -> 83, 1728 154 -> 105, 8000 316 -> 299 (13824: 476 both, 10 per
+// CTA 429); Q4 64 226 -> 115, 1728 271 -> 245 (2744: 312 -> 349); Q5 64 305 -> 213,
+// 512 312 -> 217 (729: 312 -> 322); Q6 216 460 -> 328 (729: 677 -> 674); Q7 64 549
+// -> 404 (216: 542 -> 606); Q8 216 690 -> 559, 1728 4080 -> 3279.  2D Q2 400 41 ->
+// 25; Q3 262144 544 -> 460; Q5 25 115 -> 58, 25600 323 -> 263, 262144 3223 -> 2725;
+// Q6 25600 447 -> 448; Q7 400 246 -> 123, 6400 271 -> 270 (9216: 317 -> 403); Q8
+// 1600 306 -> 168 (3600: 314 -> 345).
+template <int DIM, int K>
+struct SoloCfg {
+  static constexpr int C = 2 * K + 1;
+  static constexpr int NT = DIM == 3 && (K == 3 || K >= 7) ? 256 : DIM == 3 && K == 4 ? 192 : 128;
+  static constexpr int PP = cmax(1, NT / (DIM == 3 ? C * C : C));
+  static constexpr bool ALWAYS = DIM == 2 && K <= 6;
+  static constexpr int LIMIT = DIM == 2 ? (K == 7 ? 6400 : 3000)
+                             : K == 1 ? 32768 : K == 2 ? 10000 : K == 3 ? 12000 : K == 5 ? 600 : K == 6 ? 1000
+                             : K == 7 ? 152 : 2000;
+};
+// FP32 on small colours: as many threads as the first stage of a pair has lines
+// in 3D from degree 5, where each pair has an SM to itself (Q5 8^3 66 -> 49, Q6 82
+// -> 66, Q7 98 -> 82, Q8 115 -> 98 us a sweep), CTAs of one warp in 2D (Q3 20^2 25
+// -> 17, Q6 33 -> 25, Q8 41 -> 33; equal above 1600 patches).
+template <int DIM, int K>
+struct SmallCfg {
+  static constexpr int C = 2 * K + 1;
+  static constexpr int NT = DIM == 3 ? (C * C + 31) / 32 * 32 : 32;
+  static constexpr int PP = DIM == 3 ? 1 : cmax(1, 28 / C);
+  static constexpr int LIMIT = DIM == 3 ? (K >= 5 ? 304 : 0) : K >= 2 ? 1600 : 0;
 };
 
 template <int DIM, int K, int PP, int NT, int CTAS>
@@ -407,7 +443,7 @@ int closure_launch(PatchTable& tab, const T* dinv, cudaStream_t s) {
   int groups = 0;
   for (int i = 0; i < tab.n; ++i) {
     tab.e[i].group_begin = groups;
-    groups += (tab.e[i].n_patches + 2 * PP - 1) / (2 * PP);
+    groups += (tab.e[i].n_patches + PA::W * PP - 1) / (PA::W * PP);
   }
   tab.total_groups = groups;
   if (groups <= 0) return GMG_OK;
@@ -425,7 +461,20 @@ int closure_table(PatchTable& tab, const T* dinv, int ppc, cudaStream_t s) {
     if (ppc == 2) return closure_launch<DIM, K, 1, 64, 1>(tab, dinv, s);
     if (ppc == 4) return closure_launch<DIM, K, 2, 128, 1>(tab, dinv, s);
   }
-  return closure_launch<DIM, K, Cfg::PP, Cfg::NT, Cfg::CTAS>(tab, dinv, s);
+  long long patches = 0;
+  for (int i = 0; i < tab.n; ++i) patches += tab.e[i].n_patches;
+  if constexpr (DF) {
+    using Solo = SoloCfg<DIM, K>;
+    if (Solo::ALWAYS || patches <= Solo::LIMIT)
+      return launch_closure_solo(DIM, K, tab, reinterpret_cast<const double*>(dinv), s);
+    if constexpr (!Solo::ALWAYS) return closure_launch<DIM, K, Cfg::PP, Cfg::NT, Cfg::CTAS>(tab, dinv, s);
+  } else {
+    using Small = SmallCfg<DIM, K>;
+    if constexpr (Small::LIMIT > 0) {
+      if (patches <= Small::LIMIT) return closure_launch<DIM, K, Small::PP, Small::NT, 0>(tab, dinv, s);
+    }
+    return closure_launch<DIM, K, Cfg::PP, Cfg::NT, Cfg::CTAS>(tab, dinv, s);
+  }
 }
 
 }  // namespace

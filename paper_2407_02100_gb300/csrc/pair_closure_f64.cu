@@ -26,7 +26,8 @@ int table_launches(const PatchLaunch* pls, T* const* us, const T* const* bs, int
 
 template <>
 int upload_closure_tables<double>(int k, const double* Mp, const double* Kp, const double* That) {
-  return pl_upload(k, Mp, Kp, That);
+  const int st = pl_upload(k, Mp, Kp, That);
+  return st != GMG_OK ? st : upload_closure_solo_tables(k, Mp, Kp, That);
 }
 
 template <>

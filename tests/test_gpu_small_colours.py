@@ -1,0 +1,43 @@
+"""Closure-form sweep on both sides of the lines between its kernels.
+
+A launch of few patches takes one patch per thread (FP64) or more threads per
+pair (FP32), a large one two patches per thread.  Every patch is to come out the
+same bit for bit, whichever kernel takes it: the sizes are whole colours above
+the line, the same sweep by slabs of one vertex row stays below it, and a slab
+schedule gives each patch exactly the values that the whole colours give it.
+"""
+import numpy as np
+import pytest
+
+from paper_2407_02100_gb300 import inputs
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def gmg():
+    from paper_2407_02100_gb300 import build, gmg as g
+    build.build()
+    return g
+
+
+def sweep(gmg, dim, k, n, precision, slab, reverse):
+    P = gmg.Problem(dim, k, n, precision=precision, small_sweep=0)
+    gmg.gmg_set_shared_faces(P.h, False)
+    gmg.gmg_set_slab_width(P.h, slab)
+    assert gmg.gmg_slab_width(P.h, P.finest) == slab
+    u = P.to_device(inputs.random_nodal(dim, k, n, 51 + k))
+    gmg.gmg_smooth(P.h, P.finest, u, P.to_device(inputs.random_nodal(dim, k, n, 52 + n)), 1, reverse)
+    out = P.from_device(u)
+    P.close()
+    return out
+
+
+@pytest.mark.parametrize("dim,k,n,precision", [
+    (3, 2, 46, 0), (3, 3, 48, 0), (3, 4, 26, 0), (3, 5, 18, 0), (3, 6, 22, 0), (3, 7, 12, 0), (3, 8, 26, 0),
+    (2, 7, 256, 0), (2, 8, 112, 0),
+    (3, 5, 14, 1), (3, 6, 14, 1), (3, 7, 14, 1), (3, 8, 14, 1), (2, 2, 84, 1), (2, 4, 84, 1), (2, 7, 84, 1), (2, 8, 84, 1)])
+def test_whole_colours_and_slabs_agree_bit_for_bit(gmg, dim, k, n, precision):
+    whole = sweep(gmg, dim, k, n, precision, 0, k % 2 == 1)
+    assert np.array_equal(whole, sweep(gmg, dim, k, n, precision, 1, k % 2 == 1))
+    assert np.isfinite(whole).all()
