@@ -534,9 +534,9 @@ int gmg_three_pass_operator(const gmg_problem* p);
  * tensor.  Device-side waits are bounded: on the tensor cores' completion,
  * and on the bulk copies of the sweep kernels that use them (the shared-face
  * sweep: the faces and the interior of b; the variable-coefficient sweep with
- * a learned correction: the closures of u and b; the other sweeps load straight
- * to registers).  An expired wait makes the kernel finish early and set a
- * device flag (one per device).
+ * a learned correction, or of small FP64 3D colours: the closures of u and b;
+ * the other sweeps load straight to registers).  An expired wait makes the
+ * kernel finish early and set a device flag (one per device).
  * gmg_tc_status synchronises the device, returns GMG_OK or the recorded
  * status (GMG_ERR_TIMEOUT) of the current device and clears it. */
 int gmg_tc_status(void);

@@ -167,7 +167,7 @@ template <typename T>
 int launch_patch_var(const PatchLaunch& pl, T* u, const T* b, const T* coef, const T* vscale, const T* dinv,
                      const float* corr, int rank, cudaStream_t s);
 
-// the same without a correction, two patches per thread (pair_var.cuh)
+// the same without a correction (pair_var.cuh)
 template <typename T>
 int upload_var_pair_tables(int k, const double* Mc, const double* Kc, const double* That);
 template <typename T>

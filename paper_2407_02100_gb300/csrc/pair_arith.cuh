@@ -128,8 +128,6 @@ struct PairDF {  // double-float (FP64 problems)
     const ulonglong2 v = reinterpret_cast<const ulonglong2&>(c);
     return {{v.x}, {v.y}};
   }
-  // a pair of values as a coefficient (one per patch)
-  static __device__ __forceinline__ coef weight(const mem& a) { return coefficient(a); }
   static void make_tab(tab& c, double, float h, float l) { c = make_float4(h, h, l, l); }
   static __device__ __forceinline__ acc zero() { return {{0}, {0}}; }
   static __device__ __forceinline__ acc first(coef c, val x) { return df2_acc_first(c, x); }
@@ -163,6 +161,7 @@ struct SoloDF {  // double-float, one patch
   static __device__ __forceinline__ val load(const mem& a) { return {a.x, a.y}; }
   static __device__ __forceinline__ void store(mem& a, val v) { a = make_float2(v.hi, v.lo); }
   static __device__ __forceinline__ coef coefficient(const tab& c) { return {c.x, c.y}; }
+  // a value as a coefficient (of its patch)
   static __device__ __forceinline__ coef weight(const mem& a) { return {a.x, a.y}; }
   static void make_tab(tab& c, double, float h, float l) { c = make_float2(h, l); }
   static __device__ __forceinline__ acc zero() { return {0.f, 0.f}; }

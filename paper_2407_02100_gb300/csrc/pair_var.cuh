@@ -1,6 +1,7 @@
-// Variable-coefficient patch sweep (degree <= 3), two patches per thread
-// (pair_arith.cuh), for the arithmetic PA of the including file; patches
-// without a learned correction (those with one take patch_var_kernel).
+// Variable-coefficient patch sweep (degree <= 3), PA::W patches per thread
+// (pair_arith.cuh: two in FP32, one in FP64), for the arithmetic PA of the
+// including file; patches without a learned correction (those with one take
+// patch_var_kernel).
 //
 // One colour of Algorithm 4: the local residual is evaluated cell by cell
 // with the cell coefficients (Sec. 3.1, eq. "main:4"), the local solver is the
@@ -48,7 +49,7 @@ __device__ __forceinline__ void var_row(int p, const V (&x)[K + 1], PA::acc& acc
   }
 }
 
-// Shared memory per pair: the two fields of a contraction, [z][y][x] with 2k
+// Shared memory per pair (one patch in FP64): the two fields of a contraction, [z][y][x] with 2k
 // rows per contracted axis; stages work in place.  u and b go from global
 // memory straight to registers (lanes along x): without room for them twice
 // as many CTAs fit on an SM, which overlap one another's loads and barriers.
@@ -71,8 +72,8 @@ struct VarArgs {
   const T* dinv;
 };
 
-// A CTA takes 2 PP consecutive patches of the colour, a thread the same line
-// of patches 2q and 2q + 1.  Stages, 3D (2D: without the first, and y for z):
+// A CTA takes W PP consecutive patches of the colour, a thread the same line
+// of patches 2q and 2q + 1 (W = 2).  Stages, 3D (2D: without the first, and y for z):
 //   y: P, Q (on -u), 2k rows | x: A1, A2, 2k rows each way |
 //   z: a_c (K_z A1 + M_z A2) per column of a cell pair |
 //   z: r = h^{2-d} b + the columns of a node (1, 2 or 4), forward transform |
@@ -81,17 +82,17 @@ struct VarArgs {
 template <int DIM, int K, int NT, int PP, int CTAS, bool PRE>
 __global__ void __launch_bounds__(NT, CTAS) pair_var_kernel(const __grid_constant__ VarArgs va) {
   using Z = VarSmem<DIM, K>;
-  constexpr int C = Z::C, M = Z::M, H = Z::H, R = Z::R, F = Z::F, NP = 2 * PP;
+  constexpr int C = Z::C, M = Z::M, H = Z::H, R = Z::R, F = Z::F, W = PA::W, NP = W * PP;
   constexpr int LINES = DIM == 3 ? M * M : M, NCELL = Z::NCELL;
   static_assert(NP <= NT, "one thread sets up one patch");
   extern __shared__ __align__(128) unsigned char smem_raw[];
-  E* const W = reinterpret_cast<E*>(smem_raw);  // [PP][2][F]
-  E* const CO = W + PP * 2 * F;                  // [PP][NCELL] cell coefficients of both patches
+  E* const S = reinterpret_cast<E*>(smem_raw);  // [PP][2][F]
+  E* const CO = S + PP * 2 * F;                  // [PP][NCELL] cell coefficients of both patches
   __shared__ long long s_origin[NP], s_cell[NP];
   __shared__ T s_scale[NP];
   const PatchLaunch& pl = va.pl;
   const long long py = pl.g.py, pz = pl.g.pz;
-  const int g0 = blockIdx.x * NP, nv = min(NP, pl.n_patches - g0), npair = (nv + 1) / 2, n = pl.g.n;
+  const int g0 = blockIdx.x * NP, nv = min(NP, pl.n_patches - g0), npair = (nv + W - 1) / W, n = pl.g.n;
   const float sb = (float)pl.sb;  // an integer power of the cell count, exact in float
   if ((int)threadIdx.x < NP) {  // (a lone last patch is carried twice and stored once)
     const int q = threadIdx.x, pid = g0 + min(q, nv - 1);
@@ -107,7 +108,7 @@ __global__ void __launch_bounds__(NT, CTAS) pair_var_kernel(const __grid_constan
   for (int t = threadIdx.x; t < npair * NCELL; t += NT) {
     const int q = t / NCELL, c = t % NCELL;
     const long long o = (c & 1) + (long long)n * (((c >> 1) & 1) + (DIM == 3 ? (long long)n * (c >> 2) : 0));
-    PA::store(CO[t], PA::pack(va.coef[s_cell[2 * q] + o], va.coef[s_cell[2 * q + 1] + o]));
+    PA::store(CO[t], PA::pack(va.coef[s_cell[W * q] + o], va.coef[s_cell[W * q + W - 1] + o]));
   }
   // the rows of b are on their way from the start
   constexpr bool EARLY = PRE && PP * LINES <= NT;
@@ -115,14 +116,14 @@ __global__ void __launch_bounds__(NT, CTAS) pair_var_kernel(const __grid_constan
   T eb[EARLY ? 2 * M : 1];
   auto rhs = [&](int t, int p) -> const T* {
     const int ln = t % LINES;
-    return va.b + s_origin[2 * (t / LINES) + p] + 1 + ln % M + (DIM == 3 ? py * (1 + ln / M) : 0) + ps;
+    return va.b + s_origin[W * (t / LINES) + p] + 1 + ln % M + (DIM == 3 ? py * (1 + ln / M) : 0) + ps;
   };
   if constexpr (EARLY) {
     const int t = (int)threadIdx.x < npair * LINES ? threadIdx.x : 0;
 #pragma unroll
     for (int l = 0; l < M; ++l) {
       eb[l] = __ldg(rhs(t, 0) + ps * l);
-      eb[M + l] = __ldg(rhs(t, 1) + ps * l);
+      eb[M + l] = __ldg(rhs(t, W - 1) + ps * l);
     }
   }
   // row of a cell-wise axis that holds interior node i (the first of the two
@@ -148,8 +149,8 @@ __global__ void __launch_bounds__(NT, CTAS) pair_var_kernel(const __grid_constan
     // ---- y: P = M_y u, Q = K_y u on lines (x, z), from -u ----
     for (int t = threadIdx.x; t < npair * C * C; t += NT) {
       const int q = t / (C * C), x = t % C, z = t % (C * C) / C;
-      const T *const a = va.u + s_origin[2 * q] + x + pz * z, *const b = va.u + s_origin[2 * q + 1] + x + pz * z;
-      E* const P = W + q * 2 * F + z * H * R + x;
+      const T *const a = va.u + s_origin[W * q] + x + pz * z, *const b = va.u + s_origin[W * q + W - 1] + x + pz * z;
+      E* const P = S + q * 2 * F + z * H * R + x;
       line_rows([&](int y) -> V { return PA::pack_neg(a[py * y], b[py * y]); },
                 [&](int j, V m, V k) {
                   PA::store(P[j * R], m);
@@ -159,7 +160,7 @@ __global__ void __launch_bounds__(NT, CTAS) pair_var_kernel(const __grid_constan
     __syncthreads();
     // ---- x: A1 = M_x P, A2 = K_x P + M_x Q on rows (y, z), in place ----
     for (int t = threadIdx.x; t < npair * C * H; t += NT) {
-      E* const P = W + t / (C * H) * 2 * F + t % (C * H) * R;
+      E* const P = S + t / (C * H) * 2 * F + t % (C * H) * R;
       V a1[H], a2[H];
 #pragma unroll
       for (int r = 0; r < 2; ++r) {
@@ -189,8 +190,8 @@ __global__ void __launch_bounds__(NT, CTAS) pair_var_kernel(const __grid_constan
     // ---- x: P = M_x u, Q = K_x u on rows y, from -u ----
     for (int t = threadIdx.x; t < npair * C; t += NT) {
       const int q = t / C, y = t % C;
-      const T *const a = va.u + s_origin[2 * q] + py * y, *const b = va.u + s_origin[2 * q + 1] + py * y;
-      E* const P = W + q * 2 * F + y * R;
+      const T *const a = va.u + s_origin[W * q] + py * y, *const b = va.u + s_origin[W * q + W - 1] + py * y;
+      E* const P = S + q * 2 * F + y * R;
       line_rows([&](int x) -> V { return PA::pack_neg(a[x], b[x]); },
                 [&](int i, V m, V k) {
                   PA::store(P[i], m);
@@ -207,7 +208,7 @@ __global__ void __launch_bounds__(NT, CTAS) pair_var_kernel(const __grid_constan
     const int q = t / COLS, X = t % COLS % H, Y = t % COLS / H;
     const int c = (X >= K ? 1 : 0) + (DIM == 3 && Y >= K ? 2 : 0);  // cell of the column at the low end
     constexpr int UP = DIM == 3 ? 4 : 2;                             // and at the high end: c + UP
-    E* const P = W + q * 2 * F + (DIM == 3 ? Y * R : 0) + X;
+    E* const P = S + q * 2 * F + (DIM == 3 ? Y * R : 0) + X;
     PA::acc col[M];
 #pragma unroll
     for (int r = 0; r < 2; ++r) {
@@ -234,11 +235,11 @@ __global__ void __launch_bounds__(NT, CTAS) pair_var_kernel(const __grid_constan
   __syncthreads();
   // ---- r = h^{2-d} b + the columns of each node, forward transform ----
   auto column = [&](int q, int ln) -> E* {
-    return W + q * 2 * F + (DIM == 3 ? pos(ln / M) * R + pos(ln % M) : pos(ln));
+    return S + q * 2 * F + (DIM == 3 ? pos(ln / M) * R + pos(ln % M) : pos(ln));
   };
   for (int t = threadIdx.x; t < npair * LINES; t += NT) {
     const int q = t / LINES, ln = t % LINES, i = ln % M, j = ln / M;
-    const T *const ba = rhs(t, 0), *const bb = rhs(t, 1);
+    const T *const ba = rhs(t, 0), *const bb = rhs(t, W - 1);
     E* const w = column(q, ln);
     const bool two_x = i == K - 1, two_y = DIM == 3 && j == K - 1;
     V r[M];
@@ -263,7 +264,7 @@ __global__ void __launch_bounds__(NT, CTAS) pair_var_kernel(const __grid_constan
   auto line_y = [&](auto forward) {
     for (int t = threadIdx.x; t < npair * LINES; t += NT) {
       const int q = t / LINES, ln = t % LINES;  // x + M z
-      E* const w = W + q * 2 * F + ln / M * SL + pos(ln % M);
+      E* const w = S + q * 2 * F + ln / M * SL + pos(ln % M);
       V v[M];
 #pragma unroll
       for (int j = 0; j < M; ++j) v[j] = PA::load(w[pos(j) * R]);
@@ -276,7 +277,7 @@ __global__ void __launch_bounds__(NT, CTAS) pair_var_kernel(const __grid_constan
   if (DIM == 3) line_y(std::true_type());
   for (int t = threadIdx.x; t < npair * LINES; t += NT) {
     const int q = t / LINES, ln = t % LINES;  // 3D: y + M z; 2D: y
-    E* const w = W + q * 2 * F + (DIM == 3 ? ln / M * SL + pos(ln % M) * R : ln * SL);
+    E* const w = S + q * 2 * F + (DIM == 3 ? ln / M * SL + pos(ln % M) * R : ln * SL);
     V v[M], x[M];
 #pragma unroll
     for (int i = 0; i < M; ++i) v[i] = PA::load(w[pos(i)]);
@@ -293,11 +294,11 @@ __global__ void __launch_bounds__(NT, CTAS) pair_var_kernel(const __grid_constan
     V v[M];
 #pragma unroll
     for (int l = 0; l < M; ++l) v[l] = PA::load(w[l * SL]);
-    const bool two = 2 * q + 1 < nv;
+    const bool two = W == 2 && 2 * q + 1 < nv;
     const int x = 1 + ln % M, y = DIM == 3 ? 1 + ln / M : 0;
     const long long ofs = x + (DIM == 3 ? py * y : 0) + ps;
-    T *const ga = va.u + s_origin[2 * q] + ofs, *const gb = va.u + s_origin[2 * q + 1] + ofs;
-    const T sa = s_scale[2 * q], sc = s_scale[2 * q + 1];
+    T *const ga = va.u + s_origin[W * q] + ofs, *const gb = va.u + s_origin[W * q + W - 1] + ofs;
+    const T sa = s_scale[W * q], sc = s_scale[W * q + W - 1];
     T oa[M], ob[M];
 #pragma unroll
     for (int l = 0; l < M; ++l) {
@@ -329,31 +330,54 @@ int var_pair_launch(const PatchLaunch& pl, T* u, const T* b, const T* coef, cons
     *ready = true;
   }
   const VarArgs va{pl, u, b, coef, vscale, dinv};
-  kern<<<(pl.n_patches + 2 * PP - 1) / (2 * PP), NT, SMEM, s>>>(va);
+  kern<<<(pl.n_patches + PA::W * PP - 1) / (PA::W * PP), NT, SMEM, s>>>(va);
   count_launch();
   return cudaGetLastError() == cudaSuccess ? GMG_OK : GMG_ERR_CUDA;
 }
 
-// Patch pairs and threads per CTA, and the CTAs per SM that the registers are
-// limited for; PRE: the rows of b are loaded before the first stage.  As many
-// pairs as fill the threads with the interior lines of a stage.  Measured per
-// sweep (us), the shape taken first: FP64 Q3 64^3 10 pairs in 256 threads with
-// registers for 2 CTAs 1384 (without PRE 1474), 5 in 128 for 4 1617, for 1
-// 2070; Q2 96^3 14 in 128 for 5 1168 (1235), for 1 1504; 2D Q3 1024^2 25 in 128
-// for 5 717, for 1 1131; FP32 Q3 64^3 5 in 128 317, 1 in 32 341.
+// Shapes: patches (FP32: pairs) and threads per CTA, and the CTAs per SM that the
+// registers are limited for (0: left to the compiler); PRE: the rows of b are
+// loaded before the first stage.  Up to LIMIT patches as many as fill the threads
+// with the lines of the first stage, above it the shape of a full chip.
+//
+// FP64 takes one patch per thread: two were slower at every size, and twice as
+// slow as one patch per CTA on small colours.  Per sweep (us), one patch per CTA -> two
+// per thread -> now: 3D Q3 16^3 99 -> 197 -> 99, 24^3 205 -> 197 -> 123, 64^3 3479
+// -> 1364 -> 1193; Q2 16^3 81 -> 131 -> 66, 64^3 1688 -> 361 -> 323; Q1 16^3 49 ->
+// 89 -> 49, 64^3 600 -> 115 -> 82; 2D Q3 80^2 41 -> 62 -> 33, 640^2 1555 -> 291 ->
+// 233.  Shapes at 3D Q3 64^3: 10 in 256 threads 1209, 5 in 256 1309 (16^3: 135, 98),
+// 5 in 128 1390, limited for 2 CTAs 1588; Q2 64^3 14 in 128 331, 5 in 128 382 (16^3:
+// 114, 68).  Colours that leave an SM to each patch last as long as one patch
+// takes, and patch_var_kernel, whose threads share a patch cell by cell, is the
+// shortest there: 3D Q3 8^3 82 us against 98, Q2 66 against 74 (16^3: 99, 98), 2D Q3
+// 4^2 33 against 37.
+//
+// FP32, two patches per thread: 3D Q3 16^3 65 -> 49 with the small shape (2 pairs in
+// 128 threads; 24^3 66 both), Q2 16^3 66 -> 49 (64^3: 129, 131), Q1 32^3 65 -> 49; Q3
+// 64^3 5 in 128 317, 1 in 32 341.
 template <int DIM, int K>
 struct VarPairCfg {
-  static constexpr int LINES = DIM == 3 ? (2 * K - 1) * (2 * K - 1) : 2 * K - 1;
-  static constexpr int NT = DF && DIM == 3 && K == 3 ? 256 : 128;
-  static constexpr int PP = std::max(1, std::min(NT / LINES, 3 * NT / 8));
-  static constexpr int CTAS = !DF || K == 1 ? 1 : DIM == 3 && K == 3 ? 2 : 5;
+  static constexpr int C = 2 * K + 1, M = 2 * K - 1, LINES = DIM == 3 ? M * M : M, FIRST = DIM == 3 ? C * C : C;
   static constexpr bool PRE = DF || DIM == 2;
+  // a full chip
+  static constexpr int NT = DF && DIM == 3 && K == 3 ? 256 : 128;
+  static constexpr int PP = DF && (DIM == 2 || K == 1) ? NT / FIRST : std::max(1, std::min(NT / LINES, 3 * NT / 8));
+  static constexpr int CTAS = DF ? 0 : 1;
+  // small colours
+  static constexpr int SPP = DF ? NT / FIRST : K == 1 ? 3 : K == 2 ? 5 : 2, SNT = !DF && K == 1 ? 32 : NT;
+  static constexpr int LIMIT = DIM == 2 ? 0 : DF ? (K == 1 ? 0 : 8000) : K == 3 ? 2000 : 8000;
+  static constexpr int ONE = DF && K >= (DIM == 3 ? 2 : 3) ? 152 : 0;  // patch_var_kernel: the SMs of the chip
 };
 
 template <int DIM, int K>
 int var_pair_impl(const PatchLaunch& pl, T* u, const T* b, const T* coef, const T* vscale, const T* dinv,
                   cudaStream_t s) {
   using Cfg = VarPairCfg<DIM, K>;
+  if (pl.n_patches <= Cfg::ONE) return launch_patch_var<T>(pl, u, b, coef, vscale, dinv, nullptr, 0, s);
+  if constexpr (Cfg::LIMIT > 0) {
+    if (pl.n_patches <= Cfg::LIMIT)
+      return var_pair_launch<DIM, K, Cfg::SNT, Cfg::SPP, 0, Cfg::PRE>(pl, u, b, coef, vscale, dinv, s);
+  }
   return var_pair_launch<DIM, K, Cfg::NT, Cfg::PP, Cfg::CTAS, Cfg::PRE>(pl, u, b, coef, vscale, dinv, s);
 }
 

@@ -7,7 +7,8 @@
 //    factorisation (App. A.1), accumulated with atomics (a node is shared
 //    by up to 2^d cells); the caller initialises y.
 //  * patch_var_kernel: one colour of the patch smoother (Algorithm 4) on
-//    levels with a learned correction (the others: pair_var.cuh); the
+//    levels with a learned correction, and small colours of the others (which
+//    are the work of pair_var.cuh); the
 //    local residual is evaluated cell by cell with the cell coefficients
 //    (Sec. 3.1, eq. "main:4"), and whose local solver is the fast
 //    diagonalisation of the constant-coefficient patch scaled by the
@@ -297,9 +298,9 @@ __global__ void init_interior_kernel(T* __restrict__ y, const T* __restrict__ b,
 
 // One colour of the variable-coefficient patch smoother: persistent CTAs,
 // one patch at a time.  With TMA the closure of u and the interior of b of
-// the CTA's next patch arrive by two TMA boxes
-// into the other input slot while the current patch is computed; without it
-// they are read element by element into the same layout.
+// the CTA's next patch arrive by two TMA boxes into the other input slot while
+// the current patch is computed; without it they are read element by element
+// into the same layout.
 template <int DIM, int K, int NT, bool TMA>
 __global__ void __launch_bounds__(NT) patch_var_kernel(T* __restrict__ u, const T* __restrict__ b,
                                                        const T* __restrict__ coef,

@@ -9,6 +9,8 @@ schedule gives each patch exactly the values that the whole colours give it.
 import numpy as np
 import pytest
 
+from oracle.mesh import Mesh
+from oracle.varcoef import VarPatchSmoother
 from paper_2407_02100_gb300 import inputs
 
 pytestmark = pytest.mark.gpu
@@ -41,3 +43,34 @@ def test_whole_colours_and_slabs_agree_bit_for_bit(gmg, dim, k, n, precision):
     whole = sweep(gmg, dim, k, n, precision, 0, k % 2 == 1)
     assert np.array_equal(whole, sweep(gmg, dim, k, n, precision, 1, k % 2 == 1))
     assert np.isfinite(whole).all()
+
+
+def var_sweep(gmg, dim, k, n, precision):
+    coef = inputs.lognormal_coefficient(dim, n, 13)
+    P = gmg.Problem(dim, k, n, precision=precision)
+    gmg.gmg_set_coefficient(P.h, coef)
+    u, b = inputs.random_nodal(dim, k, n, 14), inputs.random_nodal(dim, k, n, 15)
+    ud = P.to_device(u)
+    gmg.gmg_smooth(P.h, P.finest, ud, P.to_device(b), 1, n % 2 == 1)
+    out = P.from_device(ud)
+    P.close()
+    return out, coef, u, b
+
+
+# variable coefficient, FP64 3D: up to 152 patches one per CTA, above one per
+# thread, from 8000 on in larger groups.  Against the oracle at 1e-12 (FP64) and
+# 1e-5 (FP32, whose small colours take another shape), as elsewhere
+@pytest.mark.parametrize("dim,k,n", [(3, 1, 12), (3, 2, 8), (3, 2, 12), (3, 3, 8), (3, 3, 12), (2, 3, 24), (2, 3, 32)])
+@pytest.mark.parametrize("precision,tol", [(0, 1e-12), (1, 1e-5)])
+def test_variable_coefficient(gmg, dim, k, n, precision, tol):
+    out, coef, u, b = var_sweep(gmg, dim, k, n, precision)
+    ref = VarPatchSmoother(Mesh(dim, k, n), coef, "fd_mean").sweep(u, b, n % 2 == 1)
+    assert np.linalg.norm(out - ref) <= tol * np.linalg.norm(ref)
+
+
+# the largest groups: the FP64 sweep is the reference of the FP32 one, 1e-5
+@pytest.mark.parametrize("k", [1, 2, 3])
+def test_variable_coefficient_large_colours(gmg, k):
+    ref = var_sweep(gmg, 3, k, 48, gmg.GMG_FP64)[0]
+    out = var_sweep(gmg, 3, k, 48, gmg.GMG_FP32)[0]
+    assert np.linalg.norm(out - ref) <= 1e-5 * np.linalg.norm(ref)
