@@ -10,6 +10,7 @@ import numpy as np
 import pytest
 
 from oracle.mesh import Mesh
+from oracle.multigrid import prolongation
 from oracle.varcoef import VarPatchSmoother
 from paper_2407_02100_gb300 import inputs
 
@@ -74,3 +75,17 @@ def test_variable_coefficient_large_colours(gmg, k):
     ref = var_sweep(gmg, 3, k, 48, gmg.GMG_FP64)[0]
     out = var_sweep(gmg, 3, k, 48, gmg.GMG_FP32)[0]
     assert np.linalg.norm(out - ref) <= 1e-5 * np.linalg.norm(ref)
+
+
+# FP32 prolongation on both sides of its lines, 240,000 fine nodes in 2D and 60,000 in 3D: three
+# passes of up to k + 1 terms at 2^-24 each stay below 5e-6
+@pytest.mark.parametrize("dim,k,nc", [(2, 3, 81), (2, 3, 82), (2, 8, 30), (2, 8, 31), (3, 2, 9), (3, 2, 10), (3, 4, 4), (3, 4, 5)])
+def test_fp32_prolongation(gmg, dim, k, nc):
+    Pm = prolongation(Mesh(dim, k, nc), Mesh(dim, k, 2 * nc), sparse=True)
+    P = gmg.Problem(dim, k, 2 * nc, n_levels=2, precision=gmg.GMG_FP32)
+    e, u = inputs.random_nodal(dim, k, nc, 16), inputs.random_nodal(dim, k, 2 * nc, 17)
+    f = P.to_device(u)
+    gmg.gmg_prolongate_add(P.h, 0, P.to_device(e, 0), f)
+    ref = u + Pm @ e
+    assert np.linalg.norm(P.from_device(f) - ref) <= 5e-6 * np.linalg.norm(ref)
+    P.close()
