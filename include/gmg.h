@@ -496,14 +496,17 @@ int gmg_shared_faces(const gmg_problem* p);
  * thread a whole line per stage, this kernel a single output.  Same method
  * and colour order; results agree with the other forms up to rounding.
  * Levels swept by it take no slab schedule.
- * gmg_set_small_sweep: max_patches >= 0 (0 turns the kernel off; gmg_create
- *   sets 256 for degrees up to 4 and 0 above, and where the shared-face form
- *   would take a larger colour, up to 1536 patches at degree 3, 640 at
- *   degree 4 and 128 above; a limit set here holds as it is); GMG_ERR_INVALID_ARG for a
- *   null problem or a negative count.  Single-precision and variable-
- *   coefficient problems ignore it.
- * gmg_small_sweep: the current max_patches, GMG_ERR_INVALID_ARG for a null
- *   problem. */
+ * gmg_set_small_sweep: max_patches >= 0, 0: no colour leaves the form that it
+ *   takes otherwise; GMG_ERR_INVALID_ARG for a null problem or a negative count.
+ *   Unless it is set, the limit is 256 for degrees up to 4 and 0 above, and 1536
+ *   at degree 3 and 640 at degree 4 while whole colours take the shared-face form
+ *   (gmg_shared_faces); a limit set here holds as it is.  Apart from the limit,
+ *   the shared-face form evaluates its own smallest colours (at most 128 patches,
+ *   from degree 5) with this kernel; gmg_set_shared_faces(p, 0) turns that off
+ *   with the form.  Single-precision and variable-coefficient problems ignore
+ *   the limit.
+ * gmg_small_sweep: the limit in force, which gmg_set_small_sweep can be given
+ *   back; GMG_ERR_INVALID_ARG for a null problem. */
 int gmg_set_small_sweep(gmg_problem* p, int max_patches);
 int gmg_small_sweep(const gmg_problem* p);
 

@@ -201,20 +201,21 @@ PatchLaunch colour_launch(const Level& L, int colour, double omega) {
   return pl;
 }
 
+// Largest colour that the coarse-level kernel takes (FP64 problems).  Unless the
+// caller has set it, the limit is higher where the shared-face form would run
+// (equal up to rounding, unlike the closure form and its slabs): 228 -> 152 us a
+// sweep of 512 patches a colour at k = 4, 160 -> 100 us of 1000 at k = 3, even at
+// 1728 (150 : 161 us) and behind above.
+int small_limit(const gmg_problem* p) {
+  const int k = p->desc.degree;
+  if (!p->small_auto || !p->faces || !p->shared_faces || k > 4) return p->small_patches;
+  return std::max(p->small_patches, k == 3 ? 1536 : 640);
+}
+
 int launch_colour(gmg_problem* p, const PatchLaunch& pl, void* u, const void* b) {
   if (pl.n_patches == 0) return GMG_OK;
   if (p->esize == 8) {
-    // a coarse level: one output per thread.  Where the shared-face form would
-    // run (equal up to rounding, unlike the closure form and its slabs), the
-    // coarse-level kernel wins on larger colours too: 228 -> 152 us a sweep of
-    // 512 patches a colour at k = 4, 160 -> 100 us of 1000 at k = 3, even at
-    // 1728 (150 : 161 us) and behind above; at k >= 5 while each patch has an SM
-    // to itself (us a sweep of 6^3: Q5 306 : 115, Q7 504 : 293, Q8 648 : 425);
-    // a limit that the caller sets holds as it is
-    const int k = pl.g.k;
-    const int small = p->faces && p->shared_faces && p->small_auto
-                          ? std::max(p->small_patches, k == 3 ? 1536 : k == 4 ? 640 : k >= 5 ? 128 : 0) : p->small_patches;
-    if (pl.n_patches <= small) {
+    if (pl.n_patches <= small_limit(p)) {  // a coarse level: one output per thread
       const int st = launch_patch_small<double>(pl, (double*)u, (const double*)b, (const double*)p->dinv, p->stream);
       if (st != GMG_ERR_UNSUPPORTED) return st;
     }
@@ -273,7 +274,7 @@ long long max_colour_patches(const gmg_problem* p, const Level& L) {
 
 // FP64 levels whose colours all take the coarse-level kernel (gmg_set_small_sweep)
 bool small_level(const gmg_problem* p, const Level& L) {
-  return p->esize == 8 && !p->varcoef && max_colour_patches(p, L) <= p->small_patches;
+  return p->esize == 8 && !p->varcoef && max_colour_patches(p, L) <= small_limit(p);
 }
 
 int slab_width_for(const gmg_problem* p, const Level& L) {
@@ -332,6 +333,18 @@ int build_slabs(gmg_problem* p, int level, int W) {
   }
   L.slab_w = W;
   return GMG_OK;
+}
+
+// The slab lists of every level by the problem's present settings.  The copies of
+// new lists have arrived on return, whatever stream the problem runs on.
+int rebuild_slabs(gmg_problem* p) {
+  bool changed = false;
+  for (int l = 0; l < (int)p->levels.size(); ++l) {
+    const int W = slab_width_for(p, p->levels[l]);
+    changed |= W != p->levels[l].slab_w;
+    CHECK(build_slabs(p, l, W));
+  }
+  return !changed || cudaDeviceSynchronize() == cudaSuccess ? GMG_OK : GMG_ERR_CUDA;
 }
 
 int smooth(gmg_problem* p, int level, void* u, const void* b, int n_sweeps, int reverse) {
@@ -1169,7 +1182,7 @@ int gmg_set_shared_faces(gmg_problem* p, int enable) {
   if (!p) return GMG_ERR_INVALID_ARG;
   drop_cg_graph(p);
   p->shared_faces = enable != 0;
-  return GMG_OK;
+  return rebuild_slabs(p);  // levels leave or join the coarse-level kernel with it (small_limit)
 }
 
 int gmg_shared_faces(const gmg_problem* p) {
@@ -1182,22 +1195,19 @@ int gmg_set_small_sweep(gmg_problem* p, int max_patches) {
   drop_cg_graph(p);
   p->small_patches = max_patches;
   p->small_auto = false;
-  // levels that leave or join the coarse-level kernel take or drop their slabs
-  for (int l = 0; l < (int)p->levels.size(); ++l) CHECK(build_slabs(p, l, slab_width_for(p, p->levels[l])));
-  return GMG_OK;
+  return rebuild_slabs(p);  // levels that leave or join the coarse-level kernel take or drop their slabs
 }
 
 int gmg_small_sweep(const gmg_problem* p) {
   if (!p) return GMG_ERR_INVALID_ARG;
-  return p->small_patches;
+  return small_limit(p);
 }
 
 int gmg_set_slab_width(gmg_problem* p, int width) {
   if (!p || width < -1) return GMG_ERR_INVALID_ARG;
   drop_cg_graph(p);
   p->slab_width = width;
-  for (int l = 0; l < (int)p->levels.size(); ++l) CHECK(build_slabs(p, l, slab_width_for(p, p->levels[l])));
-  return cudaDeviceSynchronize() == cudaSuccess ? GMG_OK : GMG_ERR_CUDA;
+  return rebuild_slabs(p);
 }
 
 int gmg_slab_width(const gmg_problem* p, int level) {

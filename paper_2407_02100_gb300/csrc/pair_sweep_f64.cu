@@ -534,6 +534,11 @@ struct PairSweepCfg {
 };
 constexpr int kFaceThreads = 128;
 
+// From degree 5 a colour of at most this many patches, while each patch has an SM to
+// itself, goes to the coarse-level kernel, one output per thread (us a sweep of 6^3:
+// Q5 289 -> 115, Q6 345 -> 181, Q7 489 -> 289, Q8 625 -> 421).
+constexpr int kFewPatches = 128;
+
 template <typename KernelT>
 int opt_in(KernelT kern, int smem) {
   return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) == cudaSuccess ? GMG_OK
@@ -610,6 +615,7 @@ int launch_patch_faces<double>(const PatchLaunch& pl, double* u, const double* b
   if (pl.g.dim != 3 || pl.g.k < 3 || pl.g.k > 8 || pl.mode != 0 || pl.plist || !faces) return GMG_ERR_UNSUPPORTED;
   if (!tma_vector_ok(b, 8, 3, pl.g.py, pl.g.pz)) return GMG_ERR_UNSUPPORTED;
   if (pl.n_patches <= 0) return GMG_OK;
+  if (pl.g.k >= 5 && pl.n_patches <= kFewPatches) return launch_patch_small<double>(pl, u, b, dinv, s);
   switch (pl.g.k) {
     case 3: return face_sweep<3>(pl, u, b, dinv, faces, s);
     case 4: return face_sweep<4>(pl, u, b, dinv, faces, s);

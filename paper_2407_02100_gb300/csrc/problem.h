@@ -107,7 +107,8 @@ struct gmg_problem {
   void* faces = nullptr;
   bool shared_faces = true;
   // FP64 colour steps of at most this many patches use the coarse-level
-  // kernel (gmg_set_small_sweep; 0: never; set by gmg_create)
+  // kernel (gmg_set_small_sweep; set by gmg_create; small_limit raises it where
+  // small_auto allows)
   int small_patches = 0;
   bool small_auto = false;  // the limit is the library's, not the caller's
   // workspace of the three-pass FP64 3D operator (two finest-level

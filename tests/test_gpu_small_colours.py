@@ -89,3 +89,39 @@ def test_fp32_prolongation(gmg, dim, k, nc):
     ref = u + Pm @ e
     assert np.linalg.norm(P.from_device(f) - ref) <= 5e-6 * np.linalg.norm(ref)
     P.close()
+
+
+# the limit of the coarse-level kernel: what is read can be given back, whichever
+# rule set it, and levels that the kernel sweeps keep no slabs
+@pytest.mark.parametrize("k,n,limit", [(2, 16, 256), (3, 20, 1536), (4, 16, 640), (5, 8, 0), (7, 6, 0)])
+def test_limit_that_was_read_can_be_given_back(gmg, k, n, limit):
+    u0, b = inputs.random_nodal(3, k, n, 18), inputs.random_nodal(3, k, n, 19)
+
+    def run(P):
+        u, launches = P.to_device(u0), gmg.gmg_kernel_launch_count()
+        gmg.gmg_smooth(P.h, P.finest, u, P.to_device(b), 1, False)
+        return P.from_device(u), gmg.gmg_kernel_launch_count() - launches
+
+    P = gmg.Problem(3, k, n)
+    ref, launches = run(P)
+    assert gmg.gmg_small_sweep(P.h) == limit
+    gmg.gmg_set_small_sweep(P.h, 0)
+    off, _ = run(P)
+    assert gmg.gmg_small_sweep(P.h) == 0
+    gmg.gmg_set_small_sweep(P.h, limit)
+    again, count = run(P)
+    assert np.array_equal(again, ref) and count == launches
+    assert np.linalg.norm(off - ref) <= 1e-12 * np.linalg.norm(ref)
+    P.close()
+
+
+@pytest.mark.parametrize("k,n", [(3, 20), (4, 16)])
+def test_levels_of_the_raised_limit_keep_no_slabs(gmg, k, n):
+    P = gmg.Problem(3, k, n)  # 1000 and 512 patches in the largest colour
+    gmg.gmg_set_slab_width(P.h, 2)
+    assert gmg.gmg_slab_width(P.h, P.finest) == 0
+    gmg.gmg_set_shared_faces(P.h, False)  # the closure form, whose limit is 256
+    assert gmg.gmg_small_sweep(P.h) == 256 and gmg.gmg_slab_width(P.h, P.finest) == 2
+    gmg.gmg_set_shared_faces(P.h, True)
+    assert gmg.gmg_slab_width(P.h, P.finest) == 0
+    P.close()
