@@ -502,7 +502,7 @@ int gmg_shared_faces(const gmg_problem* p);
  *   at degree 3 and 640 at degree 4 while whole colours take the shared-face form
  *   (gmg_shared_faces); a limit set here holds as it is.  Apart from the limit,
  *   the shared-face form evaluates its own smallest colours (at most 128 patches,
- *   from degree 5) with this kernel; gmg_set_shared_faces(p, 0) turns that off
+ *   degrees 5 to 7) with this kernel; gmg_set_shared_faces(p, 0) turns that off
  *   with the form.  Single-precision and variable-coefficient problems ignore
  *   the limit.
  * gmg_small_sweep: the limit in force, which gmg_set_small_sweep can be given

@@ -534,9 +534,12 @@ struct PairSweepCfg {
 };
 constexpr int kFaceThreads = 128;
 
-// From degree 5 a colour of at most this many patches, while each patch has an SM to
-// itself, goes to the coarse-level kernel, one output per thread (us a sweep of 6^3:
-// Q5 289 -> 115, Q6 345 -> 181, Q7 489 -> 289, Q8 625 -> 421).
+// At degrees 5 to 7 a colour of at most this many patches, while each patch has an
+// SM to itself, goes to the coarse-level kernel, one output per thread (us a sweep
+// of 6^3: Q5 289 -> 115, Q6 345 -> 181, Q7 489 -> 289).  Not at degree 8 (625 : 421):
+// its error against 64 bits is a quarter larger there, as it evaluates the
+// residual on the whole closure and not on its boundary (8^3: 2.5e-14 against
+// 2.0e-14; Q5 1.08e-14 and 1.05e-14, Q6 1.8e-14 and 1.9e-14, Q7 2.3e-14 and 3.0e-14).
 constexpr int kFewPatches = 128;
 
 template <typename KernelT>
@@ -615,7 +618,7 @@ int launch_patch_faces<double>(const PatchLaunch& pl, double* u, const double* b
   if (pl.g.dim != 3 || pl.g.k < 3 || pl.g.k > 8 || pl.mode != 0 || pl.plist || !faces) return GMG_ERR_UNSUPPORTED;
   if (!tma_vector_ok(b, 8, 3, pl.g.py, pl.g.pz)) return GMG_ERR_UNSUPPORTED;
   if (pl.n_patches <= 0) return GMG_OK;
-  if (pl.g.k >= 5 && pl.n_patches <= kFewPatches) return launch_patch_small<double>(pl, u, b, dinv, s);
+  if (pl.g.k >= 5 && pl.g.k <= 7 && pl.n_patches <= kFewPatches) return launch_patch_small<double>(pl, u, b, dinv, s);
   switch (pl.g.k) {
     case 3: return face_sweep<3>(pl, u, b, dinv, faces, s);
     case 4: return face_sweep<4>(pl, u, b, dinv, faces, s);

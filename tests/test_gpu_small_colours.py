@@ -125,3 +125,18 @@ def test_levels_of_the_raised_limit_keep_no_slabs(gmg, k, n):
     gmg.gmg_set_shared_faces(P.h, True)
     assert gmg.gmg_slab_width(P.h, P.finest) == 0
     P.close()
+
+
+# degrees 5 to 7 hand colours of up to 128 patches to the coarse-level kernel (one launch a
+# colour), degree 8 keeps the shared-face form's two, whose error is smaller there
+@pytest.mark.parametrize("k,n,launches", [(5, 10, 8), (6, 4, 8), (7, 4, 8), (8, 4, 16), (8, 6, 16)])
+def test_few_patches_of_the_shared_face_form(gmg, k, n, launches):
+    P = gmg.Problem(3, k, n)
+    u, b = P.to_device(inputs.random_nodal(3, k, n, 20)), P.to_device(inputs.random_nodal(3, k, n, 21))
+    u2, before = u.clone(), gmg.gmg_kernel_launch_count()
+    gmg.gmg_smooth(P.h, P.finest, u, b, 1, False)
+    assert gmg.gmg_kernel_launch_count() - before == launches
+    gmg.gmg_set_shared_faces(P.h, False)
+    gmg.gmg_smooth(P.h, P.finest, u2, b, 1, False)
+    assert float((u - u2).norm() / u2.norm()) <= 1e-12
+    P.close()
