@@ -44,3 +44,17 @@ def test_groups_agree_with_closure_form(gmg, k, n, damping, reverse):
     assert np.linalg.norm(a - c) <= 1e-12 * np.linalg.norm(c)
     # whichever CTA takes a group, its patches come out bit for bit the same
     assert np.array_equal(a, sweep(gmg, k, n, True, damping, reverse))
+
+
+# more groups than resident CTAs (at most 304; 4 an SM at k = 6) at every degree: a CTA takes
+# further groups, flips the phase of its barrier, refills the face blocks during the transforms
+# and reuses the slots of b; the first colours have odd counts, so that a lone last patch
+# follows full groups.  Largest colours: 3375, 2197, 1331, 729 and 729 patches, in groups of 10,
+# 6, 2, 2 and 2
+@pytest.mark.parametrize("k,n,damping,reverse", [
+    (4, 31, 0.9, True), (5, 27, 1.0, False), (6, 23, 1.0, True), (7, 19, 0.8, False), (8, 19, 1.0, False)])
+def test_persistent_groups_agree_with_closure_form(gmg, k, n, damping, reverse):
+    a = sweep(gmg, k, n, True, damping, reverse)
+    c = sweep(gmg, k, n, False, damping, reverse)
+    assert np.linalg.norm(a - c) <= 1e-12 * np.linalg.norm(c)
+    assert np.array_equal(a, sweep(gmg, k, n, True, damping, reverse))
