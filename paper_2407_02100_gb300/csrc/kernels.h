@@ -65,8 +65,8 @@ struct PatchTable {
 struct ApplyLaunch {
   LevelGeom g;
   double alpha, beta;
-  // FP64 3D: four level vectors of workspace (pz * N doubles each) for the
-  // halo-free three-pass form, or null for the tile kernel
+  // FP64 3D: two level vectors of workspace (pz * N doubles each) for the
+  // three-pass form, or null for the tile kernel
   void* ws = nullptr;
   // tile kernel shape in 3D at degrees 3, 4, 7 (gmg_set_operator_tile):
   // 0 the default of the precision and degree, 1 cubes, 2 flat 4x4x1,
@@ -118,6 +118,10 @@ int upload_closure_tables(int k, const double* Mp, const double* Kp, const doubl
 // the table's group ranges
 int upload_closure_solo_tables(int k, const double* Mp, const double* Kp, const double* That);
 int launch_closure_solo(int dim, int k, PatchTable& tab, const double* dinv, cudaStream_t s);
+int prepare_closure_solo(int dim, int k);
+// loads every kernel that launch_patch_colour<double> takes at this degree,
+// whatever the number of patches
+int prepare_closure_f64(int dim, int k);
 template <typename T>
 int launch_patch_colour(const PatchLaunch& pl, T* u, const T* b, const T* dinv, cudaStream_t s);
 // one colour of a coarse level with the one-output-per-thread kernel (FP64 problems,

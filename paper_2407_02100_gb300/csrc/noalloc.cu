@@ -22,8 +22,10 @@
 // names a host-side shadow) and the degree's coefficient tables are copied to
 // __constant__ memory with cudaMemcpyToSymbol, which allocates nothing but is
 // synchronous.  The generalised eigenproblem of the degree is solved on the
-// host once per process.  Later calls on that device and degree enqueue
-// kernels only.
+// host once per process.  The sweep kernels of the degree are loaded then too
+// (a launch takes one or another by the size of its colour, and a kernel that is
+// loaded at its first launch may allocate and wait for the device).  Later calls
+// on that device, dimension and degree enqueue kernels only, at any mesh size.
 #include <cuda_runtime.h>
 
 #include <cmath>
@@ -70,6 +72,7 @@ std::mutex g_mutex;
 DegreeData g_degree[gmg::kMaxDegree + 1];                  // host set-up math per degree
 double* g_fd_diag_addr[gmg::kMaxDevices] = {};             // array address per device
 bool g_tables_uploaded[gmg::kMaxDevices][gmg::kMaxDegree + 1] = {};
+bool g_kernels_loaded[gmg::kMaxDevices][2][gmg::kMaxDegree + 1] = {};
 
 // Host set-up of degree k (unit cells, level independent), solved once.
 int degree_data(int k, const DegreeData** out) {
@@ -88,9 +91,9 @@ int degree_data(int k, const DegreeData** out) {
   return GMG_OK;
 }
 
-// Per-device set-up for degree k on the current device: the array's address
-// and the degree's __constant__ tables.
-int device_setup(int k, double** diag, Lambda1d* lam) {
+// Per-device set-up for degree k on the current device: the array's address,
+// the degree's __constant__ tables and the sweep kernels of the dimension.
+int device_setup(int dim, int k, double** diag, Lambda1d* lam) {
   const int dev = gmg::current_device();
   if (dev < 0) return GMG_ERR_CUDA;
   std::lock_guard<std::mutex> lock(g_mutex);
@@ -110,6 +113,12 @@ int device_setup(int k, double** diag, Lambda1d* lam) {
                                           d->Kc.data(), nullptr);
     if (st != GMG_OK) return st;
     g_tables_uploaded[dev][k] = true;
+  }
+  bool& loaded = g_kernels_loaded[dev][dim - 2][k];
+  if (!loaded) {
+    st = gmg::prepare_closure_f64(dim, k);
+    if (st != GMG_OK) return st;
+    loaded = true;
   }
   *diag = g_fd_diag_addr[dev];
   *lam = d->lam;
@@ -132,7 +141,7 @@ extern "C" int gmg_smooth_noalloc(int dim, int degree, int n_cells, double dampi
 
   double* diag = nullptr;
   Lambda1d lam;
-  int st = device_setup(k, &diag, &lam);
+  int st = device_setup(dim, k, &diag, &lam);
   if (st != GMG_OK) return st;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
 

@@ -427,19 +427,29 @@ struct SmallCfg {
   static constexpr int LIMIT = DIM == 3 ? (K >= 5 ? 304 : 0) : K >= 2 ? 1600 : 0;
 };
 
+// Loads the kernel and sets its attribute, once per device.
 template <int DIM, int K, int PP, int NT, int CTAS>
-int closure_launch(PatchTable& tab, const T* dinv, cudaStream_t s) {
+int closure_prepare() {
   constexpr int SMEM = ClosureSmem<DIM, K>::bytes(PP);
   static_assert(SMEM <= 227 * 1024, "sweep kernel shared memory exceeds the per-CTA limit");
-  auto kern = pair_closure_kernel<DIM, K, NT, PP, CTAS>;
-  static PerDevice<bool> ready_dev;  // attribute set once per device
+  static PerDevice<bool> ready_dev;
   bool* const ready = ready_dev.get();
   if (!ready) return GMG_ERR_CUDA;
   if (!*ready) {
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM) != cudaSuccess)
+    auto kern = pair_closure_kernel<DIM, K, NT, PP, CTAS>;
+    cudaFuncAttributes attr;
+    if (cudaFuncGetAttributes(&attr, kern) != cudaSuccess ||
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM) != cudaSuccess)
       return GMG_ERR_CUDA;
     *ready = true;
   }
+  return GMG_OK;
+}
+
+template <int DIM, int K, int PP, int NT, int CTAS>
+int closure_launch(PatchTable& tab, const T* dinv, cudaStream_t s) {
+  const int st = closure_prepare<DIM, K, PP, NT, CTAS>();
+  if (st != GMG_OK) return st;
   int groups = 0;
   for (int i = 0; i < tab.n; ++i) {
     tab.e[i].group_begin = groups;
@@ -447,7 +457,7 @@ int closure_launch(PatchTable& tab, const T* dinv, cudaStream_t s) {
   }
   tab.total_groups = groups;
   if (groups <= 0) return GMG_OK;
-  kern<<<groups, NT, SMEM, s>>>(tab, dinv);
+  pair_closure_kernel<DIM, K, NT, PP, CTAS><<<groups, NT, ClosureSmem<DIM, K>::bytes(PP), s>>>(tab, dinv);
   count_launch();
   return cudaGetLastError() == cudaSuccess ? GMG_OK : GMG_ERR_CUDA;
 }

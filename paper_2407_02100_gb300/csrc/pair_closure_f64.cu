@@ -22,7 +22,20 @@ int table_launches(const PatchLaunch* pls, T* const* us, const T* const* bs, int
   return GMG_OK;
 }
 
+// both kernels of a degree: a launch takes one or the other by its patches
+template <int DIM, int K>
+int prepare_all() {
+  using Cfg = ClosureCfg<DIM, K>;
+  if constexpr (!SoloCfg<DIM, K>::ALWAYS) {
+    const int st = closure_prepare<DIM, K, Cfg::PP, Cfg::NT, Cfg::CTAS>();
+    if (st != GMG_OK) return st;
+  }
+  return prepare_closure_solo(DIM, K);
+}
+
 }  // namespace
+
+int prepare_closure_f64(int dim, int k) { GMG_DISPATCH(prepare_all, dim, k) }
 
 template <>
 int upload_closure_tables<double>(int k, const double* Mp, const double* Kp, const double* That) {

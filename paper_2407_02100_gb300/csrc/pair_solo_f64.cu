@@ -11,7 +11,15 @@ int solo_launch(PatchTable& tab, const T* dinv, cudaStream_t s) {
   return closure_launch<DIM, K, Cfg::PP, Cfg::NT, 0>(tab, dinv, s);
 }
 
+template <int DIM, int K>
+int solo_prepare() {
+  using Cfg = SoloCfg<DIM, K>;
+  return closure_prepare<DIM, K, Cfg::PP, Cfg::NT, 0>();
+}
+
 }  // namespace
+
+int prepare_closure_solo(int dim, int k) { GMG_DISPATCH(solo_prepare, dim, k) }
 
 int upload_closure_solo_tables(int k, const double* Mp, const double* Kp, const double* That) {
   return pl_upload(k, Mp, Kp, That);

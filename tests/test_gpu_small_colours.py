@@ -6,6 +6,10 @@ same bit for bit, whichever kernel takes it: the sizes are whole colours above
 the line, the same sweep by slabs of one vertex row stays below it, and a slab
 schedule gives each patch exactly the values that the whole colours give it.
 """
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 
@@ -15,6 +19,7 @@ from oracle.varcoef import VarPatchSmoother
 from paper_2407_02100_gb300 import inputs
 
 pytestmark = pytest.mark.gpu
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 
 @pytest.fixture(scope="module")
@@ -140,3 +145,35 @@ def test_few_patches_of_the_shared_face_form(gmg, k, n, launches):
     gmg.gmg_smooth(P.h, P.finest, u2, b, 1, False)
     assert float((u - u2).norm() / u2.norm()) <= 1e-12
     P.close()
+
+
+# gmg_smooth_noalloc after its first call at a degree: the kernel of another mesh size is loaded
+# already, so that the call neither allocates nor waits for the legacy stream, which a bounded
+# sleep of about 0.7 s keeps busy.  In a process of its own, where no other test has loaded the
+# kernels; the sizes lie on both sides of the lines of degree 6 (1000 patches) and 7 (152)
+NOALLOC = """
+import torch
+from paper_2407_02100_gb300 import gmg
+for k, first, later in ((6, 6, 22), (7, 13, 6)):
+    vecs = {}
+    for n in (first, later):
+        N = n * k + 1
+        vecs[n] = [torch.zeros(N * N * ((N + 3) // 4 * 4), dtype=torch.float64, device="cuda") for _ in range(2)]
+    side = torch.cuda.Stream()
+    gmg.gmg_smooth_noalloc(3, k, first, *vecs[first], stream=side.cuda_stream)
+    torch.cuda._sleep(1000)
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    torch.cuda._sleep(int(1.5e9))
+    gmg.gmg_smooth_noalloc(3, k, later, *vecs[later], stream=side.cuda_stream)
+    side.synchronize()
+    assert not torch.cuda.default_stream().query(), "the sweep waited for the legacy stream"
+    torch.cuda.synchronize()
+    assert torch.cuda.mem_get_info()[0] == free
+print("ok")
+"""
+
+
+def test_noalloc_at_another_mesh_size(gmg):
+    res = subprocess.run([sys.executable, "-c", NOALLOC], cwd=ROOT, capture_output=True, text=True, timeout=300)
+    assert res.returncode == 0 and res.stdout.endswith("ok\n"), res.stderr[-2000:]
