@@ -518,8 +518,8 @@ def run_ours(args):
                                     f"clock sampled during the sweeps ({sm_hz / 1e6:.0f} MHz); no issue-rate "
                                     "peak is measured by the driver",
                      "traffic": TRAFFIC_PER_LAUNCH,
-                     "traffic_source": "ncu dram__bytes_read.sum + dram__bytes_write.sum over every launch of 7 "
-                                       "sweeps, per colour step (face kernel + patch kernel); "
+                     "traffic_source": "ncu dram__bytes_read.sum + dram__bytes_write.sum over every launch of a "
+                                       "sweep, per colour step (face kernel + patch kernel); "
                                        "profiles/face_sweep_fp64_q4_64.md",
                      "algorithmic_bytes_per_launch": BYTES_PER_NODE * nodes / 8,
                      "executed_warp_inst_per_patch": WARP_INST_PER_PATCH,

@@ -713,8 +713,8 @@ int gmg::detail::create_problem(const gmg_desc* d, gmg_problem* p, const CreateO
   if (!device_wait_flag()) return GMG_ERR_CUDA;  // resolved once, outside any graph capture
   const int dim = d->dim, k = d->degree;
   // colour steps of up to 256 patches take the one-output-per-thread kernel
-  // at k <= 4, where it measured faster than the line kernels; above, a
-  // patch's outputs outnumber a CTA's threads and it measured slower
+  // at k <= 4, where it measured faster than the line kernels (with the
+  // shared-face form: small_limit, and kFewPatches of that form above k = 4)
   p->small_patches = k <= 4 ? 256 : 0;
   p->small_auto = true;
   // level hierarchy: n_levels given, or halve while even and >= 2
@@ -774,11 +774,11 @@ int gmg::detail::create_problem(const gmg_desc* d, gmg_problem* p, const CreateO
   CHECK(upload_table(p, &p->dinv, dinv));
   // face buffer of the shared-face sweep: the largest colour of the finest
   // level; without memory for it the closure form is used.  FP64 problems
-  // use the form from k = 3 (the sweep is bound by FP64 instructions, which
-  // it cuts by a third); FP32 ones from k = 7: at k = 3, 4 the FP32 closure
-  // kernel is faster (it is bound by issue and latency, and the face pass
-  // adds a launch and its traffic per colour), at k = 7 the form is 11 %
-  // faster.  The tensor-core precisions keep their kernel.
+  // use the form from k = 3, where it cuts the arithmetic by a third (Q4 64^3
+  // 2.14 ms a sweep against 3.13).  FP32 ones use it from k = 7, a line drawn
+  // against the closure kernel with one patch per thread (Q4 1.05 : 1.28 ms, Q7
+  // 3.06 : 2.72); the one with two is faster at k = 7 and 8 up to 24^3 at least
+  // (Q7 24^3 273 us against 454).  The tensor-core precisions keep their kernel.
   const bool faces_form = d->precision == GMG_FP64 ? k >= 3 : d->precision == GMG_FP32 && k >= 7;
   if (faces_form && dim == 3 && !opt.no_faces) {
     long long fe = 0;

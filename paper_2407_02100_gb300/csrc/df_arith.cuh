@@ -10,11 +10,13 @@ namespace gmg {
 // GB300 issues FP64 fused multiply-adds at about 1/74 of its FP32 rate, so
 // the arithmetic of FP64 problems' sweep and level operator runs in
 // double-float arithmetic on the FP32 pipe: a value is the unevaluated sum
-// hi + lo of two floats (about 48 significant bits).  A product's rounding error is recovered
-// exactly with one fmaf (TwoProd, after Dekker), a sum's with Knuth's
-// TwoSum, and each output of a line transform accumulates its leading
-// products exactly and its error terms in a second float (the Dot2 scheme
-// of Ogita, Rump and Oishi).  Every operation uses the _rn intrinsics, so
+// hi + lo of two floats (about 48 significant bits).  A single product's rounding
+// error is recovered exactly with one fmaf (TwoProd, after Dekker), a single
+// sum's with Knuth's TwoSum.  Each output of a line transform accumulates its
+// leading products in one float and the error terms in a second (the Dot2 scheme
+// of Ogita, Rump and Oishi); there the errors of the product and of the sum come
+// out of one operation, rounded together (df_acc_add), and the final sum takes
+// the ordered form (df_acc_value).  Every operation uses the _rn intrinsics, so
 // the compiler cannot contract or reassociate them.  Measured against FP64
 // on whole 3D FD solves (k = 3..8): relative error below 2e-14.
 struct dfv {
@@ -52,8 +54,8 @@ __device__ __forceinline__ dfv df_from_double(double x) {
 }
 __device__ __forceinline__ double df_to_double(dfv a) { return dfconv::from_df(a.hi, a.lo); }
 
-// Dot2 accumulator: the exact sum of the leading products is s + (the
-// rounding errors of the additions), collected with the products' errors in e
+// Dot2 accumulator: the sum of the leading products in s, the rounding errors of
+// the additions and of the products in e
 struct df_acc {
   float s, e;
 };

@@ -27,8 +27,10 @@
 // What bounds both kernels is the FP32 pipe: a Dot2 term is 10 operations.
 // Two patches per thread keep issue slots free for everything else: 3.6 + 1.6
 // thousand warp instructions per patch (9.7 with one patch per thread), FP32
-// pipe 51 % busy.  Per sweep at 64^3 (48^3): k = 3 1.12 -> 0.78 ms, k = 4
-// 3.03 -> 2.16, k = 7 (48^3) 15.9 -> 9.5.
+// pipe 51 % busy.  Per sweep at 64^3 (48^3): k = 3 1.12 -> 0.78 ms, k = 4 3.03 ->
+// 2.13, k = 7 (48^3) 15.9 -> 11.6 with another state each pass and 9.9 repeated on
+// one state: 732 bytes a thread spill there, and the local memory shares L2 with
+// the vectors.
 #include <algorithm>
 #include <type_traits>
 
