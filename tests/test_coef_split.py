@@ -58,10 +58,10 @@ def test_stiffness_rows_sum_to_zero_as_pairs(tmp_path):
 # the sums of the two-cell rows as the two-patch kernels read them: a cell's
 # row for either cell, the vertex row as twice its left half and the vertex
 # entry, the end columns from the table of negated end entries.  Exact, in
-# units of 2^-90.  No entry may move by more than the header of coef_split.h
-# says: half of the last place of the next larger one and one of its own, the
-# largest by (k + 2) / 2 of its own, and what the FP64 row itself is short of
-# zero.
+# units of 2^-90.  No entry may move from the mean of its places by more than
+# the header of coef_split.h says: half of the last place of the next larger one
+# and one of its own, the largest by (k + 2) / 2 of its own, and what the FP64 row
+# itself is short of zero.
 PATCH = r'''
 #include "coef_split.h"
 #include "setup.h"
@@ -95,15 +95,26 @@ int main() {
     for (int i = 0; i < k; ++i) {
       std::vector<double> row(k + 1);
       double defect = 0;
+      // the cell's entry (r, c) in the first cell's rows, or the mirrored one in the second's
+      auto at = [&](int r, int c) {
+        const double half = r == k && c == k ? 0.5 : 1.0;
+        return half * (Kp[(r - 1) * C + c] + Kp[(M - r) * C + 2 * k - c]) / 2;
+      };
       for (int c = 0; c <= k; ++c) {
-        row[c] = Kp[i * C + c] * (i == k - 1 && c == k ? 0.5 : 1.0);
+        const int r = i + 1, rs[4] = {r, c, k - r, k - c}, cs[4] = {c, r, k - c, k - r};
+        double sum = 0;
+        int n = 0;
+        for (int j = 0; j < 4; ++j)
+          if (rs[j] > 0) sum += at(rs[j], cs[j]), ++n;
+        row[c] = sum / n;
         defect += row[c];
+        if (!(std::fabs(row[c] - at(r, c)) <= 4e-15 * std::fabs(Kp[(k - 1) * C + k]))) { std::printf("mean %d %d %d\n", k, i, c); return 1; }
       }
       auto place = [&](double v) { return std::ldexp(1.0, std::ilogb(v) - 48); };
       for (int c = 0; c <= k; ++c) {
-        double next = 0;  // the next larger entry
+        double next = 0;  // the next larger entry (the mirror image on a middle row is as large)
         for (int d = 0; d <= k; ++d)
-          if (d != c && std::fabs(row[d]) >= std::fabs(row[c]) && (next == 0 || std::fabs(row[d]) < next)) next = std::fabs(row[d]);
+          if (std::fabs(row[d]) > std::fabs(row[c]) && (next == 0 || std::fabs(row[d]) < next)) next = std::fabs(row[d]);
         const double both = i == k - 1 && c == k ? 2.0 : 1.0;
         const double q = ((double)h[i * C + c] + (double)l[i * C + c]) / both;
         const double bound = next == 0 ? (k + 2) / 2.0 * place(row[c]) + std::fabs(defect) + 1e-15 * std::fabs(row[c])
