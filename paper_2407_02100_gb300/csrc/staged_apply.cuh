@@ -89,8 +89,9 @@ template <int K>
 struct PlanePass {
   // the widest tile whose columns with their halo, 4 cells high, take one round
   // of the threads (Q7 48^3 1449 -> 1179 us, Q3 51^3 102 -> 91, against 64 / K
-  // cells); at K = 4 16 cells, which split the usual meshes evenly, are better
-  // than 14 (Q4 64^3 368 : 410 us)
+  // cells); at K = 4 16 cells: a quarter faster than 14 where they save a tile (Q4
+  // 16^3 15.7 : 19.7 us, 32^3 52 : 66, 44^3 134 : 154, 64^3 365 : 406), up to 2.5 %
+  // slower elsewhere (28^3 equal, 42^3 124 : 121, 56^3 267 : 261)
   static constexpr int BX = K == 4 ? 16 : (63 - K) / K, BY = 4, NT = 256;
   static constexpr int EX = (BX + 1) * K + 1, EY = BY * K;
   static constexpr int EXP = EX | 1;  // odd row: lanes of the x stage lie K entries apart

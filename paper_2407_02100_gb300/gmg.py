@@ -373,7 +373,8 @@ def gmg_set_shared_faces(h, enable):
 
 def gmg_set_small_sweep(h, max_patches):
     """FP64 colour steps of at most max_patches patches use the coarse-level
-    kernel, one output per thread (0: never)."""
+    kernel, one output per thread (0: none).  The shared-face form's own colours
+    of up to 128 patches at degrees 5 to 7 use it whatever the limit."""
     _check("gmg_set_small_sweep", lib().gmg_set_small_sweep(h, int(max_patches)))
 
 
